@@ -238,13 +238,16 @@ static fm_status create_impl(const fm_config *cfg, Ctx *c)
     FM_TRY(launch_precompute(*c, 0));
     FM_CK(cudaStreamSynchronize(0));
     FM_TRY(freq_basis_setup(*c));
+    FM_TRY(fringe_setup(*c));
     FM_TRY(ha_setup(*c));
+    FM_TRY(hs_setup(*c));
     if (c->prec != FM_PREC_FP64_SIMT) {
         // monopole split: U = V(x = 1) once, in FP64, stored as FP32 (through the hour-angle
         // geometry when that form is on: one sum per fringe group; else the direct FP64 sum)
         c->dc_split = true;
         FM_TRY(dalloc(*c, &c->dc_u, (size_t)c->n_vis * 2));
         FM_TRY(dalloc_bytes(*c, &c->dc_mean, (size_t)c->F * sizeof(float)));
+        if (c->prec == FM_PREC_FP32_SIMT) FM_TRY(simt_supports<double>(*c, false));
         const fm_status hs = ha_monopole(*c, c->dc_u, 0);
         if (hs != FM_OK && hs != FM_ERR_UNSUPPORTED) return hs;
         if (hs == FM_ERR_UNSUPPORTED) {
@@ -289,6 +292,7 @@ static fm_status run_vis(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *d
             return dc ? launch_add_dc<R>(c, dc, dcs, vis, st) : FM_OK;
         }
     }
+    if (c.hs.on) return launch_vis_hs<R>(c, x, vis, st, dc, dcs);
     FM_TRY(profiled(c, 0, st, [&]() -> fm_status { return launch_vis<R>(c, x, vis, st); }));
     return dc ? launch_add_dc<R>(c, dc, dcs, vis, st) : FM_OK;
 }
@@ -300,6 +304,7 @@ static fm_status run_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st, b
         if (c.ha.on) return launch_adjoint_ha(c, omega, xbar, st, q_ready);
         if (c.prec >= FM_PREC_BF16X1) return launch_adjoint_tc(c, omega, xbar, st);
     }
+    if (c.hs.on) return launch_adjoint_hs<R>(c, omega, xbar, st);
     return profiled(c, 1, st, [&]() -> fm_status { return launch_adjoint<R>(c, omega, xbar, st); });
 }
 

@@ -157,8 +157,36 @@ struct HaState {
     float *qmax_ft = nullptr;  // [F][T] max |Re Q|, |Im Q| per (channel, LST)
     float *qscale = nullptr;   // [F]
     uint8_t *qimg = nullptr;   // [F][nkq][2][npad * 128] swizzled B tiles of the adjoint
-    std::vector<int> rep_ant;  // [U][2] antennas of each group's representative pair (host)
-    double lst0 = 0.0, dra = 0.0;
+};
+
+// Fringe groups and drift-scan geometry of a handle (k_hs.cu), shared by every form that
+// computes each distinct fringe once: baselines whose vectors are equal up to sign have equal or
+// conjugate fringes (Eq. rime_discrete), and a small antenna subset holds one member pair of
+// every group.
+struct FringeGroups {
+    int U = 0;                        // groups
+    int nant = 0;                     // antennas in the covering subset
+    std::vector<int> ant_of;          // [nant] subset entry -> antenna
+    std::vector<int> rep_i, rep_j;    // [U] representative pair (subset entries)
+    bool drift = false;               // the LST step is k / q RA pixels (q <= 4)
+    int k = 1, q = 1, nh = 0;         // hour-angle cells of 1 / q pixel: k per LST step, nh in all
+    int2 *uij = nullptr;              // [U] representative pair (subset entries), device
+    int *ant = nullptr;               // [nant] subset entry -> antenna, device
+    int *bmap = nullptr;              // [B] group * 2 + (1 if the baseline is the reversed vector)
+    int *moff = nullptr;              // [U + 1] CSR offsets of group members
+    int *mem = nullptr;               // [B] members, b * 2 + reversed
+};
+
+// Drift-scan form of the contraction on the CUDA cores (k_hs.cu), FP64 and FP32 handles.
+struct HsState {
+    bool on = false;
+    int row = 0;                      // table entries of one (channel, declination, antenna) row
+    int cls_t0[4] = {}, cls_off[4] = {}, cls_n[4] = {};   // per LST class: first LST, row offset, LSTs
+    void *E = nullptr;                // [F][D][nant][row] complex phasor table in the working type
+    // forward tiles
+    int G = 4, TU = 0, TL = 0, KS = 1, nut = 0, ntt = 0, nsplit = 0;
+    void *part = nullptr;             // [nsplit][F][T][U][2] partial sums
+    void *qsum = nullptr;             // [F][T][U][2] group sums of the residual weights
 };
 
 // Mode <-> pixel transforms on the tensor cores (k_modes.cu): FP16 hi/lo images of the
@@ -230,7 +258,9 @@ struct Ctx {
     std::vector<cudaEvent_t> prof_pool;
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> prof_rec;
     size_t prof_next = 0;
+    FringeGroups fg;
     HaState ha;
+    HsState hs;
     ModesTc mtc;
     // leapfrog scratch
     void *lf_q0 = nullptr, *lf_g = nullptr, *lf_z = nullptr;
@@ -416,6 +446,20 @@ fm_status vis_of_modes(Ctx &c, const R *a, R *xbuf, R *vis, cudaStream_t st, boo
 // shape does not fit its tiles
 fm_status launch_vis_tc(Ctx &c, const float *x, float *vis, cudaStream_t st);
 fm_status launch_adjoint_tc(Ctx &c, const float *omega, float *xbar, cudaStream_t st);
+// FM_OK when the array fits the CUDA-core contraction of the working type (forward or adjoint)
+template <typename R>
+fm_status simt_supports(const Ctx &c, bool adjoint);
+// fringe groups and drift-scan geometry (host work and small tables); the LST step as k / q RA
+// pixels, false when it is no such fraction
+fm_status fringe_setup(Ctx &c);
+bool drift_step(const Ctx &c, int &k, int &q);
+// drift-scan form on the CUDA cores (FP64 and FP32 handles); hs_setup leaves c.hs.on false when
+// the geometry or the sizes do not allow it
+fm_status hs_setup(Ctx &c);
+template <typename R>
+fm_status launch_vis_hs(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc, long long dcs);
+template <typename R>
+fm_status launch_adjoint_hs(Ctx &c, const R *omega, R *xbar, cudaStream_t st);
 // hour-angle form (drift scans with the LST step a whole number of RA pixels); ha_setup
 // leaves c.ha.on false when the geometry, precision or sizes do not allow it
 fm_status ha_setup(Ctx &c);

@@ -1377,21 +1377,8 @@ fm_status ha_setup(Ctx &c)
         if (atoi(e) == 0) return FM_OK;
     if (c.A < 2 || c.R > 512) return FM_OK;
     const double dra = (c.cfg.ra_max - c.cfg.ra_min) / c.R;
-    // LST step = k / q RA pixels (q <= 4): hour-angle cells of 1 / q pixel, k cells per LST
     int k = 1, q = 1;
-    if (c.T > 1) {
-        const double dl = c.lst[1] - c.lst[0];
-        for (int t = 1; t < c.T; ++t)
-            if (std::fabs(c.lst[t] - c.lst[0] - t * dl) > 1e-9 * dra) return FM_OK;
-        const double kr = dl / dra;
-        bool found = false;
-        for (q = 1; q <= 4 && !found; ++q) {
-            k = (int)std::llround(kr * q);
-            if (k >= 1 && k <= 32 && std::fabs(kr * q - k) <= 1e-9 * k) found = true;
-        }
-        --q;
-        if (!found) return FM_OK;
-    }
+    if (!drift_step(c, k, q)) return FM_OK;
     s.k = k;
     s.q = q;
     s.nh = (c.R - 1) * q + (c.T - 1) * k + 1;
@@ -1406,104 +1393,14 @@ fm_status ha_setup(Ctx &c)
     s.Lyc = 8 * s.Jc + 8 * k + 8;
     s.Ly = s.Lyc + ((c.T - 1) / HA_TCHUNK) * HA_TCHUNK * k;   // later passes start t0 k further in
 
-    // fringe groups: equal baseline vectors (to 1 nm) up to sign
-    bool group = true;
-    if (const char *e = getenv("FM_HA_GROUPS"))
-        if (atoi(e) == 0) group = false;
-    std::vector<int> rep_i, rep_j, bmap(c.B), bi(c.B), bj(c.B);
-    std::vector<double> rep_b;
-    std::vector<std::vector<int>> members;
-    for (int i = 0, b = 0; i < c.A; ++i)
-        for (int j = i + 1; j < c.A; ++j, ++b) {
-            bi[b] = i;
-            bj[b] = j;
-            const double v0 = c.ant[3 * i] - c.ant[3 * j], v1 = c.ant[3 * i + 1] - c.ant[3 * j + 1],
-                         v2 = c.ant[3 * i + 2] - c.ant[3 * j + 2];
-            int found = -1, cj = 0;
-            if (group)
-                for (size_t u = 0; u < rep_i.size() && found < 0; ++u) {
-                    const double *r = &rep_b[3 * u];
-                    const double dp = std::fmax(std::fabs(v0 - r[0]), std::fmax(std::fabs(v1 - r[1]), std::fabs(v2 - r[2])));
-                    const double dm = std::fmax(std::fabs(v0 + r[0]), std::fmax(std::fabs(v1 + r[1]), std::fabs(v2 + r[2])));
-                    if (dp < 1e-9) { found = (int)u; cj = 0; }
-                    else if (dm < 1e-9) { found = (int)u; cj = 1; }
-                }
-            if (found < 0) {
-                found = (int)rep_i.size();
-                rep_i.push_back(i);
-                rep_j.push_back(j);
-                rep_b.push_back(v0);
-                rep_b.push_back(v1);
-                rep_b.push_back(v2);
-                members.emplace_back();
-            }
-            bmap[b] = 2 * found + cj;
-            members[found].push_back(2 * b + cj);
-        }
-    s.U = (int)rep_i.size();
+    const FringeGroups &fg = c.fg;
+    s.U = fg.U;
     s.nmt = (s.U + 63) / 64;
     s.nkq = (s.U + 31) / 32;
-
-    // Antennas whose phasors the table holds: a small set S such that every group has a
-    // member pair inside S (greedy: add the antenna that completes the most groups, ties
-    // broken by partial coverage); each group's representative is then such a pair.
-    std::vector<int> in_s(c.A, 0), uncovered(s.U, 1);
-    int n_unc = s.U;
-    if (!group) {
-        for (int a = 0; a < c.A; ++a) in_s[a] = 1;
-        n_unc = 0;
-    }
-    while (n_unc > 0) {
-        int best = -1;
-        long long bfull = -1, bpart = -1;
-        for (int a = 0; a < c.A; ++a) {
-            if (in_s[a]) continue;
-            long long full = 0, part = 0;
-            for (int u = 0; u < s.U; ++u) {
-                if (!uncovered[u]) continue;
-                bool f1 = false, p1 = false;
-                for (int m : members[u]) {
-                    const int b = m >> 1, i = bi[b], j = bj[b];
-                    const bool hi = in_s[i] || i == a, hj = in_s[j] || j == a;
-                    if (hi && hj) { f1 = true; break; }
-                    if (hi || hj) p1 = true;
-                }
-                full += f1;
-                part += p1;
-            }
-            if (full > bfull || (full == bfull && part > bpart)) { best = a; bfull = full; bpart = part; }
-        }
-        in_s[best] = 1;
-        for (int u = 0; u < s.U; ++u) {
-            if (!uncovered[u]) continue;
-            for (int m : members[u]) {
-                const int b = m >> 1;
-                if (in_s[bi[b]] && in_s[bj[b]]) { uncovered[u] = 0; --n_unc; break; }
-            }
-        }
-    }
-    std::vector<int> pos(c.A, -1);
     // the table holds at most 63 antennas plus its zero entry
-    int n_in = 0;
-    for (int a = 0; a < c.A; ++a) n_in += in_s[a] ? 1 : 0;
-    if (n_in > 63) return FM_OK;
-    s.nant = 0;
-    for (int a = 0; a < c.A; ++a)
-        if (in_s[a]) { pos[a] = s.nant; s.ant_of[s.nant] = a; ++s.nant; }
-    // representatives inside S, member orientation relative to them
-    for (int u = 0; u < s.U; ++u) {
-        int rb = -1;
-        for (int m : members[u]) {
-            const int b = m >> 1;
-            if (in_s[bi[b]] && in_s[bj[b]]) { rb = m; break; }
-        }
-        const int rflip = rb & 1;   // representative reversed w.r.t. the group's first member
-        rep_i[u] = pos[bi[rb >> 1]];
-        rep_j[u] = pos[bj[rb >> 1]];
-        for (int &m : members[u]) m ^= rflip;
-    }
-    for (int u = 0; u < s.U; ++u)
-        for (int m : members[u]) bmap[m >> 1] = 2 * u + (m & 1);
+    if (fg.nant > 63) return FM_OK;
+    s.nant = fg.nant;
+    for (int a = 0; a < s.nant; ++a) s.ant_of[a] = fg.ant_of[a];
 
     // partition of the forward work units over the CTAs (the default grid: one CTA per SM;
     // the partial-sum buffer is sized for it, and a smaller grid needs no more contributors)
@@ -1523,7 +1420,7 @@ fm_status ha_setup(Ctx &c)
     const size_t vp_n = (size_t)s.nmt * c.F * s.J * 128 * s.npad;
     const size_t q_n = (size_t)c.F * c.T * s.U * 2;
     const size_t qi_n = (size_t)c.F * s.nkq * 2 * s.npad * 128;
-    const size_t need = 2 * e_n * 8 + ys_n * 2 + vp_n * 4 + q_n * 4 + qi_n + (size_t)c.B * 16 + (size_t)s.nmt * 64 * 8;
+    const size_t need = 2 * e_n * 8 + ys_n * 2 + vp_n * 4 + q_n * 4 + qi_n + (size_t)s.nmt * 64 * 8;
     size_t fr = 0, tot = 0;
     FM_CK(cudaMemGetInfo(&fr, &tot));
     if (need > fr / 2) return FM_OK;
@@ -1531,9 +1428,9 @@ fm_status ha_setup(Ctx &c)
     FM_TRY(ha_alloc(c, &s.E, e_n));
     FM_TRY(ha_alloc(c, &s.Ea, e_n));
     FM_TRY(ha_alloc(c, &s.uij, (size_t)s.nmt * 64));
-    FM_TRY(ha_alloc(c, &s.bmap, (size_t)c.B));
-    FM_TRY(ha_alloc(c, &s.moff, (size_t)s.U + 1));
-    FM_TRY(ha_alloc(c, &s.mem, (size_t)c.B));
+    s.bmap = fg.bmap;
+    s.moff = fg.moff;
+    s.mem = fg.mem;
     FM_TRY(ha_alloc(c, &s.ncontrib, ncontrib.size()));
     FM_TRY(ha_alloc(c, &s.ys, ys_n));
     FM_CK(cudaMemset(s.ys, 0, ys_n * sizeof(uint16_t)));     // strip elements outside the pixels stay zero
@@ -1546,23 +1443,8 @@ fm_status ha_setup(Ctx &c)
     FM_TRY(ha_alloc(c, &s.qimg, qi_n));
 
     std::vector<int2> huij((size_t)s.nmt * 64, make_int2(s.nant, s.nant));   // padding: the zero entry
-    for (int u = 0; u < s.U; ++u) huij[u] = make_int2(rep_i[u], rep_j[u]);
-    s.rep_ant.assign(2 * (size_t)s.U, 0);
-    for (int u = 0; u < s.U; ++u) {
-        s.rep_ant[2 * u] = s.ant_of[rep_i[u]];
-        s.rep_ant[2 * u + 1] = s.ant_of[rep_j[u]];
-    }
-    std::vector<int> hoff(s.U + 1, 0), hmem;
-    hmem.reserve(c.B);
-    for (int u = 0; u < s.U; ++u) {
-        hoff[u] = (int)hmem.size();
-        for (int m : members[u]) hmem.push_back(m);
-    }
-    hoff[s.U] = (int)hmem.size();
+    for (int u = 0; u < s.U; ++u) huij[u] = make_int2(fg.rep_i[u], fg.rep_j[u]);
     FM_CK(cudaMemcpy(s.uij, huij.data(), sizeof(int2) * huij.size(), cudaMemcpyHostToDevice));
-    FM_CK(cudaMemcpy(s.bmap, bmap.data(), sizeof(int) * bmap.size(), cudaMemcpyHostToDevice));
-    FM_CK(cudaMemcpy(s.moff, hoff.data(), sizeof(int) * hoff.size(), cudaMemcpyHostToDevice));
-    FM_CK(cudaMemcpy(s.mem, hmem.data(), sizeof(int) * hmem.size(), cudaMemcpyHostToDevice));
     FM_CK(cudaMemcpy(s.ncontrib, ncontrib.data(), sizeof(int) * ncontrib.size(), cudaMemcpyHostToDevice));
 
     // response scale 2^e, e even, with 2^e dOmega_max <= 2^14 (the beam is at most 1)
@@ -1581,8 +1463,6 @@ fm_status ha_setup(Ctx &c)
     a.lat = c.cfg.latitude_rad; a.amp_scale = std::ldexp(1.0, e2 / 2);
     a.kap64 = c.g.kap64; a.bcoef64 = c.g.bcoef64; a.domega64 = c.g.domega64;
     a.airy = c.g.beam32 != nullptr; a.dew = c.g.dish_ew; a.dns = c.g.dish_ns; a.freq = c.g.freq64;
-    s.lst0 = c.lst[0];
-    s.dra = dra;
     k_ha_table<<<2048, 256>>>(a, 1, reinterpret_cast<float *>(s.E));
     FM_CK_LAUNCH();
     k_ha_table<<<2048, 256>>>(a, 0, reinterpret_cast<float *>(s.Ea));
@@ -1597,30 +1477,35 @@ fm_status ha_setup(Ctx &c)
 // the direct FP64 sum)
 fm_status ha_monopole(Ctx &c, float *U, cudaStream_t st)
 {
-    const HaState &s = c.ha;
-    if (!s.on) return FM_ERR_UNSUPPORTED;
-    const size_t smem = sizeof(double) * 2 * ((size_t)s.nh + c.T);
+    const FringeGroups &fg = c.fg;
+    if (!fg.drift) return FM_ERR_UNSUPPORTED;
+    const size_t smem = sizeof(double) * 2 * ((size_t)fg.nh + c.T);
     if (smem > 200 * 1024) return FM_ERR_UNSUPPORTED;
+    std::vector<int> rep_ant(2 * (size_t)fg.U);
+    for (int u = 0; u < fg.U; ++u) {
+        rep_ant[2 * u] = fg.ant_of[fg.rep_i[u]];
+        rep_ant[2 * u + 1] = fg.ant_of[fg.rep_j[u]];
+    }
     int *rep = nullptr;
-    FM_CK(cudaMalloc(&rep, sizeof(int) * s.rep_ant.size()));
-    cudaError_t e = cudaMemcpy(rep, s.rep_ant.data(), sizeof(int) * s.rep_ant.size(), cudaMemcpyHostToDevice);
+    FM_CK(cudaMalloc(&rep, sizeof(int) * rep_ant.size()));
+    cudaError_t e = cudaMemcpy(rep, rep_ant.data(), sizeof(int) * rep_ant.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(rep);
         return cuda_fail(e, "cudaMemcpy (monopole groups)", __FILE__, __LINE__);
     }
     HaMonoArgs a;
-    a.F = c.F; a.D = c.D; a.R = c.R; a.T = c.T; a.B = c.B; a.U = s.U; a.k = s.k; a.q = s.q; a.nh = s.nh;
+    a.F = c.F; a.D = c.D; a.R = c.R; a.T = c.T; a.B = c.B; a.U = fg.U; a.k = fg.k; a.q = fg.q; a.nh = fg.nh;
     a.A_all = c.A;
-    a.lst0 = s.lst0; a.ra_min = c.cfg.ra_min; a.dra = s.dra;
+    a.lst0 = c.lst[0]; a.ra_min = c.cfg.ra_min; a.dra = (c.cfg.ra_max - c.cfg.ra_min) / c.R;
     a.dec_min = c.cfg.dec_min; a.ddec = (c.cfg.dec_max - c.cfg.dec_min) / c.D; a.lat = c.cfg.latitude_rad;
     a.kap64 = c.g.kap64; a.bcoef64 = c.g.bcoef64; a.domega64 = c.g.domega64;
     a.airy = c.g.beam32 != nullptr; a.dew = c.g.dish_ew; a.dns = c.g.dish_ns; a.freq = c.g.freq64;
-    a.rep = rep; a.moff = s.moff; a.mem = s.mem;
+    a.rep = rep; a.moff = fg.moff; a.mem = fg.mem;
     a.ug = nullptr;
     fm_status rc = FM_OK;
-    if (!c.ha.ug) {
+    if (c.ha.on && !c.ha.ug) {           // the group values are read by the hour-angle chi^2 epilogue
         void *q = nullptr;
-        if ((e = cudaMalloc(&q, sizeof(float) * 2 * (size_t)c.F * c.T * s.U)) != cudaSuccess) {
+        if ((e = cudaMalloc(&q, sizeof(float) * 2 * (size_t)c.F * c.T * fg.U)) != cudaSuccess) {
             cudaFree(rep);
             return cuda_fail(e, "cudaMalloc (group monopoles)", __FILE__, __LINE__);
         }
@@ -1630,7 +1515,7 @@ fm_status ha_monopole(Ctx &c, float *U, cudaStream_t st)
     a.ug = c.ha.ug;
     if ((e = smem_opt_in(k_ha_monopole)) != cudaSuccess) rc = cuda_fail(e, "smem_opt_in", __FILE__, __LINE__);
     if (rc == FM_OK) {
-        k_ha_monopole<<<(unsigned)((long long)c.F * s.U), 256, smem, st>>>(a, U);
+        k_ha_monopole<<<(unsigned)((long long)c.F * fg.U), 256, smem, st>>>(a, U);
         __atomic_fetch_add(&g_launches, 1LL, __ATOMIC_RELAXED);
         if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ha_monopole", __FILE__, __LINE__);
     }

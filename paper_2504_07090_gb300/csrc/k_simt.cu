@@ -369,25 +369,54 @@ __global__ void __launch_bounds__(256) k_vis_simt(DevGeom g, const R *__restrict
     }
 }
 
-template <typename R, int TPT>
-static fm_status vis_simt_launch(Ctx &c, const R *x, R *vis, cudaStream_t st)
+// antenna tiles (ntile of them, TPT a thread) and shared memory of the direct forward, and whether the
+// array fits; the drift-scan form takes the same arrays, so that what an FP64 or FP32 handle supports
+// does not depend on its LSTs
+struct VisSimtPlan {
+    int nbk, ntile, tpt, tpg, ngrp, pc;
+    size_t smem;
+};
+
+template <typename R>
+static fm_status vis_simt_plan(const Ctx &c, VisSimtPlan &p)
 {
-    int nbk = (c.A + 3) / 4, ntile = nbk * (nbk + 1) / 2;
-    int tpg = ((cdiv(ntile, TPT) + 31) / 32) * 32;
-    if (tpg > 256) { set_error("direct forward: %d antennas exceed the tile layout", c.A); return FM_ERR_UNSUPPORTED; }
-    int ngrp = 256 / tpg;
+    p.nbk = (c.A + 3) / 4;
+    p.ntile = p.nbk * (p.nbk + 1) / 2;
+    p.tpt = p.ntile <= 256 ? 1 : p.ntile <= 512 ? 2 : p.ntile <= 1024 ? 4 : 8;
+    p.tpg = (((int)cdiv(p.ntile, p.tpt) + 31) / 32) * 32;
+    if (p.tpg > 256) { set_error("direct forward: %d antennas exceed the tile layout", c.A); return FM_ERR_UNSUPPORTED; }
+    p.ngrp = 256 / p.tpg;
     // pixels staged per round: 64, halved while the phasor tiles exceed shared memory
-    int pc = 64;
-    size_t sm_e = 0, smem = 0;
-    const size_t sm_r = (size_t)ngrp * ntile * 32 * sizeof(R);
-    for (;; pc /= 2) {
-        sm_e = 2 * (size_t)pc * c.g.apad * 2 * sizeof(R) + pc * sizeof(R);
-        smem = sm_e > sm_r ? sm_e : sm_r;
-        if (smem <= 227 * 1024 || pc <= 8) break;
+    const size_t sm_r = (size_t)p.ngrp * p.ntile * 32 * sizeof(R);
+    for (p.pc = 64;; p.pc /= 2) {
+        const size_t sm_e = 2 * (size_t)p.pc * c.g.apad * 2 * sizeof(R) + p.pc * sizeof(R);
+        p.smem = sm_e > sm_r ? sm_e : sm_r;
+        if (p.smem <= 227 * 1024 || p.pc <= 8) break;
     }
-    if (smem > 227 * 1024) { set_error("direct forward: tiles exceed shared memory"); return FM_ERR_UNSUPPORTED; }
+    if (p.smem > 227 * 1024) { set_error("direct forward: tiles exceed shared memory"); return FM_ERR_UNSUPPORTED; }
+    return FM_OK;
+}
+
+template <typename R>
+static size_t adj_simt_smem(const Ctx &c) { return ((size_t)c.A * 128 + c.B) * 2 * sizeof(R); }
+
+template <typename R>
+fm_status simt_supports(const Ctx &c, bool adjoint)
+{
+    VisSimtPlan p;
+    if (!adjoint) return vis_simt_plan<R>(c, p);
+    if (adj_simt_smem<R>(c) <= 227 * 1024) return FM_OK;
+    set_error("direct adjoint: %d antennas exceed shared memory", c.A);
+    return FM_ERR_UNSUPPORTED;
+}
+template fm_status simt_supports<float>(const Ctx &, bool);
+template fm_status simt_supports<double>(const Ctx &, bool);
+
+template <typename R, int TPT>
+static fm_status vis_simt_launch(Ctx &c, const VisSimtPlan &p, const R *x, R *vis, cudaStream_t st)
+{
     FM_CK(smem_opt_in(k_vis_simt<R, TPT>));
-    k_vis_simt<R, TPT><<<c.F * c.T, 256, smem, st>>>(c.g, x, vis, nbk, ntile, tpg, ngrp, pc);
+    k_vis_simt<R, TPT><<<c.F * c.T, 256, p.smem, st>>>(c.g, x, vis, p.nbk, p.ntile, p.tpg, p.ngrp, p.pc);
     FM_CK_LAUNCH();
     return FM_OK;
 }
@@ -395,11 +424,14 @@ static fm_status vis_simt_launch(Ctx &c, const R *x, R *vis, cudaStream_t st)
 template <typename R>
 fm_status launch_vis(Ctx &c, const R *x, R *vis, cudaStream_t st)
 {
-    int nbk = (c.A + 3) / 4, ntile = nbk * (nbk + 1) / 2;
-    if (ntile <= 256) return vis_simt_launch<R, 1>(c, x, vis, st);
-    if (ntile <= 512) return vis_simt_launch<R, 2>(c, x, vis, st);
-    if (ntile <= 1024) return vis_simt_launch<R, 4>(c, x, vis, st);
-    return vis_simt_launch<R, 8>(c, x, vis, st);
+    VisSimtPlan p;
+    FM_TRY(vis_simt_plan<R>(c, p));
+    switch (p.tpt) {
+    case 1: return vis_simt_launch<R, 1>(c, p, x, vis, st);
+    case 2: return vis_simt_launch<R, 2>(c, p, x, vis, st);
+    case 4: return vis_simt_launch<R, 4>(c, p, x, vis, st);
+    default: return vis_simt_launch<R, 8>(c, p, x, vis, st);
+    }
 }
 
 // ---------------------------------------------------------------- chi^2 epilogue
@@ -888,8 +920,8 @@ __global__ void __launch_bounds__(128) k_adj_simt(DevGeom g, const R *__restrict
 template <typename R>
 fm_status launch_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st)
 {
-    size_t smem = ((size_t)c.A * 128 + c.B) * 2 * sizeof(R);
-    if (smem > 227 * 1024) return FM_ERR_UNSUPPORTED;
+    FM_TRY(simt_supports<R>(c, true));
+    const size_t smem = adj_simt_smem<R>(c);
     FM_CK(smem_opt_in(k_adj_simt<R>));
     dim3 grid(cdiv(c.npix, 128), c.F);
     k_adj_simt<R><<<grid, 128, smem, st>>>(c.g, omega, xbar);
