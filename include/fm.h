@@ -293,8 +293,8 @@ FM_API fm_status fm_sky_pixels_noalloc(int n_freq, int n_ra, int n_dec, int n_mo
 
 /* Which form of the fringe contraction (Eq. rime_discrete) the handle runs, written to
  * out[4] (host int32):
- *   out[0]  0 = sum on the CUDA cores (FP64 / FP32 precisions; for drift scans each distinct
- *               fringe is summed once and expanded to its baselines),
+ *   out[0]  0 = sum on the CUDA cores (FP64 / FP32 precisions; on drift scans, and for at most
+ *               256 distinct baseline vectors, each distinct fringe is summed once),
  *           1 = antenna form on the tensor cores (V = E W E^H per channel and LST),
  *           2 = hour-angle form on the tensor cores (drift scan with the LST step k / q RA
  *               pixels, q <= 4: one phasor table per channel over hour-angle cells of

@@ -241,6 +241,7 @@ static fm_status create_impl(const fm_config *cfg, Ctx *c)
     FM_TRY(fringe_setup(*c));
     FM_TRY(ha_setup(*c));
     FM_TRY(hs_setup(*c));
+    FM_TRY(gd_setup(*c));
     if (c->prec != FM_PREC_FP64_SIMT) {
         // monopole split: U = V(x = 1) once, in FP64, stored as FP32 (through the hour-angle
         // geometry when that form is on: one sum per fringe group; else the direct FP64 sum)
@@ -259,7 +260,8 @@ static fm_status create_impl(const fm_config *cfg, Ctx *c)
             fm_status s = FM_OK;
             if (cudaMemcpy(ones, h1.data(), sizeof(double) * h1.size(), cudaMemcpyHostToDevice) != cudaSuccess)
                 s = FM_ERR_CUDA;
-            if (s == FM_OK) s = launch_vis<double>(*c, ones, u64, 0);
+            if (s == FM_OK)
+                s = c->gd.on ? launch_vis_gd<double>(*c, ones, u64, 0, nullptr, 0) : launch_vis<double>(*c, ones, u64, 0);
             if (s == FM_OK) s = launch_d2f(2 * c->n_vis, u64, c->dc_u, 0);
             cudaError_t e2 = cudaStreamSynchronize(0);
             cudaFree(ones);
@@ -293,6 +295,7 @@ static fm_status run_vis(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *d
         }
     }
     if (c.hs.on) return launch_vis_hs<R>(c, x, vis, st, dc, dcs);
+    if (c.gd.on) return launch_vis_gd<R>(c, x, vis, st, dc, dcs);
     FM_TRY(profiled(c, 0, st, [&]() -> fm_status { return launch_vis<R>(c, x, vis, st); }));
     return dc ? launch_add_dc<R>(c, dc, dcs, vis, st) : FM_OK;
 }
@@ -305,6 +308,7 @@ static fm_status run_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st, b
         if (c.prec >= FM_PREC_BF16X1) return launch_adjoint_tc(c, omega, xbar, st);
     }
     if (c.hs.on) return launch_adjoint_hs<R>(c, omega, xbar, st);
+    if (c.gd.on) return launch_adjoint_gd<R>(c, omega, xbar, st);
     return profiled(c, 1, st, [&]() -> fm_status { return launch_adjoint<R>(c, omega, xbar, st); });
 }
 

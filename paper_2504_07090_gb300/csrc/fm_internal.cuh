@@ -189,6 +189,15 @@ struct HsState {
     void *qsum = nullptr;             // [F][T][U][2] group sums of the residual weights
 };
 
+// Distinct fringes summed on the CUDA cores on grids without a drift-scan form (k_gd.cu).
+struct GdState {
+    bool on = false;
+    int4 *ord = nullptr;              // [U] (i, j, u, 0) sorted by the representative pair (i, j)
+    int nsplit = 1;                   // pixel splits of the forward
+    void *part = nullptr;             // [nsplit][F][T][U][2] partial sums
+    void *qsum = nullptr;             // [F][T][U][2] group sums of the residual weights
+};
+
 // Mode <-> pixel transforms on the tensor cores (k_modes.cu): FP16 hi/lo images of the
 // basis tables, 128-byte-swizzled per 64-wide K atom.
 struct ModesTc {
@@ -261,6 +270,7 @@ struct Ctx {
     FringeGroups fg;
     HaState ha;
     HsState hs;
+    GdState gd;
     ModesTc mtc;
     // leapfrog scratch
     void *lf_q0 = nullptr, *lf_g = nullptr, *lf_z = nullptr;
@@ -460,6 +470,18 @@ template <typename R>
 fm_status launch_vis_hs(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc, long long dcs);
 template <typename R>
 fm_status launch_adjoint_hs(Ctx &c, const R *omega, R *xbar, cudaStream_t st);
+// distinct fringes on other grids (k_gd.cu)
+fm_status gd_setup(Ctx &c);
+template <typename R>
+fm_status launch_vis_gd(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc, long long dcs);
+template <typename R>
+fm_status launch_adjoint_gd(Ctx &c, const R *omega, R *xbar, cudaStream_t st);
+// V of every baseline from nsplit partial sums of the groups [nsplit][F][T][U][2] (plus the
+// monopole); the residual weights summed per group [F][T][U][2] (k_hs.cu)
+template <typename R>
+fm_status launch_group_finish(Ctx &c, int nsplit, const void *part, R *vis, cudaStream_t st, const R *dc, long long dcs);
+template <typename R>
+fm_status launch_group_qsum(Ctx &c, const R *omega, void *q, cudaStream_t st);
 // hour-angle form (drift scans with the LST step a whole number of RA pixels); ha_setup
 // leaves c.ha.on false when the geometry, precision or sizes do not allow it
 fm_status ha_setup(Ctx &c);

@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(256) k_hs_table(HsDev h, HsTabArgs a, typename
 // the responses P of the tile's groups are formed there from the phasor table, and thread
 // (rt, lt, ks) adds P x over the cells = ks mod KS for its G groups and LSTs lt + TL j.  A
 // declination's sum is formed before it joins the total (FP32: the rounding error grows with R + D / nsplit
-// terms, not with their product).  The splits' partial sums are added in order by k_hs_finish.
+// terms, not with their product).  The splits' partial sums are added in order by k_group_finish.
 template <typename R, int G>
 __global__ void __launch_bounds__(256) k_hs_fwd(HsDev h, const typename C2of<R>::t *__restrict__ E,
                                                 const R *__restrict__ x, typename C2of<R>::t *__restrict__ part)
@@ -411,23 +411,23 @@ __global__ void __launch_bounds__(256) k_hs_fwd(HsDev h, const typename C2of<R>:
 // V of every member of a group: the splits' partial sums in order, conjugated for reversed
 // members, plus the monopole dc[f dcs] Udc[f][t][b]
 template <typename R>
-__global__ void __launch_bounds__(256) k_hs_finish(HsDev h, int B, const typename C2of<R>::t *__restrict__ part,
+__global__ void __launch_bounds__(256) k_group_finish(int F, int T, int U, int nsplit, int B, const typename C2of<R>::t *__restrict__ part,
                                                    const int *__restrict__ moff, const int *__restrict__ mem,
                                                    const R *__restrict__ dc, long long dcs,
                                                    const float *__restrict__ Udc, R *__restrict__ vis)
 {
     using C2 = typename C2of<R>::t;
-    const long long n = (long long)h.F * h.T * h.U;
+    const long long n = (long long)F * T * U;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int u = (int)(e % h.U);
-        const long long ft = e / h.U;
+        const int u = (int)(e % U);
+        const long long ft = e / U;
         C2 s = part[e];
-        for (int k = 1; k < h.nsplit; ++k) {
+        for (int k = 1; k < nsplit; ++k) {
             const C2 w = part[(size_t)k * n + e];
             s.x += w.x;
             s.y += w.y;
         }
-        const R cf = dc ? dc[(ft / h.T) * dcs] : R(0);
+        const R cf = dc ? dc[(ft / T) * dcs] : R(0);
         for (int m = moff[u]; m < moff[u + 1]; ++m) {
             const int code = mem[m];
             const size_t o = 2 * ((size_t)ft * B + (code >> 1));
@@ -444,15 +444,15 @@ __global__ void __launch_bounds__(256) k_hs_finish(HsDev h, int B, const typenam
 // ------------------------------------------------------------ adjoint
 // Q[f][t][u]: the members' residual weights summed (conjugated for reversed members)
 template <typename R>
-__global__ void __launch_bounds__(256) k_hs_qsum(HsDev h, int B, const R *__restrict__ omega,
+__global__ void __launch_bounds__(256) k_group_qsum(int F, int T, int U, int B, const R *__restrict__ omega,
                                                  const int *__restrict__ moff, const int *__restrict__ mem,
                                                  typename C2of<R>::t *__restrict__ Q)
 {
     using C2 = typename C2of<R>::t;
-    const long long n = (long long)h.F * h.T * h.U;
+    const long long n = (long long)F * T * U;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int u = (int)(e % h.U);
-        const long long ft = e / h.U;
+        const int u = (int)(e % U);
+        const long long ft = e / U;
         C2 s = mk2(R(0), R(0));
         for (int m = moff[u]; m < moff[u + 1]; ++m) {
             const int code = mem[m];
@@ -655,6 +655,29 @@ fm_status hs_setup(Ctx &c)
     return c.prec == FM_PREC_FP64_SIMT ? hs_setup_t<double>(c) : hs_setup_t<float>(c);
 }
 
+static unsigned group_blocks(const Ctx &c)
+{
+    return (unsigned)std::min<long long>(cdiv((long long)c.F * c.T * c.fg.U, 256), 152 * 8);
+}
+
+template <typename R>
+fm_status launch_group_finish(Ctx &c, int nsplit, const void *part, R *vis, cudaStream_t st, const R *dc, long long dcs)
+{
+    k_group_finish<R><<<group_blocks(c), 256, 0, st>>>(c.F, c.T, c.fg.U, nsplit, c.B, (const typename C2of<R>::t *)part,
+                                                       c.fg.moff, c.fg.mem, dc, dcs, c.dc_u, vis);
+    FM_CK_LAUNCH();
+    return FM_OK;
+}
+
+template <typename R>
+fm_status launch_group_qsum(Ctx &c, const R *omega, void *q, cudaStream_t st)
+{
+    k_group_qsum<R><<<group_blocks(c), 256, 0, st>>>(c.F, c.T, c.fg.U, c.B, omega, c.fg.moff, c.fg.mem,
+                                                     (typename C2of<R>::t *)q);
+    FM_CK_LAUNCH();
+    return FM_OK;
+}
+
 template <typename R>
 fm_status launch_vis_hs(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc, long long dcs)
 {
@@ -665,11 +688,7 @@ fm_status launch_vis_hs(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc
                : c.hs.G == 2 ? hs_fwd_launch<R, 2>(c, h, x, st)
                              : hs_fwd_launch<R, 1>(c, h, x, st);
     }));
-    const unsigned nb = (unsigned)std::min<long long>(cdiv((long long)c.F * c.T * h.U, 256), 152 * 8);
-    k_hs_finish<R><<<nb, 256, 0, st>>>(h, c.B, (const typename C2of<R>::t *)c.hs.part, c.fg.moff, c.fg.mem, dc, dcs,
-                                       c.dc_u, vis);
-    FM_CK_LAUNCH();
-    return FM_OK;
+    return launch_group_finish<R>(c, h.nsplit, c.hs.part, vis, st, dc, dcs);
 }
 
 template <typename R>
@@ -678,9 +697,7 @@ fm_status launch_adjoint_hs(Ctx &c, const R *omega, R *xbar, cudaStream_t st)
     using C2 = typename C2of<R>::t;
     FM_TRY(simt_supports<R>(c, true));
     const HsDev h = hs_dev(c);
-    const unsigned nb = (unsigned)std::min<long long>(cdiv((long long)c.F * c.T * h.U, 256), 152 * 8);
-    k_hs_qsum<R><<<nb, 256, 0, st>>>(h, c.B, omega, c.fg.moff, c.fg.mem, (C2 *)c.hs.qsum);
-    FM_CK_LAUNCH();
+    FM_TRY(launch_group_qsum<R>(c, omega, c.hs.qsum, st));
     return profiled(c, 1, st, [&]() -> fm_status {
         FM_CK(smem_opt_in(k_hs_adj<R>));
         k_hs_adj<R><<<(unsigned)(c.F * c.D), 256, adj_smem<R>(c), st>>>(h, (const C2 *)c.hs.E, (const C2 *)c.hs.qsum,
@@ -691,6 +708,8 @@ fm_status launch_adjoint_hs(Ctx &c, const R *omega, R *xbar, cudaStream_t st)
 }
 
 #define HS_INST(R)                                                                                         \
+    template fm_status launch_group_finish<R>(Ctx &, int, const void *, R *, cudaStream_t, const R *, long long); \
+    template fm_status launch_group_qsum<R>(Ctx &, const R *, void *, cudaStream_t);                       \
     template fm_status launch_vis_hs<R>(Ctx &, const R *, R *, cudaStream_t, const R *, long long);        \
     template fm_status launch_adjoint_hs<R>(Ctx &, const R *, R *, cudaStream_t);
 HS_INST(float)
