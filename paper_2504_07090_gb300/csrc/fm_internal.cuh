@@ -495,7 +495,17 @@ fm_status modes_tc_setup(Ctx &c);
 fm_status launch_modes_tc_forward(Ctx &c, const float *a, float *x, cudaStream_t st, int skip_dc, unsigned *xmax,
                                   const StripArgs *strips = nullptr);
 fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaStream_t st);
-fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st);
+// windows of wider images as pixel maps: map f is the window of R columns from column off[f / per] of
+// image f % per, images [D][ld] (16-byte aligned, ld a multiple of 4 with 4 columns past the last window)
+// whose largest magnitudes are xmax[per] (float bits); per = 0: maps [nmaps][D][R]
+constexpr int kMapWindows = 16;
+struct MapWindows {
+    int per = 0, ld = 0;
+    int off[kMapWindows] = {};
+    const unsigned *xmax = nullptr;
+};
+fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st,
+                                       const MapWindows *w = nullptr);
 // dc != nullptr: also adds the monopole visibilities dc[f * dcs] U[f][t][b]; xmax_ready: the
 // channel maxima of x are already in c.ha.xmax (formed by the mode transform); strips_ready:
 // so are the sky strips of x (written by the mode transform); partials_only: V is not

@@ -143,6 +143,65 @@ __global__ void k_pc_fringe(DevGeom g, int f, int t, int U, const int *__restric
     }
 }
 
+// Drift scans: the response of a group at pixel (r, d) and LST t depends on the hour-angle cell only, so
+// one image per channel, X[plane][u][d][col], serves every LST as a window of R columns: LST s of class t0
+// (t = t0 + q s) starts at column off_t0 + (n_t0 - 1 - s) k.  The value of a cell is k_pc_fringe's at the
+// first (LST, pixel) that meets it; xmax[plane][u] receives each image's largest magnitude (float bits),
+// from which the transform takes its operand scale.
+struct PcCells {
+    int q, k, ld;
+    int n[4], off[4];                 // LSTs and first column of each class
+};
+
+__global__ void __launch_bounds__(256) k_pc_cells(DevGeom g, PcCells a, int f, int U, const int *__restrict__ rep,
+                                                  const float *__restrict__ W, float *__restrict__ X,
+                                                  unsigned *__restrict__ xmax)
+{
+    __shared__ float sm[2][8];
+    const int u = blockIdx.y;
+    const long long n = (long long)g.D * a.ld, plane = (long long)U * n;
+    const float wu = sqrt(W[(size_t)f * U + u] * (float)g.inv_sigma2);
+    float mr = 0.f, mi = 0.f;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+        const int col = (int)(e % a.ld), d = (int)(e / a.ld);
+        int t0 = 0;
+        while (t0 + 1 < a.q && a.n[t0 + 1] > 0 && col >= a.off[t0 + 1]) ++t0;
+        const int j = col - a.off[t0], b = min(j / a.k, a.n[t0] - 1), r = j - b * a.k;
+        float re = 0.f, im = 0.f;
+        if (r < g.R) {
+            const int t = t0 + a.q * (a.n[t0] - 1 - b), p = d * g.R + r;
+            const float z2 = g.za2_32[(size_t)t * g.npix + p];
+            if (z2 >= 0.f) {
+                const float bm = g.beam32 ? g.beam32[((size_t)f * g.T + t) * g.npix + p] : exp(g.bcoef32[f] * z2);
+                const float w = wu * g.domega32[d] * bm;
+                float kr, ki;
+                fringe(g, f, rep[2 * u], rep[2 * u + 1], t, p, kr, ki);
+                re = w * kr;
+                im = w * ki;
+            }
+        }
+        X[u * n + e] = re;
+        X[plane + u * n + e] = im;
+        mr = fmaxf(mr, fabsf(re));
+        mi = fmaxf(mi, fabsf(im));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+        mi = fmaxf(mi, __shfl_xor_sync(0xffffffffu, mi, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sm[0][threadIdx.x >> 5] = mr;
+        sm[1][threadIdx.x >> 5] = mi;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        float m = 0.f;
+        for (int k = 0; k < 8; ++k) m = fmaxf(m, sm[threadIdx.x][k]);
+        atomicMax(xmax + threadIdx.x * U + u, __float_as_uint(m));     // non-negative floats order like their bits
+    }
+}
+
 // Reuse of the strided GEMM from k_simt.cu through a local copy (one TU each keeps
 // the build parallel).
 struct GemmArgsH {
@@ -218,6 +277,100 @@ __global__ void k_pc_accum(long long n, const R *__restrict__ G, double *__restr
 {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         acc[e] += (double)G[e];
+}
+
+// acc64[j0][c][c'] += sum over rows of S[row][64 j0 + c] S[row][64 j0 + c'], one CTA per 64-block.  The
+// rows form chains of `chain` rows (a few LSTs' responses): a chain's sum is one FP32 multiply-add
+// sequence in row order, the chains join the FP64 total in order.  Thread (tile, chain) holds one of the 36
+// 8 x 8 tiles with c >= c' (the block is symmetric): 64 accumulators as 32 packed pairs against four
+// 16-byte shared-memory reads a row.  Rows arrive GR_ROWS a chain at a time by cp.async, two stages; a row
+// keeps 4 words of padding after its first half, which puts the eight 8-word tiles of a row into
+// different banks.  Bound: FP32 multiply-adds (and the shared-memory reads, at the same rate).
+constexpr int GR_ROWS = 8, GR_TILES = 36, GR_CHAINS = 4, GR_LD = 68;
+
+constexpr int gram_threads(int chains) { return (chains * GR_TILES + 31) / 32 * 32; }
+constexpr int gram_smem(int chains)
+{
+    const int stages = 2 * chains * GR_ROWS * GR_LD * (int)sizeof(float), tiles = chains * GR_TILES * 64 * (int)sizeof(float);
+    return stages > tiles ? stages : tiles;
+}
+
+__global__ void __launch_bounds__(gram_threads(GR_CHAINS)) k_pc_gram(int rows, int chain, int nk,
+                                                                     const float *__restrict__ S,
+                                                                     double *__restrict__ acc64)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *st = reinterpret_cast<float *>(smem_raw);              // [2][chains][GR_ROWS][GR_LD], then the tiles
+    const int nch = (rows + chain - 1) / chain, nthr = blockDim.x;
+    const int tid = threadIdx.x, ch = tid / GR_TILES, tile = tid % GR_TILES;
+    int ti = 0;
+    while ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
+    const int tj = tile - ti * (ti + 1) / 2;
+    const float *src = S + 64 * (size_t)blockIdx.x;
+    auto load = [&](int stage, int r0) {
+        for (int e = tid; e < nch * GR_ROWS * 16; e += nthr) {
+            const int cr = e >> 4, c = 4 * (e & 15), k = cr / GR_ROWS, r = r0 + cr % GR_ROWS;
+            const int row = k * chain + r;
+            const int full = r < chain && row < rows ? 16 : 0;    // past the chain's end: zeros
+            float *dst = st + (stage * nch * GR_ROWS + cr) * GR_LD + c + (c >= 32 ? 4 : 0);
+            const float *p = src + (size_t)(full ? row : 0) * nk + c;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(dst)), "l"(p), "r"(full));
+        }
+        asm volatile("cp.async.commit_group;");
+    };
+    float2 acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    const int ai = 8 * ti + (ti >= 4 ? 4 : 0), bi = 8 * tj + (tj >= 4 ? 4 : 0);
+    const int nst = (min(chain, rows) + GR_ROWS - 1) / GR_ROWS;
+    load(0, 0);
+    for (int s = 0; s < nst; ++s) {
+        if (s + 1 < nst) {
+            load((s + 1) & 1, (s + 1) * GR_ROWS);
+            asm volatile("cp.async.wait_group 1;");
+        } else {
+            asm volatile("cp.async.wait_group 0;");
+        }
+        __syncthreads();
+        if (ch < nch) {
+            const float *b0 = st + ((s & 1) * nch + ch) * GR_ROWS * GR_LD;
+#pragma unroll
+            for (int r = 0; r < GR_ROWS; ++r) {
+                const float4 *a = reinterpret_cast<const float4 *>(b0 + r * GR_LD + ai);
+                const float4 *b = reinterpret_cast<const float4 *>(b0 + r * GR_LD + bi);
+                const float4 a0 = a[0], a1 = a[1], c0 = b[0], c1 = b[1];
+                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                const float2 bv[4] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), make_float2(c1.x, c1.y),
+                                      make_float2(c1.z, c1.w)};
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(av[i], av[i]), bv[j], acc[i][j]);
+            }
+        }
+        __syncthreads();
+    }
+    if (ch < nch) {
+        float *o = st + (size_t)(ch * GR_TILES + tile) * 64;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) *reinterpret_cast<float2 *>(o + 8 * i + 2 * j) = acc[i][j];
+    }
+    __syncthreads();
+    double *out = acc64 + (size_t)blockIdx.x * 4096;
+    for (int e = tid; e < 4096; e += nthr) {
+        const int c = e >> 6, c2 = e & 63;
+        const int hi = c >= c2 ? c : c2, lo = c >= c2 ? c2 : c;   // entry of the stored triangle
+        const int th = hi >> 3, tl = lo >> 3;
+        const float *o = st + (size_t)(th * (th + 1) / 2 + tl) * 64 + 8 * (hi & 7) + (lo & 7);
+        double a = out[e];
+        for (int k = 0; k < nch; ++k) a += (double)o[(size_t)k * GR_TILES * 64];
+        out[e] = a;
+    }
 }
 
 // diagonal: acc[k] += sum_{plane, b} S[plane][b][k]^2
@@ -352,17 +505,107 @@ __global__ void __launch_bounds__(64) k_pc_chol_small(int n, const double *__res
     }
 }
 
-// Cholesky of the dense gain block in global FP64 scratch (one CTA), same inflation.
+// Cholesky of the dense gain block in FP64 by panels of CB columns, for the first attempt (no
+// inflation): k_pc_chol_init copies H, then per panel k_pc_chol_panel (a warp per row below the
+// diagonal block, every CTA factoring the CB x CB block itself) and k_pc_chol_trail (the trailing
+// lower triangle).  Every element takes its subtractions in ascending column order, as in k_pc_chol_big.  A
+// pivot that is not positive sets *bad, and the rest is left to k_pc_chol_big's retries.  FP64 runs at
+// 2 lanes per SM and clock, so the single CTA of k_pc_chol_big took 9.0 ms for 296 columns; spread over
+// the SMs it is bound by its 20 launches.
+constexpr int CB = 32;
+
+__global__ void k_pc_chol_init(int n, const double *__restrict__ H, double *__restrict__ W, int *bad)
+{
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n * n;
+         e += (long long)gridDim.x * blockDim.x)
+        W[e] = H[e];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *bad = 0;
+}
+
+__global__ void __launch_bounds__(256) k_pc_chol_panel(int n, int k0, double *__restrict__ W, double *__restrict__ Dg,
+                                                       int *bad)
+{
+    __shared__ double sD[CB][CB + 1];
+    __shared__ int sbad;
+    const int nb = min(CB, n - k0), tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) sbad = *bad;
+    for (int e = tid; e < nb * nb; e += 256) sD[e / nb][e % nb] = W[(size_t)(k0 + e / nb) * n + k0 + e % nb];
+    __syncthreads();
+    if (sbad) return;
+    if (tid < 32) {                    // one warp: lane = row of the diagonal block
+        for (int k = 0; k < nb; ++k) {
+            const double d = sD[k][k];
+            if (!(d > 0.0) || !isfinite(d)) {
+                if (lane == 0) sbad = 1;
+                break;
+            }
+            const double dk = sqrt(d);
+            __syncwarp();
+            if (lane == k) sD[k][k] = dk;
+            if (lane > k && lane < nb) sD[lane][k] /= dk;
+            __syncwarp();
+            if (lane > k && lane < nb)
+                for (int q = k + 1; q <= lane; ++q) sD[lane][q] -= sD[lane][k] * sD[q][k];
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    if (sbad) {
+        if (blockIdx.x == 0 && tid == 0) *bad = 1;
+        return;
+    }
+    if (blockIdx.x == 0) {             // CTA 0 leaves the diagonal block in Dg (k_pc_chol_trail puts it in
+        for (int e = tid; e < nb * nb; e += 256) Dg[e] = sD[e / nb][e % nb];   // place: the other CTAs
+        return;                                                                 // still read the old one)
+    }
+    // a warp per row: lane q holds entry q; column k is final once the columns before it are subtracted
+    for (int r = k0 + nb + (blockIdx.x - 1) * 8 + (tid >> 5); r < n; r += (gridDim.x - 1) * 8) {
+        double v = lane < nb ? W[(size_t)r * n + k0 + lane] : 0.0;
+        for (int k = 0; k < nb; ++k) {
+            if (lane == k) v /= sD[k][k];
+            const double lk = __shfl_sync(0xffffffffu, v, k);
+            if (lane > k && lane < nb) v -= lk * sD[lane][k];
+        }
+        if (lane < nb) W[(size_t)r * n + k0 + lane] = v;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_pc_chol_trail(int n, int k0, double *__restrict__ W,
+                                                       const double *__restrict__ Dg, const int *__restrict__ bad)
+{
+    __shared__ double sR[16][CB + 1], sC[16][CB + 1];
+    const int r0 = k0 + CB + 16 * blockIdx.y, c0 = k0 + CB + 16 * blockIdx.x;
+    if (c0 > r0 + 15 || *bad) return;  // the same for the whole CTA
+    const int tid = threadIdx.x, nb = min(CB, n - k0);
+    if (blockIdx.x == 0 && blockIdx.y == 0)
+        for (int e = tid; e < nb * nb; e += 256)
+            if (e % nb <= e / nb) W[(size_t)(k0 + e / nb) * n + k0 + e % nb] = Dg[e];
+    if (r0 >= n) return;
+    for (int e = tid; e < 16 * CB; e += 256) {
+        const int i = e / CB, k = e % CB;
+        sR[i][k] = r0 + i < n ? W[(size_t)(r0 + i) * n + k0 + k] : 0.0;
+        sC[i][k] = c0 + i < n ? W[(size_t)(c0 + i) * n + k0 + k] : 0.0;
+    }
+    __syncthreads();
+    const int r = r0 + tid / 16, q = c0 + tid % 16;
+    if (r >= n || q > r) return;
+    double v = W[(size_t)r * n + q];
+    for (int k = 0; k < CB; ++k) v -= sR[tid / 16][k] * sC[tid % 16][k];
+    W[(size_t)r * n + q] = v;
+}
+
+// Cholesky of the dense gain block in global FP64 scratch (one CTA), same inflation; with *retry == 0
+// (retry not NULL) W already holds the factor of the first attempt and is only stored.
 template <typename R>
 __global__ void __launch_bounds__(256) k_pc_chol_big(int n, const double *__restrict__ H, const R *__restrict__ lam,
                                                      long long lam_off, int have_prior, double *__restrict__ W,
                                                      R *__restrict__ L, double *__restrict__ L64,
-                                                     int *__restrict__ status)
+                                                     int *__restrict__ status, const int *__restrict__ retry)
 {
     __shared__ int bad;
     const int tid = threadIdx.x;
     double c = 1.0;
-    for (int attempt = 0; attempt < 200; ++attempt) {
+    for (int attempt = 0; attempt < 200 && (!retry || *retry); ++attempt) {
         for (int e = tid; e < n * n; e += blockDim.x) {
             int r = e / n, q = e % n;
             double v = H[e];
@@ -402,29 +645,36 @@ __global__ void __launch_bounds__(256) k_pc_chol_big(int n, const double *__rest
     }
 }
 
-// Inverse of the dense lower-triangular gain-block factor W (FP64, row-major): thread j
-// solves W x = e_j by forward substitution in FP64 (x kept in Xd[j][.]), then stores
+// Inverse of the dense lower-triangular gain-block factor W (FP64, row-major): warp j solves
+// W x = e_j by forward substitution in FP64 (x in shared memory, each row's product over the lanes; a
+// thread per column spent 6.4 ms on 296 columns in its serial products), keeps x in Xd[j][.] and stores
 // Ginv[r][j] = x_r.  Used by the leapfrog's dense solves, which then become triangular
 // matrix-vector products.  The gain block keeps FP64 throughout (factor, inverses, products):
 // the global gain phase is held by the prior alone, so the block's condition number
 // reaches 1e6 and a rounded inverse would misplace the data-constrained directions.
-__global__ void __launch_bounds__(128) k_pc_tri_inv(int n, const double *__restrict__ W, double *__restrict__ Xd,
-                                                    double *__restrict__ Ginv, double *__restrict__ GinvT)
+__global__ void __launch_bounds__(32) k_pc_tri_inv(int n, const double *__restrict__ W, double *__restrict__ Xd,
+                                                   double *__restrict__ Ginv, double *__restrict__ GinvT)
 {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        double *x = Xd + (size_t)j * n;
-        for (int r = 0; r < j; ++r) x[r] = 0.0;
-        x[j] = 1.0 / W[(size_t)j * n + j];
-        for (int r = j + 1; r < n; ++r) {
-            const double *row = W + (size_t)r * n;
-            double a = 0.0;
-            for (int cc = j; cc < r; ++cc) a += row[cc] * x[cc];
-            x[r] = -a / row[r];
-        }
-        for (int r = 0; r < n; ++r) {
-            Ginv[(size_t)r * n + j] = x[r];
-            GinvT[(size_t)j * n + r] = x[r];
-        }
+    extern __shared__ double sx[];                                // [n]
+    const int j = blockIdx.x, lane = threadIdx.x;
+    for (int r = lane; r < j; r += 32) sx[r] = 0.0;
+    if (lane == 0) sx[j] = 1.0 / W[(size_t)j * n + j];
+    __syncwarp();
+    for (int r = j + 1; r < n; ++r) {
+        const double *row = W + (size_t)r * n;
+        double a = 0.0;
+#pragma unroll 4
+        for (int c = j + lane; c < r; c += 32) a += row[c] * sx[c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) sx[r] = -a / row[r];
+        __syncwarp();
+    }
+    for (int r = lane; r < n; r += 32) {
+        const double v = sx[r];
+        Xd[(size_t)j * n + r] = v;
+        Ginv[(size_t)r * n + j] = v;
+        GinvT[(size_t)j * n + r] = v;
     }
 }
 
@@ -566,18 +816,56 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     // route only), S [TB][2][U][nk], G [nk/bs][bs][bs], group weights W [F][U].  The tensor-core
     // transform takes TB LSTs' response maps per launch.
     const bool tcx = std::is_same<R, float>::value && c.mtc.on;
-    const int TB = tcx ? (c.T < 4 ? c.T : 4) : 1;
-    size_t nX = 2 * (size_t)U * c.npix * TB, nQ = tcx ? 0 : 2 * (size_t)U * c.D * c.M, nS = 2 * (size_t)U * c.nk * TB;
+    // Drift scans: the channel's cell image serves every LST (PcCells), up to GR_CHAINS chains of four
+    // LSTs a launch so that the 2 U TB maps fill whole waves of two CTAs an SM (504 maps leave the second
+    // of two waves a third full, 1512 take five full ones) within 128 MB of results.
+    bool cells = tcx && c.fg.drift;
+    PcCells pc{};
+    const int chain_t = tcx ? (c.T < 4 ? c.T : 4) : 1;            // LSTs of one FP32 Gram sum
+    int TB = chain_t;
+    if (cells) {
+        pc.q = c.fg.q;
+        pc.k = c.fg.k;
+        for (int t0 = 0; t0 < pc.q; ++t0) {
+            pc.n[t0] = t0 < c.T ? (c.T - t0 + pc.q - 1) / pc.q : 0;
+            pc.off[t0] = pc.ld;
+            if (pc.n[t0]) pc.ld += (c.R + (pc.n[t0] - 1) * pc.k + 3) & ~3;
+        }
+        pc.ld += 4;                    // the transform reads whole 16-byte words around a window
+        // steps so long that the image would need more than the maps of four LSTs, and over 1 GB
+        const size_t img = (size_t)U * c.D * pc.ld;
+        cells = img <= (size_t)U * c.npix * 4 || img * 2 * sizeof(R) <= (size_t)1 << 30;
+    }
+    if (cells) {
+        const long long maps = 2LL * U * cdiv(c.M, 128), slots = 2 * 152;
+        double best = 0.0;
+        for (int k = 1; k <= GR_CHAINS && (k - 1) * chain_t < c.T; ++k) {
+            const int tb = std::min(k * chain_t, c.T);
+            if (k > 1 && 2.0 * U * tb * c.nk * sizeof(R) > 128e6) break;
+            const double fill = (double)(maps * tb) / (double)(cdiv(maps * tb, slots) * slots);
+            if (fill > best + 0.02) { best = fill; TB = tb; }
+        }
+    }
+    size_t nX = cells ? 2 * (size_t)U * c.D * pc.ld : 2 * (size_t)U * c.npix * TB, nQ = tcx ? 0 : 2 * (size_t)U * c.D * c.M, nS = 2 * (size_t)U * c.nk * TB;
     // (counts rounded up to even so that the FP64 scratch after them stays 8-byte aligned)
     size_t nG = ((size_t)c.nk * bs + 1) & ~(size_t)1, nW = ((size_t)c.F * U + 1) & ~(size_t)1;
     R *X = nullptr;
-    size_t scratch = (nX + nQ + nS + nG + nW) * sizeof(R) + sizeof(double) * ((size_t)c.F * c.B + (size_t)ng * ng);
+    nX = (nX + 3) & ~(size_t)3;                 // S after X and Q: 16-byte rows
+    nQ = (nQ + 3) & ~(size_t)3;
+    nS = (nS + 1) & ~(size_t)1;
+    const size_t nM = cells ? 2 * (size_t)U : 0;        // image maxima
+    size_t scratch = (nX + nQ + nS + nG + nW + nM) * sizeof(R) +
+                     sizeof(double) * ((size_t)c.F * c.B + (size_t)ng * ng + CB * CB + 1);
     if (cudaMalloc(&X, scratch) != cudaSuccess) { set_error("cudaMalloc precond scratch (%zu bytes)", scratch); return FM_ERR_ALLOC; }
     R *Q = X + nX, *S = Q + nQ, *G = S + nS, *Wg = G + nG;
-    double *s2 = reinterpret_cast<double *>(Wg + nW);
+    unsigned *xmax = reinterpret_cast<unsigned *>(Wg + nW);
+    double *s2 = reinterpret_cast<double *>(Wg + nW + nM);
     double *W = s2 + (size_t)c.F * c.B;
+    double *chol_dg = W + (size_t)ng * ng;
+    int *chol_bad = reinterpret_cast<int *>(chol_dg + CB * CB);
     fm_status rc = FM_OK;
     do {
+        if (smem_opt_in(k_pc_gram) != cudaSuccess || smem_opt_in(k_pc_tri_inv) != cudaSuccess) { rc = FM_ERR_CUDA; break; }
         R *gn = (R *)c.gains;
         R *x = (R *)c.x, *vis = (R *)c.vis;
         if ((rc = launch_gains<R>(c, theta + c.n_sky, gn, st)) != FM_OK) break;
@@ -603,12 +891,32 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                 rc = FM_ERR_CUDA;
                 break;
             }
+            if constexpr (std::is_same<R, float>::value)
+                if (cells) {
+                    if (cudaMemsetAsync(xmax, 0, sizeof(unsigned) * 2 * U, st) != cudaSuccess) { rc = FM_ERR_CUDA; break; }
+                    k_pc_cells<<<dim3(std::max(1u, std::min(cdiv((long long)c.D * pc.ld, 256), 4864u / U)), U), 256, 0, st>>>(
+                        c.g, pc, f, U, g_rep, Wg, X, xmax);
+                }
             for (int t = 0; t < c.T; t += TB) {
                 const int tbn = c.T - t < TB ? c.T - t : TB;
-                for (int tb = 0; tb < tbn; ++tb)
-                    k_pc_fringe<R><<<2048, 256, 0, st>>>(c.g, f, t + tb, U, g_rep, Wg, X + (size_t)tb * 2 * U * c.npix);
+                if (!cells)
+                    for (int tb = 0; tb < tbn; ++tb)
+                        k_pc_fringe<R><<<2048, 256, 0, st>>>(c.g, f, t + tb, U, g_rep, Wg, X + (size_t)tb * 2 * U * c.npix);
                 if (cudaGetLastError() != cudaSuccess) { rc = FM_ERR_CUDA; break; }
-                if (tcx) {
+                if (cells) {
+                    // the same transform over the windows of tbn LSTs in the channel's cell image
+                    MapWindows w;
+                    w.per = 2 * U;
+                    w.ld = pc.ld;
+                    w.xmax = xmax;
+                    for (int tb = 0; tb < tbn; ++tb) {
+                        const int t0 = (t + tb) % pc.q, s = (t + tb) / pc.q;
+                        const int col = pc.off[t0] + (pc.n[t0] - 1 - s) * pc.k;
+                        w.off[tb] = col;
+                    }
+                    if ((rc = launch_modes_tc_adjoint_maps(c, (const float *)X, 2 * U * tbn, (float *)S, st, &w)) != FM_OK)
+                        break;
+                } else if (tcx) {
                     // S[tb,pl,b][m][n] = sum_{d,r} Phi[r][m] X[tb,pl,b][d][r] P[d][n]: the tensor-core
                     // pixel -> mode transform over the 2U response maps of tbn LSTs
                     if ((rc = launch_modes_tc_adjoint_maps(c, (const float *)X, 2 * U * tbn, (float *)S, st)) != FM_OK)
@@ -623,7 +931,11 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                     GemmArgsH q2{c.M, c.N, c.D, (long long)c.D * c.M, 1, c.M, 0, c.N, 1, c.nk, c.N, 1};
                     if ((rc = gemm_h<R>(q2, 2LL * U, Q, leg, S, st)) != FM_OK) break;
                 }
-                if (bs > 1) {
+                if (bs > 1 && std::is_same<R, float>::value) {
+                    const int nch = (int)cdiv(tbn, chain_t);
+                    k_pc_gram<<<(unsigned)(c.nk / 64), gram_threads(nch), gram_smem(nch), st>>>(
+                        2 * U * tbn, 2 * U * chain_t, c.nk, (const float *)S, accf);
+                } else if (bs > 1) {
                     // G[j0][c][c'] = sum_{tb,pl,b} S[tb,pl,b][j0*bs+c] S[tb,pl,b][j0*bs+c']
                     GemmArgsH q3{bs, bs, 2 * U * tbn, bs, 1, c.nk, bs, c.nk, 1, (long long)bs * bs, bs, 1};
                     if ((rc = gemm_h<R>(q3, c.nk / bs, S, S, G, st)) != FM_OK) break;
@@ -668,8 +980,15 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
             }
             // FP64 gain block: [0] L_g, [1] L_g^-1, [2] L_g^-T, [3] L_g^-T L_g^-1
             double *G64 = (double *)c.pc_ginv;
+            k_pc_chol_init<<<cdiv((long long)ng * ng, 256), 256, 0, st>>>(ng, c.pc_blocks + sky_sz, W, chol_bad);
+            for (int k0 = 0; k0 < ng; k0 += CB) {
+                const int left = std::max(ng - k0 - CB, 0);
+                const unsigned nt = std::max(cdiv(left, 16), 1u);
+                k_pc_chol_panel<<<1 + std::min(cdiv(left, 8), 152u), 256, 0, st>>>(ng, k0, W, chol_dg, chol_bad);
+                k_pc_chol_trail<<<dim3(nt, nt), 256, 0, st>>>(ng, k0, W, chol_dg, chol_bad);
+            }
             k_pc_chol_big<R><<<1, 256, 0, st>>>(ng, c.pc_blocks + sky_sz, (const R *)c.lam, c.n_sky,
-                                                c.have_prior ? 1 : 0, W, Lf + sky_sz, G64, c.status);
+                                                c.have_prior ? 1 : 0, W, Lf + sky_sz, G64, c.status, chol_bad);
             if (!c.pc_linv) {
                 if (cudaMalloc(&c.pc_linv, sizeof(R) * (size_t)nsky_blk * tri_block_elems<R>()) != cudaSuccess) {
                     rc = FM_ERR_ALLOC;
@@ -681,7 +1000,7 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
             smem_opt_in(k_pc_blk_inv<R>);
             k_pc_blk_inv<R><<<(unsigned)nsky_blk, 64, 2 * 64 * 65 * sizeof(double), st>>>(Lf, (R *)c.pc_linv);
             if (ng > 0) {
-                k_pc_tri_inv<<<cdiv(ng, 128), 128, 0, st>>>(ng, W, c.pc_tmp, G64 + (size_t)ng * ng,
+                k_pc_tri_inv<<<ng, 32, sizeof(double) * ng, st>>>(ng, W, c.pc_tmp, G64 + (size_t)ng * ng,
                                                             G64 + 2 * (size_t)ng * ng);
                 k_pc_gm<<<cdiv((long long)ng * ng, 256), 256, 0, st>>>(ng, c.pc_tmp, G64 + 3 * (size_t)ng * ng);
             }

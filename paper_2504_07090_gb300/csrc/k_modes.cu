@@ -157,7 +157,7 @@ __device__ __forceinline__ float md_absmax(const float *a, int rows, int cols, b
 {
     float m = 0.f;
     const long long n = (long long)rows * cols;
-    if ((cols & 3) == 0) {
+    if ((cols & 3) == 0 && (reinterpret_cast<uintptr_t>(a) & 15) == 0) {
         const float4 *a4 = reinterpret_cast<const float4 *>(a);
         const long long n4 = n / 4;
         for (long long e0 = threadIdx.x; e0 < n4; e0 += 8LL * blockDim.x) {
@@ -181,14 +181,15 @@ __device__ __forceinline__ float md_absmax(const float *a, int rows, int cols, b
     return block_max(m, red);
 }
 
-// B operand atom from a row-major FP32 matrix src [rows][cols] (rows_pad rows, K values
-// 64 ka .. 64 ka + 63), scaled and split into FP16 hi / lo rows; entry (0, 0) is read as
-// zero when zero00.  16-byte loads (eight in flight) when cols is a multiple of 4.
-__device__ __forceinline__ void md_convert_atom(const float *src, int rows, int cols, int rows_pad, int ka,
-                                                float sc, bool zero00, uint8_t *b)
+// B operand atom from a row-major FP32 matrix src [rows][cols] (rows ld apart, src `mis` columns
+// past a 16-byte boundary; rows_pad rows, K values 64 ka .. 64 ka + 63), scaled and split into FP16
+// hi / lo rows; entry (0, 0) is read as zero when zero00.  16-byte loads (eight in flight) when cols
+// and ld are multiples of 4 and src - mis is on that boundary.
+__device__ __forceinline__ void md_convert_atom(const float *src, int rows, int cols, int ld, int mis, int rows_pad,
+                                                int ka, float sc, bool zero00, uint8_t *b)
 {
     const int n4 = rows_pad * 16;                  // 4-value pieces in the atom
-    const bool vec = (cols & 3) == 0;
+    const bool vec = ((cols | ld) & 3) == 0 && (reinterpret_cast<uintptr_t>(src - mis) & 15) == 0;
     for (int e0 = threadIdx.x; e0 < n4; e0 += 8 * blockDim.x) {
         float4 v[8];
 #pragma unroll
@@ -197,9 +198,18 @@ __device__ __forceinline__ void md_convert_atom(const float *src, int rows, int 
             const int row = e >> 4, k = 64 * ka + 4 * (e & 15);
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
             if (e < n4 && row < rows) {
-                const float *p = src + (size_t)row * cols + k;
-                if (vec && k + 3 < cols) x = __ldg(reinterpret_cast<const float4 *>(p));
-                else {
+                const float *p = src + (size_t)row * ld + k;
+                if (vec && k + 3 < cols) {
+                    // the 16-byte words around an offset window; `mis` is the CTA's own
+                    const float4 *q = reinterpret_cast<const float4 *>(p - mis);
+                    x = __ldg(q);
+                    if (mis) {
+                        const float4 y = __ldg(q + 1);
+                        x = mis == 1   ? make_float4(x.y, x.z, x.w, y.x)
+                            : mis == 2 ? make_float4(x.z, x.w, y.x, y.y)
+                                       : make_float4(x.w, y.x, y.y, y.z);
+                    }
+                } else {
                     if (k < cols) x.x = __ldg(p);
                     if (k + 1 < cols) x.y = __ldg(p + 1);
                     if (k + 2 < cols) x.z = __ldg(p + 2);
@@ -387,7 +397,9 @@ struct MdPlan {
     const uint8_t *img1;    // stage-1 A image atoms (2 x 128 rows x 128 bytes each)
     const uint8_t *img2;    // stage-2 B image atoms (2 x nb2 rows x 128 bytes each)
     const float *src;       // stage-1 B operand, row-major [src_rows][src_cols]
-    int src_rows, src_cols;
+    int src_rows, src_cols, src_ld;
+    int src_mis;            // columns from a 16-byte boundary to src, the same in every row (windows)
+    const unsigned *src_max;   // largest magnitude known beforehand (float bits), or NULL
     int n1;                 // stage-1 K atoms
     int nb1;                // stage-1 N (rows of its B atoms, padded) = stage-2 K
     int nb2;                // stage-2 N
@@ -446,7 +458,7 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             img_issue(i);
             (i == 0 ? last_img0 : last_img1) = i;
         }
-    sa = pow2_below(md_absmax(p.src, p.src_rows, p.src_cols, p.skip_dc, m.red));
+    sa = pow2_below(p.src_max ? __uint_as_float(*p.src_max) : md_absmax(p.src, p.src_rows, p.src_cols, p.skip_dc, m.red));
     g = 1.f;
     const uint32_t idesc1 = idesc_f16(128, p.nb1, 0), idesc2 = idesc_f16(128, p.nb2, 0);
     bool ok = true;
@@ -467,7 +479,7 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             break;
         }
         if (i < p.n1) {
-            md_convert_atom(p.src, p.src_rows, p.src_cols, p.nb1, i, sa, p.skip_dc, m.b(s));
+            md_convert_atom(p.src, p.src_rows, p.src_cols, p.src_ld, p.src_mis, p.nb1, i, sa, p.skip_dc, m.b(s));
         } else {
             if (i == p.n1) {
                 tc_fence_after();
@@ -531,7 +543,9 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
     p.img2 = phi_img;
     p.src = a_all + (size_t)f * z.M * z.N;
     p.src_rows = z.M;
-    p.src_cols = z.N;
+    p.src_cols = p.src_ld = z.N;
+    p.src_mis = 0;
+    p.src_max = nullptr;
     p.n1 = z.Np / 64;
     p.nb1 = z.Mp;
     p.nb2 = z.Rp;
@@ -572,7 +586,8 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
 // image); abar = D2 / scales.
 __global__ void __launch_bounds__(MD_THREADS, 1)
 k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *__restrict__ phit_img,
-            const uint8_t *__restrict__ legt_img, float *__restrict__ abar_all, int *__restrict__ status, int ncols)
+            const uint8_t *__restrict__ legt_img, float *__restrict__ abar_all, int *__restrict__ status, int ncols,
+            MapWindows w)
 {
     const int f = blockIdx.x, mtile = blockIdx.y;
     const MdSmem m = md_smem(z.Dp > z.Np ? z.Dp : z.Np, ns);
@@ -582,7 +597,16 @@ k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *_
     p.img2 = legt_img;
     p.src = xb_all + (size_t)f * z.D * z.R;
     p.src_rows = z.D;
-    p.src_cols = z.R;
+    p.src_cols = p.src_ld = z.R;
+    p.src_mis = 0;
+    p.src_max = nullptr;
+    if (w.per > 0) {                            // map f: window f / per of image f % per
+        const int wi = f / w.per, im = f - wi * w.per;
+        p.src = xb_all + w.off[wi] + (size_t)im * z.D * w.ld;
+        p.src_ld = w.ld;
+        p.src_mis = w.off[wi] & 3;
+        p.src_max = w.xmax + im;
+    }
     p.n1 = z.Rp / 64;
     p.nb1 = z.Dp;
     p.nb2 = z.Np;
@@ -695,14 +719,16 @@ fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaSt
     return launch_modes_tc_adjoint_maps(c, xbar, c.F, abar, st);
 }
 
-// the same transform for nmaps pixel maps xbar[nmaps][D][R] -> abar[nmaps][M][N]
-fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st)
+// the same transform for nmaps pixel maps xbar[nmaps][D][R] -> abar[nmaps][M][N], or the windows w of
+// wider images
+fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st,
+                                       const MapWindows *w)
 {
     MdDims z = md_dims(c);
     z.F = nmaps;
     const int nmt = (c.M + 127) / 128, ns = md_slots(nmaps * nmt);
     k_modes_adj<<<dim3(nmaps, nmt), MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
-        z, ns, xbar, c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np));
+        z, ns, xbar, c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np), w ? *w : MapWindows{});
     FM_CK_LAUNCH();
     return FM_OK;
 }
