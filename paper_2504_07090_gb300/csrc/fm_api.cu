@@ -284,11 +284,16 @@ static fm_status create_impl(const fm_config *cfg, Ctx *c)
 // (inside the last kernel of the hour-angle form, as a separate pass otherwise)
 template <typename R>
 static fm_status run_vis(Ctx &c, const R *x, R *vis, cudaStream_t st, const R *dc = nullptr, long long dcs = 0,
-                         bool xmax_ready = false, bool strips_ready = false, bool partials_only = false)
+                         bool partials_only = false)
 {
     // the tensor-core launchers time their main kernel themselves
     if constexpr (std::is_same<R, float>::value) {
-        if (c.ha.on) return launch_vis_ha(c, x, vis, st, dc, dcs, xmax_ready, strips_ready, partials_only);
+        if (c.ha.on) {
+            HaSky k{x, vis, st};
+            k.dc = dc;
+            k.dcs = dcs;
+            return launch_vis_ha(c, k, partials_only);
+        }
         if (c.prec >= FM_PREC_BF16X1) {
             FM_TRY(launch_vis_tc(c, x, vis, st));
             return dc ? launch_add_dc<R>(c, dc, dcs, vis, st) : FM_OK;
@@ -312,28 +317,60 @@ static fm_status run_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st, b
     return profiled(c, 1, st, [&]() -> fm_status { return launch_adjoint<R>(c, omega, xbar, st); });
 }
 
+// mode transform of one sky for the hour-angle forward.  After the tensor-core transform the
+// channel maxima of x that scale the sky strip are formed, and with one CTA per channel the strips
+// themselves
+static fm_status sky_of_modes(Ctx &c, const float *a, float *x, float *vis, int slot, cudaStream_t st, HaSky &k)
+{
+    const bool dc = c.dc_split;
+    k = HaSky{x, vis, st};
+    k.dc = dc ? a : nullptr;
+    k.dcs = dc ? c.nk : 0;
+    k.slot = slot;
+    unsigned *xmax = c.mtc.on ? c.ha.xmax + (size_t)slot * c.F : nullptr;
+    StripArgs sa;
+    if (xmax) {
+        k.xmax_ready = true;
+        k.strips_ready = ha_strip_args(c, sa, slot);
+        if (!k.strips_ready) FM_CK(cudaMemsetAsync(xmax, 0, sizeof(unsigned) * c.F, st));
+    }
+    return launch_modes_forward<float>(c, a, x, st, dc ? 1 : 0, xmax, k.strips_ready ? &sa : nullptr);
+}
+
 template <typename R>
 fm_status vis_of_modes(Ctx &c, const R *a, R *xbuf, R *vis, cudaStream_t st, bool partials_only)
 {
-    if (partials_only && !(std::is_same<R, float>::value && c.ha.on)) {
+    if constexpr (std::is_same<R, float>::value)
+        if (c.ha.on) {
+            HaSky k;
+            FM_TRY(sky_of_modes(c, a, xbuf, vis, 0, st, k));
+            return launch_vis_ha(c, k, partials_only);
+        }
+    if (partials_only) {
         set_error("unfinished visibilities exist only in the hour-angle form");
         return FM_ERR_STATE;
     }
-    // hour-angle form after the tensor-core transform: the transform forms the channel maxima
-    // of x that scale the sky strip, and with one CTA per channel the strips themselves
-    unsigned *xmax = nullptr;
-    StripArgs sa;
-    bool strips = false;
-    if constexpr (std::is_same<R, float>::value)
-        if (c.ha.on && c.mtc.on) {
-            strips = ha_strip_args(c, sa);
-            if (!strips) FM_CK(cudaMemsetAsync(c.ha.xmax, 0, sizeof(unsigned) * c.F, st));
-            xmax = c.ha.xmax;
-        }
     const bool dc = c.dc_split;
-    FM_TRY(launch_modes_forward<R>(c, a, xbuf, st, dc ? 1 : 0, xmax, strips ? &sa : nullptr));
-    return run_vis<R>(c, xbuf, vis, st, dc ? a : nullptr, dc ? c.nk : 0, xmax != nullptr, strips, partials_only);
+    FM_TRY(launch_modes_forward<R>(c, a, xbuf, st, dc ? 1 : 0));
+    return run_vis<R>(c, xbuf, vis, st, dc ? a : nullptr, dc ? c.nk : 0);
 }
+
+template <typename R>
+fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st)
+{
+    if constexpr (std::is_same<R, float>::value)
+        if (c.ha.on && c.ha.dual) {
+            HaSky ka, kb;
+            FM_TRY(sky_of_modes(c, a, xa, va, 0, st, ka));
+            FM_TRY(sky_of_modes(c, b, xb, vb, 1, st, kb));
+            return launch_vis_ha_dual(c, ka, kb);
+        }
+    FM_TRY(vis_of_modes<R>(c, a, xa, va, st));
+    return vis_of_modes<R>(c, b, xb, vb, st);
+}
+template fm_status vis_of_two<float>(Ctx &, const float *, float *, float *, const float *, float *, float *, cudaStream_t);
+template fm_status vis_of_two<double>(Ctx &, const double *, double *, double *, const double *, double *, double *,
+                                      cudaStream_t);
 template fm_status vis_of_modes<float>(Ctx &, const float *, float *, float *, cudaStream_t, bool);
 template fm_status vis_of_modes<double>(Ctx &, const double *, double *, double *, cudaStream_t, bool);
 
@@ -392,8 +429,7 @@ static fm_status run_hvp(Ctx &c, const R *theta, const R *v, R *hv, int full, cu
         sky = (const R *)c.ax;
         vsky = (const R *)c.avx;
     }
-    FM_TRY(vis_of_modes<R>(c, sky, x, (R *)c.vis, st));
-    FM_TRY(vis_of_modes<R>(c, vsky, xv, (R *)c.dvis, st));
+    FM_TRY(vis_of_two<R>(c, sky, x, (R *)c.vis, vsky, xv, (R *)c.dvis, st));
     FM_TRY(launch_hvp_mid<R>(c, (R *)c.vis, (R *)c.dvis, (R *)c.gains, (R *)c.dgains, full, (R *)c.omega,
                              (R *)c.zpart, st));
     FM_TRY(run_adjoint<R>(c, (R *)c.omega, (R *)c.xbar, st));

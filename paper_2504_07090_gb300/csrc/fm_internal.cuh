@@ -136,8 +136,11 @@ struct HaState {
     int nmt = 0;               // forward M-tiles, ceil(U / 64)
     int nkq = 0;               // adjoint K-chunks, ceil(U / 32)
     int npad = 0;              // LSTs per pass (at most 64) rounded up to 16 (MMA N)
+    int npf = 0;               // the forward's LSTs per pass (at most 64; wide: 128) rounded up to 16
+    bool wide = false;         // forward passes of up to 128 LSTs (T > 64)
+    bool dual = false;         // T <= 64: the forward can take two skies in one pass
     int Jc = 0, Ly = 0;        // forward sky image chunks; sky-strip length (16-bit elements)
-    int Lyc = 0;               // strip elements one pass of at most 64 LSTs reads
+    int Lyc = 0;               // strip elements one forward pass reads
     int grid = 0, J = 0;       // forward CTAs; partial sums per (M-tile, channel) segment (vpart stride)
     int J_alloc = 0;           // J of the default grid (the allocation)
     int grid_adj = 0;          // adjoint CTAs (0: one per SM)
@@ -149,10 +152,10 @@ struct HaState {
     int *moff = nullptr;       // [U + 1] CSR offsets of group members
     int *mem = nullptr;        // [B] members, b * 2 + reversed
     int *ncontrib = nullptr;   // [nmt * F] forward CTAs contributing to each segment
-    uint16_t *ys = nullptr;    // [2][F][D][Ly] scaled sky strips in the forward's cell order, hi then lo
-    unsigned *xmax = nullptr;  // [F] max |x| of the centred sky per channel, as float bits
+    uint16_t *ys = nullptr;    // [sky][2][F][D][Ly] scaled sky strips in the forward's cell order, hi then lo
+    unsigned *xmax = nullptr;  // [sky][F] max |x| of the centred sky per channel, as float bits
     float *ug = nullptr;       // [F][T][U][2] monopole visibility of each group (k_ha_monopole)
-    float *vpart = nullptr;    // [nmt * F][J][128][npad] forward partial sums
+    float *vpart = nullptr;    // [nmt * F][J][npf (two skies: 2 npad)][128] forward partial sums
     float *q32 = nullptr;      // [F][T][U][2] residual weights summed per group
     float *qmax_ft = nullptr;  // [F][T] max |Re Q|, |Im Q| per (channel, LST)
     float *qscale = nullptr;   // [F]
@@ -380,7 +383,7 @@ struct StripArgs {
 };
 // the hour-angle form's strips as a StripArgs when the transform can write them (one CTA
 // per channel: at most 128 declinations)
-bool ha_strip_args(const Ctx &c, StripArgs &sa);
+bool ha_strip_args(const Ctx &c, StripArgs &sa, int slot);
 
 template <typename R>
 // a -> x; xmax != NULL (tensor-core transform only): also each channel's largest |x| (as
@@ -451,6 +454,9 @@ fm_status launch_center(Ctx &c, const R *x, R *xc, R *mean, cudaStream_t st);
 fm_status launch_d2f(long long n, const double *a, float *b, cudaStream_t st);
 template <typename R>
 fm_status vis_of_modes(Ctx &c, const R *a, R *xbuf, R *vis, cudaStream_t st, bool partials_only = false);
+// the same for two skies a and b (into xa, va and xb, vb), in one forward pass where the handle has it
+template <typename R>
+fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st);
 
 // tensor-core contraction (sm_103a tcgen05); returns FM_ERR_UNSUPPORTED when the
 // shape does not fit its tiles
@@ -506,13 +512,24 @@ struct MapWindows {
 };
 fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st,
                                        const MapWindows *w = nullptr);
-// dc != nullptr: also adds the monopole visibilities dc[f * dcs] U[f][t][b]; xmax_ready: the
-// channel maxima of x are already in c.ha.xmax (formed by the mode transform); strips_ready:
-// so are the sky strips of x (written by the mode transform); partials_only: V is not
-// finished (the forward's partial sums stay in c.ha.vpart for the chi^2 epilogue, HaVSrc)
-fm_status launch_vis_ha(Ctx &c, const float *x, float *vis, cudaStream_t st, const float *dc = nullptr,
-                        long long dcs = 0, bool xmax_ready = false, bool strips_ready = false,
-                        bool partials_only = false);
+// One sky of the hour-angle forward: pixels x -> visibilities vis.  dc != nullptr: also adds the
+// monopole visibilities dc[f * dcs] U[f][t][b]; slot: which of the two strip and maxima buffers it uses;
+// xmax_ready: the channel maxima of x are already in c.ha.xmax (formed by the mode transform);
+// strips_ready: so are the sky strips of x (written by the mode transform).
+struct HaSky {
+    const float *x;
+    float *vis;
+    cudaStream_t st;
+    const float *dc = nullptr;
+    long long dcs = 0;
+    int slot = 0;
+    bool xmax_ready = false, strips_ready = false;
+};
+// partials_only: V is not finished (the forward's partial sums stay in c.ha.vpart for the chi^2
+// epilogue, HaVSrc)
+fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only = false);
+// two skies (slots 0 and 1) in one pass over the responses; needs c.ha.dual
+fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b);
 // q_ready: the group sums q32 / qmax_ft were already formed from omega (by the chi^2 epilogue)
 fm_status launch_adjoint_ha(Ctx &c, const float *omega, float *xbar, cudaStream_t st, bool q_ready = false);
 

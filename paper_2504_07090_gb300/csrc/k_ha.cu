@@ -55,21 +55,24 @@ constexpr int HA_SMEM_BUDGET = 227 * 1024 - 1024 - 512;
 constexpr int HA_EW = 66;                 // float2 entries per table row: 64 cells + 16 bytes of padding
 constexpr int HA_NSTAGE = 4;              // adjoint operand stages (A in TMEM, B in shared memory)
 constexpr int HA_TCHUNK = 64;             // LSTs per pass (the GEMM's N); more run as several passes
-constexpr int HA_NSTAGE_FWD = 5;          // forward A stages in TMEM
+constexpr int HA_TWIDE = 128;             // LSTs per pass of the wide forward
+constexpr int HA_NSTAGE_FWD = 5;          // forward A stages in TMEM (as many as fit beside the wide accumulators)
 // the forward's roles: HF_PROD_WARPS producer warps in HF_PGROUPS groups of four (one unit each),
-// then four TMEM-drain warps, the MMA warp and the bulk-copy warp
+// then four (wide: eight) TMEM-drain warps, the MMA warp and the bulk-copy warp
 constexpr int HF_PROD_WARPS = 12;
 constexpr int HF_PGROUPS = HF_PROD_WARPS / 4;
 constexpr int HF_EPI_WARP0 = HF_PROD_WARPS;
-constexpr int HF_MMA_WARP = HF_PROD_WARPS + 4;
-constexpr int HF_LOAD_WARP = HF_PROD_WARPS + 5;
-constexpr int HF_THREADS = (HF_PROD_WARPS + 6) * 32;
-static_assert((HF_MMA_WARP & 3) == 0 && HF_EPI_WARP0 + 4 == HF_MMA_WARP, "the MMA warp on the first sub-partition");
+template <bool WIDE> struct HfRole {
+    static constexpr int epi = WIDE ? 8 : 4;                   // drain warps
+    static constexpr int mma = HF_PROD_WARPS + epi, load = mma + 1, threads = (load + 1) * 32;
+    static_assert((mma & 3) == 0, "the MMA warp on the first sub-partition");
+};
 
 // kernel parameters, by value
 struct HaDev {
     int F, D, T, R, A, U, k, q, nhp, nbc, npad, Ly, Jc, nchunk, nmt, nkq, J;   // k: LST step, q: cells per pixel
     int Tt, t0, Lyc;                      // all LSTs; this LST chunk: [t0, t0 + T); strip bytes / 2 it reads
+    int N, dual;                          // forward: MMA columns (partial-sum rows a contributor); two skies
     long long Q;                          // forward work units: nmt * F * nchunk
     const float2 *E;                      // phasor table, cells paired (forward)
     const float2 *Ea;                     // the same, one (Re, Im) per cell (adjoint)
@@ -80,6 +83,7 @@ struct HaLayout {
     int nstage, neslot, ncols, abase, acols;   // TMEM: allocated columns, first A column, columns per A stage
     uint32_t b_bytes, stage_bytes, eslot_bytes, img_bytes;
     uint32_t e_off, v_off, bar_off;
+    uint32_t tab_off;                          // wide forward: image offset and K step of every MMA
     size_t smem;
 };
 
@@ -298,9 +302,15 @@ __global__ void k_ha_yprep(HaDev h, const float *__restrict__ x, const unsigned 
 // img[part][j][rho][e] = ys[part][8 j + rho k + e], 16 bytes per (j, rho), j < Jc.
 // K known at compile time: thread task (part, j) loads the strip words it needs with
 // 16-byte loads and forms the eight chunks in registers (byte permutes for odd shifts).
+// Place of chunk j of sky s in the image.  One sky: j.  Two skies share an image so that one MMA reads both
+// (N = their LSTs, in alternating groups of eight): chunk (j mod k) + k (2 (j div k) + s), in which j + k,
+// the next group of eight LSTs, lies 2 k further on and the other sky's group k further on, so the
+// tile's 8-row groups are k chunks apart throughout.
+__device__ __forceinline__ int img_chunk(int j, int k, int s, bool dual) { return dual ? j % k + k * (2 * (j / k) + s) : j; }
+
 template <int K, int NT>
 __device__ __forceinline__ void build_image(const uint32_t *strip, int Ly, int Jc, uint32_t img_bytes, uint8_t *img,
-                                            int t0, int nthr)
+                                            int t0, int nthr, int s = 0, bool dual = false)
 {
     constexpr int NW4 = ((7 * K + 7) / 2 + 5) / 4;   // 16-byte words covering elements 8 j .. 8 j + 7 K + 8
     for (int task = t0; task < NT * Jc; task += nthr) {
@@ -312,7 +322,7 @@ __device__ __forceinline__ void build_image(const uint32_t *strip, int Ly, int J
             const uint4 v = src[q];
             w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(img + (size_t)part * img_bytes + (size_t)j * 128);
+        uint4 *dst = reinterpret_cast<uint4 *>(img + (size_t)part * img_bytes + (size_t)img_chunk(j, K, s, dual) * 128);
 #pragma unroll
         for (int rho = 0; rho < 8; ++rho) {
             const int sft = rho * K, ws = sft >> 1;
@@ -333,7 +343,7 @@ __device__ __forceinline__ void build_image(const uint32_t *strip, int Ly, int J
 // the same for any k: one 16-byte chunk per thread task
 template <int NT>
 __device__ __forceinline__ void build_image_any(const uint32_t *strip, int Ly, int Jc, int k, uint32_t img_bytes,
-                                                uint8_t *img, int t0, int nthr)
+                                                uint8_t *img, int t0, int nthr, int s = 0, bool dual = false)
 {
     const int nch = Jc * 8;
     for (int e = t0; e < NT * nch; e += nthr) {
@@ -349,7 +359,7 @@ __device__ __forceinline__ void build_image_any(const uint32_t *strip, int Ly, i
         } else {
             o = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        *reinterpret_cast<uint4 *>(img + (size_t)part * img_bytes + (size_t)j * 128 + rho * 16) = o;
+        *reinterpret_cast<uint4 *>(img + (size_t)part * img_bytes + (size_t)img_chunk(j, k, s, dual) * 128 + rho * 16) = o;
     }
 }
 
@@ -378,11 +388,19 @@ __device__ __forceinline__ void build_image_any(const uint32_t *strip, int Ly, i
 //     a group, and accf[q] at the end of a chain of HA_SUB units or a segment
 //   epilogue (16-19): adds the chain into the segment's running sum in TMEM columns
 //     [2 npad, 3 npad), writes it at the end of a segment;  acce[q] (4 arrivals)
-template <int ET, bool X3>
-__global__ void __launch_bounds__(HF_THREADS, 1)
+// WIDE: up to 128 MMA columns instead of 64, for more than 64 LSTs or for two skies at once (ys2: the
+// Hessian-vector product's model and tangent), so that a P tile, the kernel's main cost, is formed once
+// for all of them; an N = 128 MMA also runs at the dense rate (64 cycles against 46 for N = 64).  The
+// accumulators then leave 256 TMEM columns, four A stages, and the running sums live in the registers of eight
+// drain warps (alternate 16-column groups).  Two skies: see img_chunk; column 16 g + 8 s + rho is LST
+// 8 g + rho of sky s, stored in partial row s npad + t.  The sums of every LST are those of the narrow form.
+template <int ET, bool X3, bool WIDE>
+__global__ void __launch_bounds__(HfRole<WIDE>::threads, 1)
 k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t *__restrict__ ys_lo,
-         float *__restrict__ vpart, int *__restrict__ status)
+         const uint16_t *__restrict__ ys2_hi, const uint16_t *__restrict__ ys2_lo, float *__restrict__ vpart,
+         int *__restrict__ status)
 {
+    using Role = HfRole<WIDE>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = su32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -407,13 +425,19 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
         }
         for (int q = 0; q < 2; ++q) {
             mbar_init(accf0 + 8 * q, 1);
-            mbar_init(acce0 + 8 * q, 4);
+            mbar_init(acce0 + 8 * q, Role::epi);
             mbar_init(iempty0 + 8 * q, 1);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == HF_MMA_WARP) tmem_alloc(su32(tmem_slot), (uint32_t)L.ncols);
+    if (warp == Role::mma) tmem_alloc(su32(tmem_slot), (uint32_t)L.ncols);
+    uint2 *tab = reinterpret_cast<uint2 *>(gbase + L.tab_off);       // wide: [nbc][4] image offset and K step
+    if (WIDE)
+        for (int e = tid; e < 4 * h.nbc; e += blockDim.x) {
+            const int j0 = img_chunk(2 * e, h.k, 0, h.dual != 0), j1 = img_chunk(2 * e + 1, h.k, 0, h.dual != 0);
+            tab[e] = make_uint2(128u * (uint32_t)j0, 128u * (uint32_t)(j1 - j0));
+        }
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -469,11 +493,14 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
                     mbar_wait_ab(iempty0 + 8 * gb, (uint32_t)(((gi >> 1) - 1) & 1), abort_flag);
                 __syncwarp();
                 if (*abort_flag) goto done;
-                const uint32_t *strip = reinterpret_cast<const uint32_t *>(eslot + eb);
                 uint8_t *img = gbase + (size_t)(gb * NT) * L.img_bytes;
-                if (h.k == 1) build_image<1, NT>(strip, h.Lyc, h.Jc, L.img_bytes, img, gt, 128);
-                else if (h.k == 2) build_image<2, NT>(strip, h.Lyc, h.Jc, L.img_bytes, img, gt, 128);
-                else build_image_any<NT>(strip, h.Lyc, h.Jc, h.k, L.img_bytes, img, gt, 128);
+                const bool dual = WIDE && h.dual;
+                for (int sk = 0; sk < (dual ? 2 : 1); ++sk) {
+                    const uint32_t *strip = reinterpret_cast<const uint32_t *>(eslot + eb + (uint32_t)(sk * NT) * sb);
+                    if (h.k == 1) build_image<1, NT>(strip, h.Lyc, h.Jc, L.img_bytes, img, gt, 128, sk, dual);
+                    else if (h.k == 2) build_image<2, NT>(strip, h.Lyc, h.Jc, L.img_bytes, img, gt, 128, sk, dual);
+                    else build_image_any<NT>(strip, h.Lyc, h.Jc, h.k, L.img_bytes, img, gt, 128, sk, dual);
+                }
             }
             {
                 const uint32_t ta = ta_row + (uint32_t)(s * L.acols);
@@ -520,7 +547,7 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
             if (lane == 0) mbar_arrive(full0 + 8 * s);
             c = (c + HF_PGROUPS) % h.nbc;
         }
-    } else if (warp == HF_LOAD_WARP) {
+    } else if (warp == Role::load) {
         // ------------------------------------------------------------ bulk loads of E chunks
         if (lane == 0) {
             int se = 0, last_se = -1;
@@ -535,11 +562,16 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
                 const uint32_t dst = base + L.e_off + (uint32_t)se * L.eslot_bytes;
                 // the chunk's LSTs start t0 k elements into the strip (t0 a multiple of 64)
                 const size_t row = ((size_t)f * h.D + d) * h.Ly + (size_t)h.t0 * h.k;
-                mbar_expect_tx(efull0 + 8 * se, eb + (gstart ? (uint32_t)NT * sb : 0u));
+                const bool dual = WIDE && h.dual;
+                mbar_expect_tx(efull0 + 8 * se, eb + (gstart ? (uint32_t)(dual ? 2 * NT : NT) * sb : 0u));
                 bulk_g2s(dst, src, eb, efull0 + 8 * se);
                 if (gstart) {
                     bulk_g2s(dst + eb, ys_hi + row, sb, efull0 + 8 * se);
                     if (X3) bulk_g2s(dst + eb + sb, ys_lo + row, sb, efull0 + 8 * se);
+                    if (dual) {
+                        bulk_g2s(dst + eb + NT * sb, ys2_hi + row, sb, efull0 + 8 * se);
+                        if (X3) bulk_g2s(dst + eb + 3 * sb, ys2_lo + row, sb, efull0 + 8 * se);
+                    }
                 }
                 last_se = se;
                 last_eph = eph;
@@ -560,10 +592,10 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
                 }
             }
         }
-    } else if (warp == HF_MMA_WARP) {
+    } else if (warp == Role::mma) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16(128, h.npad, Elem<ET>::kFmt);
+            const uint32_t idesc = idesc_f16(128, h.N, Elem<ET>::kFmt);
             const uint32_t sbo = 128u * (uint32_t)h.k;
             int s = 0, last_s = -1, gb = 0;
             uint32_t ph = 0, last_ph = 0;
@@ -581,15 +613,16 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
                 if (!mbar_wait_ab<32>(full0 + 8 * s, ph, abort_flag)) goto mma_done;
                 tc_fence_after();
                 {
-                    const uint32_t dacc = tmem_d + (uint32_t)(qa * h.npad);
+                    const uint32_t dacc = tmem_d + (uint32_t)(qa * h.N);
                     const uint32_t ta = tmem_d + (uint32_t)(L.abase + s * L.acols);
-                    const uint32_t ib = base + (uint32_t)(gb * NT) * L.img_bytes + (uint32_t)(8 * c) * 128u;
+                    const uint32_t ib = base + (uint32_t)(gb * NT) * L.img_bytes + (WIDE ? 0u : (uint32_t)(8 * c) * 128u);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        const uint64_t dbh = sdesc_none(ib + 256u * kk, 128u, sbo);
+                        const uint2 e = WIDE ? tab[4 * c + kk] : make_uint2(256u * kk, 128u);
+                        const uint64_t dbh = sdesc_none(ib + e.x, e.y, sbo);
                         mma_ts(dacc, ta + 8u * kk, dbh, idesc, (chain_first && kk == 0) ? 0u : 1u);
                         if (X3) {
-                            mma_ts(dacc, ta + 8u * kk, sdesc_none(ib + L.img_bytes + 256u * kk, 128u, sbo), idesc, 1u);
+                            mma_ts(dacc, ta + 8u * kk, sdesc_none(ib + L.img_bytes + e.x, e.y, sbo), idesc, 1u);
                             mma_ts(dacc, ta + 32u + 8u * kk, dbh, idesc, 1u);
                         }
                     }
@@ -615,14 +648,17 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
         // u = 16 quarter + 8 b + j (the producers' 16-lane blocks)
         const int quarter = warp & 3, lb = lane & 15;
         const int row = 32 * quarter + 16 * (lane >> 4) + 2 * (lb & 7) + (lb >> 3);
-        // the running sum of the segment lives in TMEM columns [2 npad, 3 npad)
+        // the running sum of the segment lives in TMEM columns [2 npad, 3 npad); wide: in registers,
+        // 16-column groups 2 i + half of the drain warp's half
+        const int half = WIDE ? (warp - HF_EPI_WARP0) >> 2 : 0;
         const uint32_t tsum = tmem_d + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(2 * h.npad);
-        {
-            float z[16];
+        float sum[WIDE ? 4 : 1][16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = 0.f;
-            for (int c16 = 0; c16 < h.npad; c16 += 16) tmem_st16(tsum + (uint32_t)c16, z);
-        }
+        for (int i = 0; i < (WIDE ? 4 : 1); ++i)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[i][j] = 0.f;
+        if (!WIDE)
+            for (int c16 = 0; c16 < h.npad; c16 += 16) tmem_st16(tsum + (uint32_t)c16, sum[0]);
         long long nacc = 0;
         int local = 0, seg = (int)(q0 / h.nchunk), c = (int)(q0 % h.nchunk);
         for (long long q = q0; q < q1; ++q) {
@@ -636,12 +672,34 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
             __syncwarp();
             if (*abort_flag) goto done;
             tc_fence_after();
-            const uint32_t taddr = tmem_d + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(qa * h.npad);
+            const uint32_t taddr = tmem_d + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(qa * h.N);
             float *dst = nullptr;
             if (seg_last) {
                 const int jrank = blockIdx.x - cta_of((long long)seg * h.nchunk, h.Q, G);
-                dst = vpart + ((size_t)seg * h.J + jrank) * h.npad * 128 + row;
+                dst = vpart + ((size_t)seg * h.J + jrank) * h.N * 128 + row;
             }
+            if constexpr (WIDE) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int c16 = 16 * (2 * i + half);
+                    if (c16 < h.N) {
+                        float v[16];
+                        tmem_ld16(taddr + (uint32_t)c16, v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[i][j] += v[j];
+                        if (seg_last) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                // two skies: the group's first eight columns are sky 0's LSTs, the others sky 1's
+                                const int t = h.dual ? (c16 >> 1) + (j & 7) : c16 + j;
+                                const int prow = h.dual && j >= 8 ? h.npad + t : t;
+                                if (t < h.T) dst[(size_t)prow * 128] = sum[i][j];
+                                sum[i][j] = 0.f;
+                            }
+                        }
+                    }
+                }
+            } else
             for (int c16 = 0; c16 < h.npad; c16 += 16) {
                 float v[16], a[16];
                 tmem_ld16(taddr + (uint32_t)c16, v);
@@ -666,7 +724,7 @@ k_vis_ha(HaDev h, HaLayout L, const uint16_t *__restrict__ ys_hi, const uint16_t
 done:
     __syncthreads();
     if (*abort_flag && tid == 0) atomicExch(status, (int)FM_ERR_TIMEOUT);
-    if (warp == HF_MMA_WARP) {
+    if (warp == Role::mma) {
         tc_fence_after();
         tmem_dealloc(tmem_d, (uint32_t)L.ncols);
     }
@@ -693,8 +751,8 @@ __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float 
         const int row = e % 128, tl = e / 128;
         float a = 0.f;
         if (tl < tn) {      // the contributors' rows in rank order, four loads ahead
-            const float *src = vpart + ((size_t)seg * h.J * h.npad + t0 + tl) * 128 + row;
-            const size_t js = (size_t)h.npad * 128;
+            const float *src = vpart + ((size_t)seg * h.J * h.N + t0 + tl) * 128 + row;
+            const size_t js = (size_t)h.N * 128;
             for (int j0 = 0; j0 < nc; j0 += 4) {
                 float v[4];
 #pragma unroll
@@ -1151,7 +1209,7 @@ HaDev make_dev(const Ctx &c)
     HaDev h;
     h.F = c.F; h.D = c.D; h.T = c.T; h.R = c.R; h.A = s.nant + 1; h.U = s.U; h.k = s.k; h.q = s.q;
     h.nhp = s.nhp; h.nbc = s.nbc; h.npad = s.npad; h.Ly = s.Ly; h.Jc = s.Jc;
-    h.Tt = c.T; h.t0 = 0; h.Lyc = s.Lyc; h.T = c.T < HA_TCHUNK ? c.T : HA_TCHUNK;
+    h.Tt = c.T; h.t0 = 0; h.Lyc = s.Lyc; h.T = c.T < HA_TCHUNK ? c.T : HA_TCHUNK; h.N = s.npad; h.dual = 0;
     h.nchunk = c.D * s.nbc; h.nmt = s.nmt; h.nkq = s.nkq; h.J = s.J;
     h.Q = (long long)s.nmt * c.F * h.nchunk;
     h.E = s.E; h.Ea = s.Ea; h.uij = s.uij;
@@ -1168,35 +1226,48 @@ uint32_t adj_scratch_bytes(const Ctx &c)
     return (2u * 32u * (128u + 64u * (uint32_t)c.ha.k + 1u) + 4u * 128u) * 4u + 32u * (uint32_t)c.ha.nkq * 8u;
 }
 
-// TMEM columns of both kernels: the accumulators (two sets, and the forward's running sum),
-// then `nstage` A stages of 32 columns per part
-void tmem_layout(const Ctx &c, bool x3, int nacc_sets, int nstage, HaLayout &L)
+// TMEM columns of both kernels: `acc` columns of accumulators (and the narrow forward's running sum),
+// then up to `nstage` A stages of 32 columns per part
+void tmem_layout(bool x3, int acc, int nstage, HaLayout &L)
 {
-    L.nstage = nstage;
     L.acols = (x3 ? 2 : 1) * 32;
-    L.abase = (nacc_sets * c.ha.npad + 31) / 32 * 32;
+    L.abase = (acc + 31) / 32 * 32;
     L.ncols = 512;
+    L.nstage = std::min(nstage, (L.ncols - L.abase) / L.acols);
 }
 
+// The forward's variants: one pass of at most 64 LSTs (narrow), of at most 128 (wide), or two skies of at
+// most 64 LSTs each.
+enum class HaFwd { narrow, wide, dual };
+
 // forward: two image buffers (hi, lo), then as many table slots (E chunk [A][HA_EW] and
-// the two sky strips) as fit, up to 8, at least 2
-bool make_layout_fwd(const Ctx &c, bool x3, HaLayout &L)
+// the sky strips) as fit, up to 8, at least 2
+bool make_layout_fwd(const Ctx &c, bool x3, HaFwd v, HaLayout &L)
 {
-    const int nt = x3 ? 2 : 1;
-    tmem_layout(c, x3, 3, HA_NSTAGE_FWD, L);
-    if (L.abase + L.nstage * L.acols > L.ncols) return false;
+    const int nt = x3 ? 2 : 1, skies = v == HaFwd::dual ? 2 : 1;
+    const HaState &s = c.ha;
+    if (v == HaFwd::narrow) {
+        tmem_layout(x3, 3 * s.npad, HA_NSTAGE_FWD, L);
+        if (L.nstage < HA_NSTAGE_FWD) return false;
+    } else {
+        tmem_layout(x3, 2 * (v == HaFwd::dual ? 2 * s.npad : s.npf), HA_NSTAGE_FWD, L);
+    }
     L.b_bytes = 0;
     L.stage_bytes = 0;
-    L.img_bytes = (uint32_t)c.ha.Jc * 128u;
-    L.eslot_bytes = (uint32_t)(c.ha.nant + 1) * (uint32_t)(HA_EW * 8) + (uint32_t)nt * (uint32_t)c.ha.Lyc * 2u;
+    // two skies: chunk j < Jc of sky 1 lies below 2 k ceil(Jc / k)
+    const int chunks = v == HaFwd::dual ? 2 * s.k * ((s.Jc + s.k - 1) / s.k) : s.Jc;
+    L.img_bytes = (uint32_t)chunks * 128u;
+    L.eslot_bytes = (uint32_t)(s.nant + 1) * (uint32_t)(HA_EW * 8) + (uint32_t)(skies * nt) * (uint32_t)s.Lyc * 2u;
     L.e_off = 2u * (uint32_t)nt * L.img_bytes;
-    const size_t bars = 16 * (size_t)L.nstage + 48 + 16;
+    const size_t tab = v == HaFwd::narrow ? 0 : 32 * (size_t)s.nbc;
+    const size_t bars = 16 * (size_t)L.nstage + 48 + 16 + tab;
     L.neslot = 8;
     while (L.neslot >= 2 && (size_t)L.e_off + (size_t)L.neslot * L.eslot_bytes + bars + 16 * L.neslot >
                                 (size_t)HA_SMEM_BUDGET)
         --L.neslot;
     if (L.neslot < 2) return false;
-    L.v_off = L.e_off + (uint32_t)L.neslot * L.eslot_bytes;
+    L.tab_off = L.e_off + (uint32_t)L.neslot * L.eslot_bytes;
+    L.v_off = L.tab_off + (uint32_t)tab;
     L.bar_off = L.v_off;
     L.smem = 1024 + (size_t)L.bar_off + 16 * (L.nstage + L.neslot) + 48 + 16;
     return L.smem <= 227 * 1024;
@@ -1207,8 +1278,8 @@ bool make_layout_fwd(const Ctx &c, bool x3, HaLayout &L)
 bool make_layout_adj(const Ctx &c, bool x3, HaLayout &L)
 {
     const int nt = x3 ? 2 : 1;
-    tmem_layout(c, x3, 2, HA_NSTAGE, L);
-    if (L.abase + L.nstage * L.acols > L.ncols) return false;
+    tmem_layout(x3, 2 * c.ha.npad, HA_NSTAGE, L);
+    if (L.nstage < HA_NSTAGE) return false;
     L.b_bytes = (uint32_t)c.ha.npad * 128u;
     L.stage_bytes = (uint32_t)nt * L.b_bytes;
     L.img_bytes = 0;
@@ -1227,49 +1298,94 @@ bool make_layout_adj(const Ctx &c, bool x3, HaLayout &L)
     return L.smem <= 227 * 1024;
 }
 
-template <int ET, bool X3>
-fm_status vis_ha_launch(Ctx &c, const HaDev &h, const float *x, float *vis, cudaStream_t st, const float *dc,
-                        long long dcs, bool xmax_ready, bool strips_ready, bool partials_only)
+// channel maxima and sky strips of one sky, where the mode transform has not left them already
+template <int ET>
+fm_status sky_prep(Ctx &c, const HaDev &h, const HaSky &k)
 {
-    HaState &s = c.ha;
-    HaLayout L;
-    if (!make_layout_fwd(c, X3, L)) {
-        set_error("hour-angle forward tiles exceed shared memory");
-        return FM_ERR_UNSUPPORTED;
-    }
-    uint16_t *ys_hi = s.ys, *ys_lo = s.ys + (size_t)c.F * c.D * s.Ly;
-    if (!xmax_ready) {
-        FM_CK(cudaMemsetAsync(s.xmax, 0, sizeof(unsigned) * c.F, st));
-        k_ha_xmax<<<dim3(cdiv(c.npix, 256 * 8), c.F), 256, 0, st>>>(c.npix, x, s.xmax);
+    const HaState &s = c.ha;
+    unsigned *xmax = s.xmax + (size_t)k.slot * c.F;
+    uint16_t *ys = s.ys + (size_t)k.slot * 2 * c.F * c.D * s.Ly;
+    if (!k.xmax_ready) {
+        FM_CK(cudaMemsetAsync(xmax, 0, sizeof(unsigned) * c.F, k.st));
+        k_ha_xmax<<<dim3(cdiv(c.npix, 256 * 8), c.F), 256, 0, k.st>>>(c.npix, k.x, xmax);
         FM_CK_LAUNCH();
     }
-    if (!strips_ready) {
-        k_ha_yprep<ET><<<1024, 256, 0, st>>>(h, x, s.xmax, ys_hi, ys_lo);
-        FM_CK_LAUNCH();
-    }
-    FM_CK(smem_opt_in(k_vis_ha<ET, X3>));
-    // one pass per chunk of at most HA_TCHUNK LSTs (the partial sums are reused)
-    for (int t0 = 0; t0 < c.T; t0 += HA_TCHUNK) {
-        HaDev hc = h;
-        hc.t0 = t0;
-        hc.T = c.T - t0 < HA_TCHUNK ? c.T - t0 : HA_TCHUNK;
-        FM_TRY(profiled(c, 0, st, [&]() -> fm_status {
-            k_vis_ha<ET, X3><<<s.grid, HF_THREADS, L.smem, st>>>(hc, L, ys_hi, ys_lo, s.vpart, c.status);
-            FM_CK_LAUNCH();
-            return FM_OK;
-        }));
-        if (partials_only) {
-            if (c.T > HA_TCHUNK) {
-                set_error("the forward's partial sums hold one pass of at most %d LSTs", HA_TCHUNK);
-                return FM_ERR_STATE;
-            }
-            continue;
-        }
-        k_ha_vfinish<<<dim3(s.nmt * c.F, cdiv(hc.T, HA_VF_T)), 256, 0, st>>>(hc, c.B, s.vpart, s.ncontrib, s.bmap,
-                                                                             s.xmax, s.sp, dc, dcs, c.dc_u, vis);
+    if (!k.strips_ready) {
+        k_ha_yprep<ET><<<1024, 256, 0, k.st>>>(h, k.x, xmax, ys, ys + (size_t)c.F * c.D * s.Ly);
         FM_CK_LAUNCH();
     }
     return FM_OK;
+}
+
+template <int ET, bool X3, bool WIDE>
+fm_status fwd_pass(Ctx &c, const HaDev &h, const HaLayout &L, cudaStream_t st)
+{
+    const HaState &s = c.ha;
+    const size_t part = (size_t)c.F * c.D * s.Ly;      // strips: [sky][hi, lo][F][D][Ly]
+    FM_CK(smem_opt_in(k_vis_ha<ET, X3, WIDE>));
+    return profiled(c, 0, st, [&]() -> fm_status {
+        k_vis_ha<ET, X3, WIDE><<<s.grid, HfRole<WIDE>::threads, L.smem, st>>>(
+            h, L, s.ys, s.ys + part, s.ys + 2 * part, s.ys + 3 * part, s.vpart, c.status);
+        FM_CK_LAUNCH();
+        return FM_OK;
+    });
+}
+
+fm_status fwd_finish(Ctx &c, const HaDev &h, const HaSky &k)
+{
+    const HaState &s = c.ha;
+    k_ha_vfinish<<<dim3(s.nmt * c.F, cdiv(h.T, HA_VF_T)), 256, 0, k.st>>>(
+        h, c.B, s.vpart + (size_t)(h.dual ? k.slot : 0) * s.npad * 128, s.ncontrib, s.bmap,
+        s.xmax + (size_t)k.slot * c.F, s.sp, k.dc, k.dcs, c.dc_u, k.vis);
+    FM_CK_LAUNCH();
+    return FM_OK;
+}
+
+template <int ET, bool X3>
+fm_status vis_ha_launch(Ctx &c, const HaDev &h, const HaSky &k, bool partials_only)
+{
+    HaState &s = c.ha;
+    HaLayout L;
+    if (!make_layout_fwd(c, X3, s.wide ? HaFwd::wide : HaFwd::narrow, L)) {
+        set_error("hour-angle forward tiles exceed shared memory");
+        return FM_ERR_UNSUPPORTED;
+    }
+    FM_TRY(sky_prep<ET>(c, h, k));
+    // one pass per chunk of at most 64 (wide: 128) LSTs (the partial sums are reused)
+    const int tc = s.wide ? HA_TWIDE : HA_TCHUNK;
+    if (partials_only && c.T > tc) {
+        set_error("the forward's partial sums hold one pass of at most %d LSTs", tc);
+        return FM_ERR_STATE;
+    }
+    for (int t0 = 0; t0 < c.T; t0 += tc) {
+        HaDev hc = h;
+        hc.t0 = t0;
+        hc.T = c.T - t0 < tc ? c.T - t0 : tc;
+        hc.N = s.npf;
+        FM_TRY(s.wide ? (fwd_pass<ET, X3, true>(c, hc, L, k.st)) : (fwd_pass<ET, X3, false>(c, hc, L, k.st)));
+        if (!partials_only) FM_TRY(fwd_finish(c, hc, k));
+    }
+    return FM_OK;
+}
+
+// two skies in one pass (s.dual)
+template <int ET, bool X3>
+fm_status vis_ha_dual_launch(Ctx &c, const HaDev &h, const HaSky &a, const HaSky &b)
+{
+    HaState &s = c.ha;
+    HaLayout L;
+    if (!s.dual || !make_layout_fwd(c, X3, HaFwd::dual, L)) {
+        set_error("the handle has no two-sky forward");
+        return FM_ERR_STATE;
+    }
+    FM_TRY(sky_prep<ET>(c, h, a));
+    FM_TRY(sky_prep<ET>(c, h, b));
+    HaDev hc = h;
+    hc.N = 2 * s.npad;
+    hc.dual = 1;
+    FM_TRY((fwd_pass<ET, X3, true>(c, hc, L, a.st)));
+    FM_TRY(fwd_finish(c, hc, a));
+    return fwd_finish(c, hc, b);
 }
 
 template <int ET, bool X3>
@@ -1387,11 +1503,15 @@ fm_status ha_setup(Ctx &c)
     const int tc = c.T < HA_TCHUNK ? c.T : HA_TCHUNK;       // LSTs per pass
     s.npad = (tc + 15) / 16 * 16;
     if (s.npad < 16) s.npad = 16;
+    s.npf = s.npad;
     // forward image: chunks j < Jc of 8 cells; the sky strip holds the Ly >= 8 Jc + 7 k + 8
     // elements the image reads (a multiple of 8, so strips stay 16-byte aligned)
-    s.Jc = 8 * s.nbc + (s.npad / 8 - 1) * k;
-    s.Lyc = 8 * s.Jc + 8 * k + 8;
-    s.Ly = s.Lyc + ((c.T - 1) / HA_TCHUNK) * HA_TCHUNK * k;   // later passes start t0 k further in
+    auto image = [&](int tchunk) {
+        s.Jc = 8 * s.nbc + (s.npf / 8 - 1) * k;
+        s.Lyc = 8 * s.Jc + 8 * k + 8;
+        s.Ly = s.Lyc + ((c.T - 1) / tchunk) * tchunk * k;     // later passes start t0 k further in
+    };
+    image(HA_TCHUNK);
 
     const FringeGroups &fg = c.fg;
     s.U = fg.U;
@@ -1411,13 +1531,27 @@ fm_status ha_setup(Ctx &c)
     {
         HaLayout L1, L2;
         const bool x3 = x3_of(c.prec);
-        if (!make_layout_fwd(c, x3, L1) || !make_layout_adj(c, x3, L2)) return FM_OK;
+        if (!make_layout_fwd(c, x3, HaFwd::narrow, L1) || !make_layout_adj(c, x3, L2)) return FM_OK;
+        // more than 64 LSTs: passes of 128 where their image fits; else two skies a pass where theirs does
+        s.wide = s.dual = false;
+        if (c.T > HA_TCHUNK) {
+            s.npf = (std::min(c.T, HA_TWIDE) + 15) / 16 * 16;
+            image(HA_TWIDE);
+            s.wide = make_layout_fwd(c, x3, HaFwd::wide, L1);
+            if (!s.wide) {
+                s.npf = s.npad;
+                image(HA_TCHUNK);
+            }
+        } else {
+            s.dual = make_layout_fwd(c, x3, HaFwd::dual, L1);
+        }
     }
 
     // device memory, all of it within half of what is free
     const size_t e_n = (size_t)c.F * c.D * s.nbc * (s.nant + 1) * HA_EW;
-    const size_t ys_n = 2 * (size_t)c.F * c.D * s.Ly;
-    const size_t vp_n = (size_t)s.nmt * c.F * s.J * 128 * s.npad;
+    const int nsky = s.dual ? 2 : 1;
+    const size_t ys_n = 2 * (size_t)nsky * c.F * c.D * s.Ly;
+    const size_t vp_n = (size_t)s.nmt * c.F * s.J * 128 * (s.dual ? 2 * s.npad : s.npf);
     const size_t q_n = (size_t)c.F * c.T * s.U * 2;
     const size_t qi_n = (size_t)c.F * s.nkq * 2 * s.npad * 128;
     const size_t need = 2 * e_n * 8 + ys_n * 2 + vp_n * 4 + q_n * 4 + qi_n + (size_t)s.nmt * 64 * 8;
@@ -1434,7 +1568,7 @@ fm_status ha_setup(Ctx &c)
     FM_TRY(ha_alloc(c, &s.ncontrib, ncontrib.size()));
     FM_TRY(ha_alloc(c, &s.ys, ys_n));
     FM_CK(cudaMemset(s.ys, 0, ys_n * sizeof(uint16_t)));     // strip elements outside the pixels stay zero
-    FM_TRY(ha_alloc(c, &s.xmax, (size_t)c.F));
+    FM_TRY(ha_alloc(c, &s.xmax, (size_t)nsky * c.F));
     FM_TRY(ha_alloc(c, &s.vpart, vp_n));
     s.J_alloc = s.J;
     FM_TRY(ha_alloc(c, &s.q32, q_n));
@@ -1524,22 +1658,26 @@ fm_status ha_monopole(Ctx &c, float *U, cudaStream_t st)
     return rc;
 }
 
-fm_status launch_vis_ha(Ctx &c, const float *x, float *vis, cudaStream_t st, const float *dc, long long dcs,
-                        bool xmax_ready, bool strips_ready, bool partials_only)
+fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only)
 {
     const HaDev h = make_dev(c);
     const bool x3 = x3_of(c.prec), po = partials_only;
-    if (f16_of(c.prec))
-        return x3 ? vis_ha_launch<1, true>(c, h, x, vis, st, dc, dcs, xmax_ready, strips_ready, po)
-                  : vis_ha_launch<1, false>(c, h, x, vis, st, dc, dcs, xmax_ready, strips_ready, po);
-    return x3 ? vis_ha_launch<0, true>(c, h, x, vis, st, dc, dcs, xmax_ready, strips_ready, po)
-              : vis_ha_launch<0, false>(c, h, x, vis, st, dc, dcs, xmax_ready, strips_ready, po);
+    if (f16_of(c.prec)) return x3 ? vis_ha_launch<1, true>(c, h, k, po) : vis_ha_launch<1, false>(c, h, k, po);
+    return x3 ? vis_ha_launch<0, true>(c, h, k, po) : vis_ha_launch<0, false>(c, h, k, po);
+}
+
+fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b)
+{
+    const HaDev h = make_dev(c);
+    const bool x3 = x3_of(c.prec);
+    if (f16_of(c.prec)) return x3 ? vis_ha_dual_launch<1, true>(c, h, a, b) : vis_ha_dual_launch<1, false>(c, h, a, b);
+    return x3 ? vis_ha_dual_launch<0, true>(c, h, a, b) : vis_ha_dual_launch<0, false>(c, h, a, b);
 }
 
 bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
 {
     const HaState &s = c.ha;
-    if (!s.on || c.T > HA_TCHUNK || (dc && !s.ug)) return false;
+    if (!s.on || c.T > (s.wide ? HA_TWIDE : HA_TCHUNK) || (dc && !s.ug)) return false;
     if (const char *e = getenv("FM_HA_FUSED_CHI2"))      // 0: V finished by its own kernel
         if (atoi(e) == 0) return false;
     v.vpart = s.vpart;
@@ -1551,20 +1689,20 @@ bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
     v.ug = s.ug;
     v.sp = s.sp;
     v.J = s.J;
-    v.npad = s.npad;
+    v.npad = s.npf;
     v.nmt = s.nmt;
     v.F = c.F;
     return true;
 }
 
-bool ha_strip_args(const Ctx &c, StripArgs &sa)
+bool ha_strip_args(const Ctx &c, StripArgs &sa, int slot)
 {
     if (!c.ha.on || c.D > 128) return false;
     if (const char *e = getenv("FM_MODES_STRIPS"))      // 0: strips from their own kernel
         if (atoi(e) == 0) return false;
     const HaState &s = c.ha;
-    sa.hi = s.ys;
-    sa.lo = s.ys + (size_t)c.F * c.D * s.Ly;
+    sa.hi = s.ys + (size_t)slot * 2 * c.F * c.D * s.Ly;
+    sa.lo = sa.hi + (size_t)c.F * c.D * s.Ly;
     sa.Ly = s.Ly;
     sa.q = s.q;
     sa.off = s.nhp - 1 - (c.R - 1) * s.q;       // element of pixel 0 (k_ha_yprep)
