@@ -587,7 +587,7 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
 __global__ void __launch_bounds__(MD_THREADS, 1)
 k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *__restrict__ phit_img,
             const uint8_t *__restrict__ legt_img, float *__restrict__ abar_all, int *__restrict__ status, int ncols,
-            MapWindows w)
+            const __grid_constant__ MapWindows w)
 {
     const int f = blockIdx.x, mtile = blockIdx.y;
     const MdSmem m = md_smem(z.Dp > z.Np ? z.Dp : z.Np, ns);
