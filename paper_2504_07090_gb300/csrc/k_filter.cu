@@ -59,9 +59,52 @@ __global__ void __launch_bounds__(256) k_df_resid(DevGeom g, const R *__restrict
     }
 }
 
+// acc[j] = sum_g F[j][g] v[g] (T = false) or sum_g F[g][j] v[g] (T = true) of eight channels j, g ascending,
+// for the lane's column v[g] = s[g DF_COLS]: the column entry is read once for the eight sums, F as
+// 16-byte broadcasts (FP32).  f points at F[f0][0] (T = false) or F[0][f0], rows ld apart.
+template <typename R, bool T>
+__device__ __forceinline__ void df_rows(const R *f, int ld, int nf, const typename Cx<R>::t *s, R (&ar)[8], R (&ai)[8])
+{
+    struct alignas(16) Four { R v[4]; };
+#pragma unroll
+    for (int j = 0; j < 8; ++j) ar[j] = ai[j] = R(0);
+    int g = 0;
+    for (; g + 4 <= nf; g += 4) {
+        typename Cx<R>::t v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = s[(g + q) * DF_COLS];
+#pragma unroll
+        for (int h = 0; h < 8; h += 4) {
+            Four a[4];             // T: rows g + q, channels h ..; else rows (channels) h + q, entries g ..
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                a[q] = *reinterpret_cast<const Four *>(T ? f + (size_t)(g + q) * ld + h : f + (size_t)(h + q) * ld + g);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const R fv = T ? a[q].v[j] : a[j].v[q];
+                    ar[h + j] += fv * v[q].x;
+                    ai[h + j] += fv * v[q].y;
+                }
+        }
+    }
+    for (; g < nf; ++g) {
+        const typename Cx<R>::t v = s[g * DF_COLS];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const R fv = T ? f[(size_t)g * ld + j] : f[(size_t)j * ld + g];
+            ar[j] += fv * v.x;
+            ai[j] += fv * v.y;
+        }
+    }
+}
+
 // In place, per column q = t B + b of r[f][q]: r~ = F r, the CTA's chi^2 partial
-// sum_f w_f |r~_f|^2 (FP64 across warps), then r <- sigma^2 F^T (w r~).  A warp holds one
-// channel row at a time (F read as a broadcast), its lanes the CTA's 32 columns.
+// sum_f w_f |r~_f|^2 (FP64 across warps), then r <- sigma^2 F^T (w r~).  A warp forms eight channels at a
+// time, its lanes the CTA's 32 columns: bound by multiply-adds, where one channel at a time (117 us at 64
+// channels and 39,960 columns) was bound by the two shared-memory reads of every term.  F is held with
+// rows and columns padded to a multiple of eight by zeros.
 template <typename R>
 __global__ void __launch_bounds__(DF_THREADS) k_df_apply(int nf, long long ncol, R sigma2, const R *__restrict__ Fm,
                                                          const R *__restrict__ w, R *__restrict__ r,
@@ -69,37 +112,41 @@ __global__ void __launch_bounds__(DF_THREADS) k_df_apply(int nf, long long ncol,
 {
     using C2 = typename Cx<R>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    R *sF = reinterpret_cast<R *>(smem_raw);                       // [nf][nf]
-    C2 *sA = reinterpret_cast<C2 *>(sF + (size_t)nf * nf + (nf & 1));   // [nf][DF_COLS]
+    const int ld = (nf + 7) & ~7;
+    R *sF = reinterpret_cast<R *>(smem_raw);                       // [ld][ld]
+    C2 *sA = reinterpret_cast<C2 *>(sF + (size_t)ld * ld);         // [nf][DF_COLS]
     C2 *sB = sA + (size_t)nf * DF_COLS;                            // [nf][DF_COLS]
     __shared__ double red[DF_THREADS / 32];
     const int tid = threadIdx.x, c = tid & 31, w0 = tid >> 5;
     const long long q0 = (long long)blockIdx.x * DF_COLS;
     const long long q = q0 + c;
     C2 *rc = reinterpret_cast<C2 *>(r);
-    for (int e = tid; e < nf * nf; e += DF_THREADS) sF[e] = Fm[e];
+#pragma unroll 4
     for (int f = w0; f < nf; f += DF_THREADS / 32) {
         C2 v;
         v.x = v.y = R(0);
         if (q < ncol) v = rc[(size_t)f * ncol + q];
         sA[f * DF_COLS + c] = v;
     }
+    for (int e = tid; e < ld * ld; e += DF_THREADS) {
+        const int i = e / ld, j = e - i * ld;
+        sF[e] = i < nf && j < nf ? Fm[(size_t)i * nf + j] : R(0);
+    }
     __syncthreads();
     R c2 = 0;
-    for (int f = w0; f < nf; f += DF_THREADS / 32) {
-        R ar = 0, ai = 0;
-        for (int g2 = 0; g2 < nf; ++g2) {
-            const R fv = sF[f * nf + g2];
-            const C2 v = sA[g2 * DF_COLS + c];
-            ar += fv * v.x;
-            ai += fv * v.y;
+    R ar[8], ai[8];
+    for (int f = 8 * w0; f < nf; f += DF_THREADS / 4) {
+        df_rows<R, false>(sF + (size_t)f * ld, ld, nf, sA + c, ar, ai);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (f + j >= nf) break;
+            const R wf = w[f + j];
+            c2 += wf * (ar[j] * ar[j] + ai[j] * ai[j]);
+            C2 s;
+            s.x = wf * ar[j];
+            s.y = wf * ai[j];
+            sB[(f + j) * DF_COLS + c] = s;
         }
-        const R wf = w[f];
-        c2 += wf * (ar * ar + ai * ai);
-        C2 s;
-        s.x = wf * ar;
-        s.y = wf * ai;
-        sB[f * DF_COLS + c] = s;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
@@ -110,27 +157,26 @@ __global__ void __launch_bounds__(DF_THREADS) k_df_apply(int nf, long long ncol,
         for (int k = 0; k < DF_THREADS / 32; ++k) a += red[k];
         chi2p[blockIdx.x] = a;
     }
-    for (int f = w0; f < nf; f += DF_THREADS / 32) {
-        R ar = 0, ai = 0;
-        for (int g2 = 0; g2 < nf; ++g2) {
-            const R fv = sF[g2 * nf + f];
-            const C2 v = sB[g2 * DF_COLS + c];
-            ar += fv * v.x;
-            ai += fv * v.y;
-        }
-        if (q < ncol) {
-            C2 o;
-            o.x = sigma2 * ar;
-            o.y = sigma2 * ai;
-            rc[(size_t)f * ncol + q] = o;
-        }
+    for (int f = 8 * w0; f < nf; f += DF_THREADS / 4) {
+        df_rows<R, true>(sF + f, ld, nf, sB + c, ar, ai);
+        if (q < ncol)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (f + j >= nf) break;
+                C2 o;
+                o.x = sigma2 * ar[j];
+                o.y = sigma2 * ai[j];
+                rc[(size_t)(f + j) * ncol + q] = o;
+            }
     }
 }
 
+// shared memory of k_df_apply
 template <typename R>
 size_t df_smem(int nf)
 {
-    return sizeof(R) * ((size_t)nf * nf + (nf & 1)) + 2 * sizeof(typename Cx<R>::t) * (size_t)nf * DF_COLS;
+    const size_t ld = (nf + 7) & ~7;
+    return sizeof(R) * ld * ld + 2 * sizeof(typename Cx<R>::t) * (size_t)nf * DF_COLS;
 }
 
 // F = I - C (C + eps I)^-1 in FP64: Cholesky of M = C + eps I, Y = M^-1 C column by column,
@@ -238,7 +284,9 @@ extern "C" fm_status fm_set_delay_filter(fm_handle h, double tau_max_s, double n
         return FM_ERR_INVALID_ARG;
     }
     const bool fp64 = c.prec == FM_PREC_FP64_SIMT;
-    if (df_smem<float>(c.F) * (fp64 ? 2 : 1) > 200 * 1024) {
+    // F and two columns of every channel; the padding of F to a multiple of eight fits beyond this limit
+    const size_t need = sizeof(float) * ((size_t)c.F * c.F + (c.F & 1)) + 2 * sizeof(float2) * (size_t)c.F * DF_COLS;
+    if (need * (fp64 ? 2 : 1) > 200 * 1024) {
         set_error("delay filter: %d channels exceed the filter kernel's shared memory", c.F);
         return FM_ERR_UNSUPPORTED;
     }
