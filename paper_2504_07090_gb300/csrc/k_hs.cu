@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(256) k_hs_fwd(HsDev h, const typename C2of<R>:
 // V of every member of a group: the splits' partial sums in order, conjugated for reversed
 // members, plus the monopole dc[f dcs] Udc[f][t][b]
 template <typename R>
-__global__ void __launch_bounds__(256) k_group_finish(int F, int T, int U, int nsplit, int B, const typename C2of<R>::t *__restrict__ part,
+__global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int nsplit, int B, const typename C2of<R>::t *__restrict__ part,
                                                    const int *__restrict__ moff, const int *__restrict__ mem,
                                                    const R *__restrict__ dc, long long dcs,
                                                    const float *__restrict__ Udc, R *__restrict__ vis)
@@ -421,11 +421,16 @@ __global__ void __launch_bounds__(256) k_group_finish(int F, int T, int U, int n
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const int u = (int)(e % U);
         const long long ft = e / U;
-        C2 s = part[e];
-        for (int k = 1; k < nsplit; ++k) {
-            const C2 w = part[(size_t)k * n + e];
-            s.x += w.x;
-            s.y += w.y;
+        C2 s = mk2(R(0), R(0));
+        for (int k0 = 0; k0 < nsplit; k0 += 8) {       // in order, eight loads ahead
+            C2 w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) w[k] = k0 + k < nsplit ? part[(size_t)(k0 + k) * n + e] : mk2(R(0), R(0));
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                s.x += w[k].x;
+                s.y += w[k].y;
+            }
         }
         const R cf = dc ? dc[(ft / T) * dcs] : R(0);
         for (int m = moff[u]; m < moff[u + 1]; ++m) {
@@ -663,7 +668,7 @@ static unsigned group_blocks(const Ctx &c)
 template <typename R>
 fm_status launch_group_finish(Ctx &c, int nsplit, const void *part, R *vis, cudaStream_t st, const R *dc, long long dcs)
 {
-    k_group_finish<R><<<group_blocks(c), 256, 0, st>>>(c.F, c.T, c.fg.U, nsplit, c.B, (const typename C2of<R>::t *)part,
+    k_group_finish<R><<<2 * group_blocks(c), 128, 0, st>>>(c.F, c.T, c.fg.U, nsplit, c.B, (const typename C2of<R>::t *)part,
                                                        c.fg.moff, c.fg.mem, dc, dcs, c.dc_u, vis);
     FM_CK_LAUNCH();
     return FM_OK;

@@ -74,9 +74,41 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs a, const R *__restrict__ 
         }
 }
 
+// 16 x 16 tiles, one output a thread: the FP64 form.  FP64 runs at 2 lanes per SM and clock, so the shared
+// memory reads of an untiled product are no bound, and small tiles waste nothing on padding and reach
+// every SM (16 channels of 96 x 16 x 32: 111 us in 64 x 64 tiles on 32 SMs).
+template <typename R>
+__global__ void __launch_bounds__(256) k_gemm16(GemmArgs a, const R *__restrict__ A, const R *__restrict__ B,
+                                                R *__restrict__ C)
+{
+    __shared__ R sA[16][17], sB[16][17];               // [i][k], [k][j]
+    const int b = blockIdx.z, i0 = blockIdx.y * 16, j0 = blockIdx.x * 16, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const R *Ab = A + b * a.sAb, *Bb = B + b * a.sBb;
+    // the fastest thread index runs along the operand's unit stride
+    const int ai = a.sAk == 1 ? ty : tx, ak = a.sAk == 1 ? tx : ty;
+    const int bk = a.sBj == 1 ? ty : tx, bj = a.sBj == 1 ? tx : ty;
+    R acc = R(0);
+    for (int k0 = 0; k0 < a.K; k0 += 16) {
+        sA[ai][ak] = i0 + ai < a.M && k0 + ak < a.K ? Ab[(i0 + ai) * a.sAi + (k0 + ak) * a.sAk] : R(0);
+        sB[bk][bj] = k0 + bk < a.K && j0 + bj < a.N && !(a.zero_b00 && k0 + bk == 0 && j0 + bj == 0)
+                         ? Bb[(k0 + bk) * a.sBk + (j0 + bj) * a.sBj]
+                         : R(0);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc += sA[ty][k] * sB[k][tx];
+        __syncthreads();
+    }
+    if (i0 + ty < a.M && j0 + tx < a.N) C[b * a.sCb + (i0 + ty) * a.sCi + (j0 + tx) * a.sCj] = acc;
+}
+
 template <typename R>
 static fm_status gemm(const GemmArgs &a, int batch, const R *A, const R *B, R *C, cudaStream_t st)
 {
+    if (std::is_same<R, double>::value) {
+        k_gemm16<R><<<dim3(cdiv(a.N, 16), cdiv(a.M, 16), batch), 256, 0, st>>>(a, A, B, C);
+        FM_CK_LAUNCH();
+        return FM_OK;
+    }
     dim3 grid(cdiv(a.N, 64), cdiv(a.M, 64), batch);
     k_gemm<R><<<grid, 256, 0, st>>>(a, A, B, C);
     FM_CK_LAUNCH();
@@ -448,16 +480,20 @@ __global__ void __launch_bounds__(256) k_chi2_mid(DevGeom g, const R *__restrict
 // omega_pq = conj(g_p) g_q r_pq / sigma^2 and the per-antenna gain partials
 // Z_a = [sum_{q>a} r_aq g_q conj(V_aq) + sum_{p<a} conj(r_pa) g_p V_pa] / sigma^2.  The two
 // terms of every baseline are formed once, with its residual; Z_a then sums its A - 1 terms
-// in CF_THREADS / A interleaved chunks (one thread each) and adds the chunks in order.  The
+// in NT / A interleaved chunks (one thread each) and adds the chunks in order.  The
 // gains g_i(nu_f) = sum_k X_k(nu_f) gamma_ik are formed from the coefficients gamma in the
 // prologue.  With q32 != NULL (hour-angle form) omega is not written: its sums over the
 // baseline groups go to q32[f][t][u] and their largest |Re|, |Im| to qmax_ft[f][t].  With
 // hv.vpart != NULL (hour-angle form, one LST pass) V is formed here from the forward's partial
 // sums and the groups' monopole visibilities (HaVSrc) instead of being read from vis.  Needs
 // A <= CF_THREADS.
-constexpr int CF_THREADS = 256;
-template <typename R>
-__global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(DevGeom g, const R *__restrict__ vis, const R *__restrict__ data,
+//
+// NT threads a CTA: 256, eight CTAs an SM, while a (channel, LST)'s terms are small; 1024 where they take
+// so much shared memory (24 bytes a baseline: 192 KB for 127 antennas) that at most three of 256 would
+// fit an SM and its loads would be left uncovered (127 antennas: 3.23 ms with 256).
+constexpr int CF_THREADS = 256, CF_BIG = 1024;
+template <typename R, int NT>
+__global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1) k_chi2_ft(DevGeom g, const R *__restrict__ vis, const R *__restrict__ data,
                                                         const R *__restrict__ gamma, R *__restrict__ omega,
                                                         R *__restrict__ zpart, double *__restrict__ chi2p, int U,
                                                         const int *__restrict__ moff, const int *__restrict__ mem,
@@ -471,13 +507,13 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     C2 *sTj = sTi + g.B;                                   // [B] term of baseline (i, j) in Z_j
     C2 *sW = sTj + g.B;                                    // [B] omega (hour-angle form)
     float *sS = reinterpret_cast<float *>(sW + g.B);       // [nmt][128] forward partial sums (hv)
-    __shared__ C2 sZ[CF_THREADS];                          // chunk sums of Z_a
-    __shared__ double dred[CF_THREADS / 32];
-    __shared__ float fred[CF_THREADS / 32];
+    __shared__ C2 sZ[NT];                          // chunk sums of Z_a
+    __shared__ double dred[NT / 32];
+    __shared__ float fred[NT / 32];
     const int ft = blockIdx.x, f = ft / g.T, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     {
         const R *X = Tab<R>::gleg(g) + (size_t)f * g.NG;
-        for (int i = tid; i < g.A; i += CF_THREADS) {     // as k_gains
+        for (int i = tid; i < g.A; i += NT) {     // as k_gains
             R re = 0, im = 0;
             for (int k = 0; k < g.NG; ++k) {
                 re += X[k] * gamma[(i * g.NG + k) * 2];
@@ -490,7 +526,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     float hsc = 0.f, hcf = 0.f;
     if (hv.vpart) {     // the partial rows of every M-tile at this LST, summed in rank order
         const int t = ft - f * g.T;
-        for (int e = tid; e < hv.nmt * 128; e += CF_THREADS) {
+        for (int e = tid; e < hv.nmt * 128; e += NT) {
             const int seg = (e >> 7) * hv.F + f, row = e & 127, nc = hv.ncontrib[seg];
             // the contributors' rows in rank order, four loads ahead
             const float *src = hv.vpart + ((size_t)seg * hv.J * hv.npad + t) * 128 + row;
@@ -524,7 +560,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     const C2 *rrow = rin ? reinterpret_cast<const C2 *>(rin) + (size_t)ft * g.B : nullptr;
     C2 *orow = reinterpret_cast<C2 *>(omega) + (size_t)ft * g.B;
     R c2 = 0;   // a warp's terms in the working type; FP64 across warps
-    for (int b = tid; b < g.B; b += CF_THREADS) {
+    for (int b = tid; b < g.B; b += NT) {
         const int i = g.bl_i[b], j = g.bl_j[b];
         C2 V;
         if (hv.vpart) {
@@ -575,12 +611,12 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     __syncthreads();
     if (tid == 0) {
         double a = 0.0;
-        for (int k = 0; k < CF_THREADS / 32; ++k) a += dred[k];
+        for (int k = 0; k < NT / 32; ++k) a += dred[k];
         chi2p[ft] = a * g.inv_sigma2;
     }
     if (q32) {
         float qm = 0.f;
-        for (int u = tid; u < U; u += CF_THREADS) {
+        for (int u = tid; u < U; u += NT) {
             float qr = 0.f, qi = 0.f;
             for (int m = moff[u]; m < moff[u + 1]; ++m) {
                 const int code = mem[m], b = code >> 1;
@@ -597,7 +633,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
         if (lane == 0) fred[w] = qm;
     }
     // Z_a, chunk c: partners j = c, c + nc, ... (j != a); pair_index(a, j) = rowa + j for j > a
-    const int nc = CF_THREADS / g.A;
+    const int nc = NT / g.A;
     if (tid < nc * g.A) {
         const int a = tid / nc, c = tid - a * nc;
         const int rowa = a * g.A - (a * (a + 1)) / 2 - a - 1;
@@ -614,7 +650,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     __syncthreads();
     if (q32 && tid == 0) {
         float m = 0.f;
-        for (int k = 0; k < CF_THREADS / 32; ++k) m = fmaxf(m, fred[k]);
+        for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, fred[k]);
         qmax_ft[ft] = m;
     }
     if (tid < g.A) {
@@ -688,8 +724,10 @@ fm_status launch_chi2_chan(Ctx &c, const R *vis, const R *gamma, R *omega, R *zp
         set_error("chi^2 epilogue: %d antennas (at most %d, %zu bytes of shared memory)", c.A, CF_THREADS, smem);
         return FM_ERR_UNSUPPORTED;
     }
-    FM_CK(smem_opt_in(k_chi2_ft<R>));
-    k_chi2_ft<R><<<c.F * c.T, CF_THREADS, smem, st>>>(c.g, vis, (const R *)c.data, gamma, omega, zpart, chi2p, c.ha.U,
+    const bool big = smem > 56 * 1024 && smem <= 208 * 1024;    // the larger CTA's static arrays take up to 17 KB
+    auto *kern = big ? k_chi2_ft<R, CF_BIG> : k_chi2_ft<R, CF_THREADS>;
+    FM_CK(smem_opt_in(kern));
+    kern<<<c.F * c.T, big ? CF_BIG : CF_THREADS, smem, st>>>(c.g, vis, (const R *)c.data, gamma, omega, zpart, chi2p, c.ha.U,
                                                 c.ha.moff, c.ha.mem, groups ? c.ha.q32 : nullptr, c.ha.qmax_ft, rin,
                                                 hv ? *hv : HaVSrc{});
     FM_CK_LAUNCH();

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 GEOMETRIES = {
     "step1": (3, 3, 10, 7, 32), "step2": (2, 2, 5, 9, 32), "half": (2, 2, 30, 5, 48), "step3_2": (4, 2, 20, 5, 96),
     "step3_4": (3, 2, 20, 6, 48), "one": (2, 2, 1, 5, 33), "lst70": (2, 1, 70, 3, 224), "cells300": (2, 1, 5, 3, 304),
-    "offgrid": (3, 6, 3, 7, 41), "offgrid_odd": (4, 5, 2, 5, 29),
+    "hex61": (5, 1, 5, 3, 32), "offgrid": (3, 6, 3, 7, 41), "offgrid_odd": (4, 5, 2, 5, 29),
 }
 
 
