@@ -137,6 +137,7 @@ struct HaState {
     int nkq = 0;               // adjoint K-chunks, ceil(U / 32)
     int npad = 0;              // LSTs per pass (at most 64) rounded up to 16 (MMA N)
     int npf = 0;               // the forward's LSTs per pass (at most 64; wide: 128) rounded up to 16
+    int npa = 0, adj_stages = 4;   // the adjoint's LSTs per pass rounded up to 16, its operand stages
     bool wide = false;         // forward passes of up to 128 LSTs (T > 64)
     bool dual = false;         // T <= 64: the forward can take two skies in one pass
     int Jc = 0, Ly = 0;        // forward sky image chunks; sky-strip length (16-bit elements)
@@ -159,7 +160,7 @@ struct HaState {
     float *q32 = nullptr;      // [F][T][U][2] residual weights summed per group
     float *qmax_ft = nullptr;  // [F][T] max |Re Q|, |Im Q| per (channel, LST)
     float *qscale = nullptr;   // [F]
-    uint8_t *qimg = nullptr;   // [F][nkq][2][npad * 128] swizzled B tiles of the adjoint
+    uint8_t *qimg = nullptr;   // [F][nkq][2][npa * 128] swizzled B tiles of the adjoint
 };
 
 // Fringe groups and drift-scan geometry of a handle (k_hs.cu), shared by every form that

@@ -894,7 +894,9 @@ __global__ void k_ha_qimg(HaDev h, const float *__restrict__ q32, const float *_
 //   MMA warp (20): D[n][t] of the M-tile into TMEM set (M-tile count & 1);  accf[q]
 //   epilogue (16-19 and 23-26, one set per 32-LST half): the diagonal sums over the
 //     M-tiles of the item (see below), one output row xbar(., d) per item.
-template <int ET, bool X3>
+// WIDE: up to 128 LSTs (N = 128), the sets taking alternate groups of 32 in two rounds, so that the P
+// operand is formed once for all of them (127 antennas, 120 LSTs, two passes of 64: 2 x 4.85 ms).
+template <int ET, bool X3, bool WIDE>
 __global__ void __launch_bounds__(HA_ADJ_THREADS, 1)
 k_adj_ha(HaDev h, HaLayout L, const uint8_t *__restrict__ qimg, const float *__restrict__ qscale, float sp,
          float *__restrict__ xbar, int *__restrict__ status)
@@ -1109,7 +1111,6 @@ k_adj_ha(HaDev h, HaLayout L, const uint8_t *__restrict__ qimg, const float *__r
         float *xs1 = reinterpret_cast<float *>(gbase + L.v_off) + (size_t)2 * 32 * skw;  // [4][128]
         for (int e = et; e < 32 * skw; e += 128) sk[e] = 0.f;
         bar_or(1 + eh, 128, false);
-        const int t0 = 32 * eh;
         long long nacc = 0;
         for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
             const int f = it / h.D, d = it % h.D;
@@ -1123,7 +1124,16 @@ k_adj_ha(HaDev h, HaLayout L, const uint8_t *__restrict__ qimg, const float *__r
                 tc_fence_after();
                 const uint32_t taddr = tmem_d + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(qa * h.npad);
                 const int c0 = (h.R - 1) * h.q - 128 * mt + h.t0 * h.k;      // n = t k + c0 - r q (t in the chunk)
-                if (t0 < h.T) {
+                constexpr int rounds = WIDE ? 2 : 1;
+#pragma unroll 1
+                for (int rr = 0; rr < rounds; ++rr) {
+                    const int t0 = 32 * eh + 64 * rr;
+                    const bool last = !WIDE || rr == rounds - 1 || t0 + 64 >= h.T;      // last read of the accumulator
+                    if (t0 >= h.T) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(acce0 + 8 * qa);
+                        break;
+                    }
                     // LST columns t >= T hold zeros (zero residual rows); those past npad are
                     // not loaded and set to zero here
                     float v[32];
@@ -1134,9 +1144,11 @@ k_adj_ha(HaDev h, HaLayout L, const uint8_t *__restrict__ qimg, const float *__r
 #pragma unroll
                         for (int q = 16; q < 32; ++q) v[q] = 0.f;
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(acce0 + 8 * qa);   // the accumulator is read
+                    if (last) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(acce0 + 8 * qa);   // the accumulator is read
+                    }
 #pragma unroll
                     for (int q = 0; q < 32; ++q) sk[q * skw + pk + et] = v[q];
                     bar_or(1 + eh, 128, false);
@@ -1161,9 +1173,7 @@ k_adj_ha(HaDev h, HaLayout L, const uint8_t *__restrict__ qimg, const float *__r
                         xr[j] += (a0 + a1) + (a2 + a3);
                     }
                     bar_or(1 + eh, 128, false);
-                } else {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(acce0 + 8 * qa);
+                    if (last) break;
                 }
             }
             if (stop) break;
@@ -1273,14 +1283,14 @@ bool make_layout_fwd(const Ctx &c, bool x3, HaFwd v, HaLayout &L)
     return L.smem <= 227 * 1024;
 }
 
-// adjoint: HA_NSTAGE residual tiles (B operand), table slots of two E chunks (up to 4, at
+// adjoint: nstage residual tiles of npad LSTs (B operand), table slots of two E chunks (up to 4, at
 // least 2) and the epilogue's scratch
-bool make_layout_adj(const Ctx &c, bool x3, HaLayout &L)
+bool make_layout_adj(const Ctx &c, bool x3, int npad, int nstage, HaLayout &L)
 {
     const int nt = x3 ? 2 : 1;
-    tmem_layout(x3, 2 * c.ha.npad, HA_NSTAGE, L);
-    if (L.nstage < HA_NSTAGE) return false;
-    L.b_bytes = (uint32_t)c.ha.npad * 128u;
+    tmem_layout(x3, 2 * npad, nstage, L);
+    if (L.nstage < nstage) return false;
+    L.b_bytes = (uint32_t)npad * 128u;
     L.stage_bytes = (uint32_t)nt * L.b_bytes;
     L.img_bytes = 0;
     L.eslot_bytes = 2u * (uint32_t)(c.ha.nant + 1) * (uint32_t)(HA_EW * 8);
@@ -1393,7 +1403,7 @@ fm_status adj_ha_launch(Ctx &c, const HaDev &h, const float *omega, float *xbar,
 {
     HaState &s = c.ha;
     HaLayout L;
-    if (!make_layout_adj(c, X3, L)) {
+    if (!make_layout_adj(c, X3, s.npa, s.adj_stages, L)) {
         set_error("hour-angle adjoint tiles exceed shared memory");
         return FM_ERR_UNSUPPORTED;
     }
@@ -1404,16 +1414,20 @@ fm_status adj_ha_launch(Ctx &c, const HaDev &h, const float *omega, float *xbar,
     }
     int grid = s.grid_adj > 0 ? s.grid_adj : sm_count();
     if (grid > c.F * c.D) grid = c.F * c.D;
-    FM_CK(smem_opt_in(k_adj_ha<ET, X3>));
-    // one pass per chunk of at most HA_TCHUNK LSTs; passes after the first add to xbar
-    for (int t0 = 0; t0 < c.T; t0 += HA_TCHUNK) {
+    const bool wide = s.npa > HA_TCHUNK;
+    const int tc = wide ? HA_TWIDE : HA_TCHUNK;
+    auto *kern = wide ? k_adj_ha<ET, X3, true> : k_adj_ha<ET, X3, false>;
+    FM_CK(smem_opt_in(kern));
+    // one pass per chunk of at most 64 (wide: 128) LSTs; passes after the first add to xbar
+    for (int t0 = 0; t0 < c.T; t0 += tc) {
         HaDev hc = h;
         hc.t0 = t0;
-        hc.T = c.T - t0 < HA_TCHUNK ? c.T - t0 : HA_TCHUNK;
+        hc.T = c.T - t0 < tc ? c.T - t0 : tc;
+        hc.npad = s.npa;
         k_ha_qimg<ET, X3><<<c.F * s.nkq, 256, 0, st>>>(hc, s.q32, s.qmax_ft, s.qscale, s.qimg);
         FM_CK_LAUNCH();
         FM_TRY(profiled(c, 1, st, [&]() -> fm_status {
-            k_adj_ha<ET, X3><<<grid, HA_ADJ_THREADS, L.smem, st>>>(hc, L, s.qimg, s.qscale, s.sp, xbar, c.status);
+            kern<<<grid, HA_ADJ_THREADS, L.smem, st>>>(hc, L, s.qimg, s.qscale, s.sp, xbar, c.status);
             FM_CK_LAUNCH();
             return FM_OK;
         }));
@@ -1531,11 +1545,19 @@ fm_status ha_setup(Ctx &c)
     {
         HaLayout L1, L2;
         const bool x3 = x3_of(c.prec);
-        if (!make_layout_fwd(c, x3, HaFwd::narrow, L1) || !make_layout_adj(c, x3, L2)) return FM_OK;
+        if (!make_layout_fwd(c, x3, HaFwd::narrow, L1) || !make_layout_adj(c, x3, s.npad, HA_NSTAGE, L2)) return FM_OK;
         // more than 64 LSTs: passes of 128 where their image fits; else two skies a pass where theirs does
         s.wide = s.dual = false;
+        s.npa = s.npad;
+        s.adj_stages = HA_NSTAGE;
         if (c.T > HA_TCHUNK) {
-            s.npf = (std::min(c.T, HA_TWIDE) + 15) / 16 * 16;
+            const int n = (std::min(c.T, HA_TWIDE) + 15) / 16 * 16;
+            for (int st = HA_NSTAGE; st >= 3 && s.npa == s.npad; --st)
+                if (make_layout_adj(c, x3, n, st, L2)) {
+                    s.npa = n;
+                    s.adj_stages = st;
+                }
+            s.npf = n;
             image(HA_TWIDE);
             s.wide = make_layout_fwd(c, x3, HaFwd::wide, L1);
             if (!s.wide) {
@@ -1553,7 +1575,7 @@ fm_status ha_setup(Ctx &c)
     const size_t ys_n = 2 * (size_t)nsky * c.F * c.D * s.Ly;
     const size_t vp_n = (size_t)s.nmt * c.F * s.J * 128 * (s.dual ? 2 * s.npad : s.npf);
     const size_t q_n = (size_t)c.F * c.T * s.U * 2;
-    const size_t qi_n = (size_t)c.F * s.nkq * 2 * s.npad * 128;
+    const size_t qi_n = (size_t)c.F * s.nkq * 2 * s.npa * 128;
     const size_t need = 2 * e_n * 8 + ys_n * 2 + vp_n * 4 + q_n * 4 + qi_n + (size_t)s.nmt * 64 * 8;
     size_t fr = 0, tot = 0;
     FM_CK(cudaMemGetInfo(&fr, &tot));

@@ -185,10 +185,12 @@ __device__ __forceinline__ float md_absmax(const float *a, int rows, int cols, b
 // past a 16-byte boundary; rows_pad rows, K values 64 ka .. 64 ka + 63), scaled and split into FP16
 // hi / lo rows; entry (0, 0) is read as zero when zero00.  16-byte loads (eight in flight) when cols
 // and ld are multiples of 4 and src - mis is on that boundary.
-__device__ __forceinline__ void md_convert_atom(const float *src, int rows, int cols, int ld, int mis, int rows_pad,
+template <bool WIN>
+__device__ __forceinline__ void md_convert_atom(const float *src, int rows, int cols, int ld_, int mis_, int rows_pad,
                                                 int ka, float sc, bool zero00, uint8_t *b)
 {
     const int n4 = rows_pad * 16;                  // 4-value pieces in the atom
+    const int ld = WIN ? ld_ : cols, mis = WIN ? mis_ : 0;
     const bool vec = ((cols | ld) & 3) == 0 && (reinterpret_cast<uintptr_t>(src - mis) & 15) == 0;
     for (int e0 = threadIdx.x; e0 < n4; e0 += 8 * blockDim.x) {
         float4 v[8];
@@ -399,7 +401,7 @@ struct MdPlan {
     const float *src;       // stage-1 B operand, row-major [src_rows][src_cols]
     int src_rows, src_cols, src_ld;
     int src_mis;            // columns from a 16-byte boundary to src, the same in every row (windows)
-    const unsigned *src_max;   // largest magnitude known beforehand (float bits), or NULL
+    const unsigned *src_max;   // largest magnitude known beforehand (float bits; windows)
     int n1;                 // stage-1 K atoms
     int nb1;                // stage-1 N (rows of its B atoms, padded) = stage-2 K
     int nb2;                // stage-2 N
@@ -433,6 +435,7 @@ __device__ __forceinline__ uint32_t md_setup(const MdSmem &m, int ncols)
 // of atom i.  The first product occupies TMEM columns 0 .. nb1, the second nb1 .. nb1 + nb2.
 // sa and g are the power-of-two scales of the two products' B and A operands.  Returns false
 // after a timeout (abort flag raised; the copies and MMAs in flight drained).
+template <bool WIN>
 __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t tmem, const MdPlan &p, float &sa,
                                              float &g)
 {
@@ -458,7 +461,8 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             img_issue(i);
             (i == 0 ? last_img0 : last_img1) = i;
         }
-    sa = pow2_below(p.src_max ? __uint_as_float(*p.src_max) : md_absmax(p.src, p.src_rows, p.src_cols, p.skip_dc, m.red));
+    if constexpr (WIN) sa = pow2_below(__uint_as_float(*p.src_max));
+    else sa = pow2_below(md_absmax(p.src, p.src_rows, p.src_cols, p.skip_dc, m.red));
     g = 1.f;
     const uint32_t idesc1 = idesc_f16(128, p.nb1, 0), idesc2 = idesc_f16(128, p.nb2, 0);
     bool ok = true;
@@ -479,7 +483,7 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             break;
         }
         if (i < p.n1) {
-            md_convert_atom(p.src, p.src_rows, p.src_cols, p.src_ld, p.src_mis, p.nb1, i, sa, p.skip_dc, m.b(s));
+            md_convert_atom<WIN>(p.src, p.src_rows, p.src_cols, p.src_ld, p.src_mis, p.nb1, i, sa, p.skip_dc, m.b(s));
         } else {
             if (i == p.n1) {
                 tc_fence_after();
@@ -551,7 +555,7 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
     p.nb2 = z.Rp;
     p.skip_dc = skip_dc != 0;
     float sa, g;
-    const bool ok = md_two_stage(m, ns, tmem, p, sa, g);
+    const bool ok = md_two_stage<false>(m, ns, tmem, p, sa, g);
     // x = D2 / (g 2^28 sa), through slot 0's A atom (free once the last MMAs are complete);
     // with strips (one CTA per channel) the channel's largest |x| is read from TMEM first
     // (inv is a power of two, so it is the largest stored |x| exactly) and sets their scale
@@ -584,6 +588,7 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
 // CTA (f, m tile): stage 1 D1[m][d] = PhiT_tile xbar_f^T over r (A = PhiT tile image, B =
 // xbar_f rows d); stage 2 D2[m][n] = U LegT^T over d (A = scaled U from TMEM, B = LegT
 // image); abar = D2 / scales.
+template <bool WIN>
 __global__ void __launch_bounds__(MD_THREADS, 1)
 k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *__restrict__ phit_img,
             const uint8_t *__restrict__ legt_img, float *__restrict__ abar_all, int *__restrict__ status, int ncols,
@@ -600,7 +605,7 @@ k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *_
     p.src_cols = p.src_ld = z.R;
     p.src_mis = 0;
     p.src_max = nullptr;
-    if (w.per > 0) {                            // map f: window f / per of image f % per
+    if constexpr (WIN) {                        // map f: window f / per of image f % per
         const int wi = f / w.per, im = f - wi * w.per;
         p.src = xb_all + w.off[wi] + (size_t)im * z.D * w.ld;
         p.src_ld = w.ld;
@@ -612,7 +617,7 @@ k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *_
     p.nb2 = z.Np;
     p.skip_dc = false;
     float sx, g;
-    const bool ok = md_two_stage(m, ns, tmem, p, sx, g);
+    const bool ok = md_two_stage<WIN>(m, ns, tmem, p, sx, g);
     if (ok) {
         const float inv = 1.f / (g * MD_CSCALE * MD_CSCALE * sx);
         md_store_rows(tmem, z.Dp, z.Np, 128 * mtile, z.M, z.N, inv, abar_all + (size_t)f * z.M * z.N, (size_t)z.N,
@@ -692,7 +697,8 @@ fm_status modes_tc_setup(Ctx &c)
     k_md_image<<<256, 256>>>(c.g.leg64, c.D, c.N, 1, 0, z.Np, z.Dp, MD_CSCALE, s.legt_img);
     FM_CK_LAUNCH();
     FM_CK(smem_opt_in(k_modes_fwd));
-    FM_CK(smem_opt_in(k_modes_adj));
+    FM_CK(smem_opt_in(k_modes_adj<false>));
+    FM_CK(smem_opt_in(k_modes_adj<true>));
     FM_CK(cudaDeviceSynchronize());
     s.on = true;
     return FM_OK;
@@ -727,7 +733,8 @@ fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, flo
     MdDims z = md_dims(c);
     z.F = nmaps;
     const int nmt = (c.M + 127) / 128, ns = md_slots(nmaps * nmt);
-    k_modes_adj<<<dim3(nmaps, nmt), MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
+    auto *kern = w ? k_modes_adj<true> : k_modes_adj<false>;
+    kern<<<dim3(nmaps, nmt), MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
         z, ns, xbar, c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np), w ? *w : MapWindows{});
     FM_CK_LAUNCH();
     return FM_OK;
