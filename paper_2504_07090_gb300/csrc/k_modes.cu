@@ -25,6 +25,10 @@ namespace {
 using namespace tc;
 
 constexpr int MD_THREADS = 256;
+// At most one CTA an SM and a source of at most 128 x 192: 512 threads that hold the whole source in
+// registers (MD_RES_K atoms x MD_RES_U pieces of 16 bytes), so that its largest magnitude and its operand
+// atoms come from one round of loads instead of one for each.
+constexpr int MD_WIDE = 512, MD_RES_K = 3, MD_RES_U = 4;
 constexpr float MD_CSCALE = 16384.f;     // basis tables (|value| <= 1) are stored times 2^14
 
 struct MdDims {
@@ -181,6 +185,22 @@ __device__ __forceinline__ float md_absmax(const float *a, int rows, int cols, b
     return block_max(m, red);
 }
 
+// four consecutive K values of one row of a B atom, scaled and split into its hi and lo rows
+__device__ __forceinline__ void md_put4(const float4 &v, int row, int k, int rows_pad, float sc, uint8_t *b)
+{
+    __half h0, l0, h1, l1, h2, l2, h3, l3;
+    split_h(v.x * sc, h0, l0);
+    split_h(v.y * sc, h1, l1);
+    split_h(v.z * sc, h2, l2);
+    split_h(v.w * sc, h3, l3);
+    const uint32_t off = atom_off(row, k);             // 4 consecutive K values stay in one 16-byte chunk
+    auto pk = [](__half lo16, __half hi16) {
+        return (uint32_t)__half_as_ushort(lo16) | ((uint32_t)__half_as_ushort(hi16) << 16);
+    };
+    *reinterpret_cast<uint2 *>(b + off) = make_uint2(pk(h0, h1), pk(h2, h3));
+    *reinterpret_cast<uint2 *>(b + (size_t)rows_pad * 128 + off) = make_uint2(pk(l0, l1), pk(l2, l3));
+}
+
 // B operand atom from a row-major FP32 matrix src [rows][cols] (rows ld apart, src `mis` columns
 // past a 16-byte boundary; rows_pad rows, K values 64 ka .. 64 ka + 63), scaled and split into FP16
 // hi / lo rows; entry (0, 0) is read as zero when zero00.  16-byte loads (eight in flight) when cols
@@ -225,33 +245,22 @@ __device__ __forceinline__ void md_convert_atom(const float *src, int rows, int 
         for (int u = 0; u < 8; ++u) {
             const int e = e0 + u * blockDim.x;
             if (e >= n4) break;
-            const int row = e >> 4, k = 4 * (e & 15);
-            __half h0, l0, h1, l1, h2, l2, h3, l3;
-            split_h(v[u].x * sc, h0, l0);
-            split_h(v[u].y * sc, h1, l1);
-            split_h(v[u].z * sc, h2, l2);
-            split_h(v[u].w * sc, h3, l3);
-            const uint32_t off = atom_off(row, k);     // 4 consecutive K values stay in one 16-byte chunk
-            auto pk = [](__half lo16, __half hi16) {
-                return (uint32_t)__half_as_ushort(lo16) | ((uint32_t)__half_as_ushort(hi16) << 16);
-            };
-            *reinterpret_cast<uint2 *>(b + off) = make_uint2(pk(h0, h1), pk(h2, h3));
-            *reinterpret_cast<uint2 *>(b + (size_t)rows_pad * 128 + off) = make_uint2(pk(l0, l1), pk(l2, l3));
+            md_put4(v[u], e >> 4, 4 * (e & 15), rows_pad, sc, b);
         }
     }
 }
 
 // TMEM accumulator (128 lanes x ncols columns at column c0) -> scaled FP16 hi/lo A atom
-// for K atom ka of the next product; warps w and w + 4 share lane quarter w & 3 and take
+// for K atom ka of the next product; the warps w & 3 = quarter share that lane quarter and take
 // alternate 16-column groups
+template <int NT>
 __device__ __forceinline__ void md_tmem_to_atom(uint32_t tmem, int c0, int ka, float sc, uint8_t *a)
 {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = w & 3, half = w >> 2;
     const int row = 32 * quarter + lane;
     const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(c0 + 64 * ka);
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-        const int cg = 16 * (2 * g + half);          // columns cg .. cg + 15 of the atom
+    for (int cg = 16 * half; cg < 64; cg += 16 * (NT / 128)) {   // columns cg .. cg + 15 of the atom
         float v[16];
         tmem_ld16(taddr + (uint32_t)cg, v);
 #pragma unroll
@@ -314,6 +323,7 @@ __device__ __forceinline__ void strip_put4(const StripOut &so, int row, int col,
 // float otherwise, two rows an instruction); rows >= nrows and columns >= ncols are skipped.
 // Every stored value also goes to the strips `so` when so.hi != nullptr.  Returns the largest
 // |value| this thread stored.
+template <int NT>
 __device__ __forceinline__ float md_store_rows(uint32_t tmem, int c0, int cols_pad, int row_base, int nrows, int ncols,
                                                float inv, float *__restrict__ out, size_t ld, float *tile,
                                                const StripOut &so)
@@ -324,7 +334,7 @@ __device__ __forceinline__ float md_store_rows(uint32_t tmem, int c0, int cols_p
     float *t = tile + (size_t)w * (32 * 20);
     const bool vec = (ld & 3) == 0 && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
     float mx = 0.f;
-    for (int cg = 16 * half; cg < cols_pad; cg += 32) {
+    for (int cg = 16 * half; cg < cols_pad; cg += NT / 8) {
         float v[16];
         tmem_ld16(taddr + (uint32_t)cg, v);
 #pragma unroll
@@ -380,12 +390,13 @@ __device__ __forceinline__ float md_store_rows(uint32_t tmem, int c0, int cols_p
 }
 
 // largest |value| of a TMEM accumulator (all threads receive it)
+template <int NT>
 __device__ __forceinline__ float md_tmem_max(uint32_t tmem, int c0, int ncols, float *red)
 {
     const int w = threadIdx.x >> 5, quarter = w & 3, half = w >> 2;
     const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)c0;
     float m = 0.f;
-    for (int cg = 16 * half; cg < ncols; cg += 32) {
+    for (int cg = 16 * half; cg < ncols; cg += NT / 8) {
         float v[16];
         tmem_ld16(taddr + (uint32_t)cg, v);
 #pragma unroll
@@ -435,7 +446,7 @@ __device__ __forceinline__ uint32_t md_setup(const MdSmem &m, int ncols)
 // of atom i.  The first product occupies TMEM columns 0 .. nb1, the second nb1 .. nb1 + nb2.
 // sa and g are the power-of-two scales of the two products' B and A operands.  Returns false
 // after a timeout (abort flag raised; the copies and MMAs in flight drained).
-template <bool WIN>
+template <int NT, bool WIN>
 __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t tmem, const MdPlan &p, float &sa,
                                              float &g)
 {
@@ -461,7 +472,40 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             img_issue(i);
             (i == 0 ? last_img0 : last_img1) = i;
         }
-    if constexpr (WIN) sa = pow2_below(__uint_as_float(*p.src_max));
+    constexpr bool RES = NT == MD_WIDE;
+    float4 res[RES ? MD_RES_K : 1][RES ? MD_RES_U : 1];       // piece tid + u NT of K atom ka
+    if constexpr (RES) {
+        const bool vec = (p.src_cols & 3) == 0 && (reinterpret_cast<uintptr_t>(p.src) & 15) == 0;
+#pragma unroll
+        for (int ka = 0; ka < MD_RES_K; ++ka)
+#pragma unroll
+            for (int u = 0; u < MD_RES_U; ++u) {
+                const int e = tid + u * NT, row = e >> 4, k = 64 * ka + 4 * (e & 15);
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row < p.src_rows) {
+                    const float *q = p.src + (size_t)row * p.src_cols + k;
+                    if (vec && k + 3 < p.src_cols) {
+                        x = __ldg(reinterpret_cast<const float4 *>(q));
+                    } else {
+                        if (k < p.src_cols) x.x = __ldg(q);
+                        if (k + 1 < p.src_cols) x.y = __ldg(q + 1);
+                        if (k + 2 < p.src_cols) x.z = __ldg(q + 2);
+                        if (k + 3 < p.src_cols) x.w = __ldg(q + 3);
+                    }
+                    if (p.skip_dc && row == 0 && k == 0) x.x = 0.f;
+                }
+                res[ka][u] = x;
+            }
+        float mx = 0.f;
+#pragma unroll
+        for (int ka = 0; ka < MD_RES_K; ++ka)
+#pragma unroll
+            for (int u = 0; u < MD_RES_U; ++u) {
+                const float4 x = res[ka][u];
+                mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+            }
+        sa = pow2_below(block_max(mx, m.red));
+    } else if constexpr (WIN) sa = pow2_below(__uint_as_float(*p.src_max));
     else sa = pow2_below(md_absmax(p.src, p.src_rows, p.src_cols, p.skip_dc, m.red));
     g = 1.f;
     const uint32_t idesc1 = idesc_f16(128, p.nb1, 0), idesc2 = idesc_f16(128, p.nb2, 0);
@@ -483,13 +527,24 @@ __device__ __forceinline__ bool md_two_stage(const MdSmem &m, int ns, uint32_t t
             break;
         }
         if (i < p.n1) {
-            md_convert_atom<WIN>(p.src, p.src_rows, p.src_cols, p.src_ld, p.src_mis, p.nb1, i, sa, p.skip_dc, m.b(s));
+            if constexpr (RES) {
+#pragma unroll
+                for (int ka = 0; ka < MD_RES_K; ++ka)
+                    if (ka == i)
+#pragma unroll
+                        for (int u = 0; u < MD_RES_U; ++u) {
+                            const int e = tid + u * NT;
+                            if (e < p.nb1 * 16) md_put4(res[ka][u], e >> 4, 4 * (e & 15), p.nb1, sa, m.b(s));
+                        }
+            } else {
+                md_convert_atom<WIN>(p.src, p.src_rows, p.src_cols, p.src_ld, p.src_mis, p.nb1, i, sa, p.skip_dc, m.b(s));
+            }
         } else {
             if (i == p.n1) {
                 tc_fence_after();
-                g = pow2_below(md_tmem_max(tmem, 0, p.nb1, m.red));
+                g = pow2_below(md_tmem_max<NT>(tmem, 0, p.nb1, m.red));
             }
-            md_tmem_to_atom(tmem, 0, i - p.n1, g, m.a(s));
+            md_tmem_to_atom<NT>(tmem, 0, i - p.n1, g, m.a(s));
             tc_fence_before();
         }
         md_filled();
@@ -534,7 +589,8 @@ __device__ __forceinline__ void md_finish(const MdSmem &m, bool ok, int *status,
 // x[f][d][r] = D2 / scales.  xmax != NULL: the largest |x| the CTA wrote goes to xmax[f] by
 // atomicMax on its float bits (non-negative floats order like their bit patterns, so the
 // result is independent of order).
-__global__ void __launch_bounds__(MD_THREADS, 1)
+template <int NT>
+__global__ void __launch_bounds__(NT, 1)
 k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, const uint8_t *__restrict__ leg_img,
             const uint8_t *__restrict__ phi_img, float *__restrict__ x_all, int *__restrict__ status, int ncols,
             unsigned *__restrict__ xmax, StripArgs sp)
@@ -555,14 +611,14 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
     p.nb2 = z.Rp;
     p.skip_dc = skip_dc != 0;
     float sa, g;
-    const bool ok = md_two_stage<false>(m, ns, tmem, p, sa, g);
+    const bool ok = md_two_stage<NT, false>(m, ns, tmem, p, sa, g);
     // x = D2 / (g 2^28 sa), through slot 0's A atom (free once the last MMAs are complete);
     // with strips (one CTA per channel) the channel's largest |x| is read from TMEM first
     // (inv is a power of two, so it is the largest stored |x| exactly) and sets their scale
     const float inv = 1.f / (g * MD_CSCALE * MD_CSCALE * sa);
     StripOut so{nullptr, nullptr, 0, 1, 0, 0, 1.f};
     if (sp.hi && ok) {                          // uniform
-        const float cm = md_tmem_max(tmem, z.Mp, z.Rp, m.red) * inv;
+        const float cm = md_tmem_max<NT>(tmem, z.Mp, z.Rp, m.red) * inv;
         so.hi = sp.hi + (size_t)f * z.D * sp.Ly + sp.off;
         so.lo = sp.lo + (size_t)f * z.D * sp.Ly + sp.off;
         so.Ly = sp.Ly;
@@ -575,7 +631,7 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
     }
     float xm = 0.f;
     if (ok)
-        xm = md_store_rows(tmem, z.Mp, z.Rp, 128 * dt, z.D, z.R, inv, x_all + (size_t)f * z.D * z.R, (size_t)z.R,
+        xm = md_store_rows<NT>(tmem, z.Mp, z.Rp, 128 * dt, z.D, z.R, inv, x_all + (size_t)f * z.D * z.R, (size_t)z.R,
                            reinterpret_cast<float *>(m.a(0)), so);
     if (xmax && !sp.hi) {                       // uniform: every thread takes part
         const float bm = block_max(xm, m.red);
@@ -588,8 +644,8 @@ k_modes_fwd(MdDims z, int ns, const float *__restrict__ a_all, int skip_dc, cons
 // CTA (f, m tile): stage 1 D1[m][d] = PhiT_tile xbar_f^T over r (A = PhiT tile image, B =
 // xbar_f rows d); stage 2 D2[m][n] = U LegT^T over d (A = scaled U from TMEM, B = LegT
 // image); abar = D2 / scales.
-template <bool WIN>
-__global__ void __launch_bounds__(MD_THREADS, 1)
+template <int NT, bool WIN>
+__global__ void __launch_bounds__(NT, 1)
 k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *__restrict__ phit_img,
             const uint8_t *__restrict__ legt_img, float *__restrict__ abar_all, int *__restrict__ status, int ncols,
             const __grid_constant__ MapWindows w)
@@ -617,10 +673,10 @@ k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *_
     p.nb2 = z.Np;
     p.skip_dc = false;
     float sx, g;
-    const bool ok = md_two_stage<WIN>(m, ns, tmem, p, sx, g);
+    const bool ok = md_two_stage<NT, WIN>(m, ns, tmem, p, sx, g);
     if (ok) {
         const float inv = 1.f / (g * MD_CSCALE * MD_CSCALE * sx);
-        md_store_rows(tmem, z.Dp, z.Np, 128 * mtile, z.M, z.N, inv, abar_all + (size_t)f * z.M * z.N, (size_t)z.N,
+        md_store_rows<NT>(tmem, z.Dp, z.Np, 128 * mtile, z.M, z.N, inv, abar_all + (size_t)f * z.M * z.N, (size_t)z.N,
                       reinterpret_cast<float *>(m.a(0)), StripOut{nullptr, nullptr, 0, 1, 0, 0, 1.f});
     }
     md_finish(m, ok, status, tmem, ncols);
@@ -649,6 +705,12 @@ int md_slots(int grid)
         if (sms <= 0) sms = 1;
     }
     return grid <= sms ? 2 : 1;
+}
+
+// the 512-thread kernels: two slots (one CTA an SM) and a source of rows_pad x k_pad that fits their registers
+bool md_wide(int ns, int rows_pad, int k_pad)
+{
+    return ns == 2 && rows_pad * 16 <= MD_RES_U * MD_WIDE && k_pad <= 64 * MD_RES_K;
 }
 
 int md_cols(int n)
@@ -696,9 +758,11 @@ fm_status modes_tc_setup(Ctx &c)
     }
     k_md_image<<<256, 256>>>(c.g.leg64, c.D, c.N, 1, 0, z.Np, z.Dp, MD_CSCALE, s.legt_img);
     FM_CK_LAUNCH();
-    FM_CK(smem_opt_in(k_modes_fwd));
-    FM_CK(smem_opt_in(k_modes_adj<false>));
-    FM_CK(smem_opt_in(k_modes_adj<true>));
+    FM_CK(smem_opt_in(k_modes_fwd<MD_THREADS>));
+    FM_CK(smem_opt_in(k_modes_fwd<MD_WIDE>));
+    FM_CK(smem_opt_in((k_modes_adj<MD_THREADS, false>)));
+    FM_CK(smem_opt_in((k_modes_adj<MD_WIDE, false>)));
+    FM_CK(smem_opt_in((k_modes_adj<MD_THREADS, true>)));
     FM_CK(cudaDeviceSynchronize());
     s.on = true;
     return FM_OK;
@@ -713,7 +777,9 @@ fm_status launch_modes_tc_forward(Ctx &c, const float *a, float *x, cudaStream_t
         set_error("sky strips need one CTA per channel and the channel maxima");
         return FM_ERR_STATE;
     }
-    k_modes_fwd<<<dim3(c.F, ndt), MD_THREADS, md_smem_bytes(z.Mp > z.Rp ? z.Mp : z.Rp, ns), st>>>(
+    const bool wide = md_wide(ns, z.Mp, z.Np);
+    auto *kern = wide ? k_modes_fwd<MD_WIDE> : k_modes_fwd<MD_THREADS>;
+    kern<<<dim3(c.F, ndt), wide ? MD_WIDE : MD_THREADS, md_smem_bytes(z.Mp > z.Rp ? z.Mp : z.Rp, ns), st>>>(
         z, ns, a, skip_dc, c.mtc.leg_img, c.mtc.phi_img, x, c.status, md_cols(z.Mp + z.Rp), xmax,
         strips ? *strips : StripArgs{});
     FM_CK_LAUNCH();
@@ -733,8 +799,9 @@ fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, flo
     MdDims z = md_dims(c);
     z.F = nmaps;
     const int nmt = (c.M + 127) / 128, ns = md_slots(nmaps * nmt);
-    auto *kern = w ? k_modes_adj<true> : k_modes_adj<false>;
-    kern<<<dim3(nmaps, nmt), MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
+    const bool wide = !w && md_wide(ns, z.Dp, z.Rp);
+    auto *kern = w ? k_modes_adj<MD_THREADS, true> : wide ? k_modes_adj<MD_WIDE, false> : k_modes_adj<MD_THREADS, false>;
+    kern<<<dim3(nmaps, nmt), wide ? MD_WIDE : MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
         z, ns, xbar, c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np), w ? *w : MapWindows{});
     FM_CK_LAUNCH();
     return FM_OK;
