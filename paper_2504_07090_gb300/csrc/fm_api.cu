@@ -356,21 +356,26 @@ fm_status vis_of_modes(Ctx &c, const R *a, R *xbuf, R *vis, cudaStream_t st, boo
 }
 
 template <typename R>
-fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st)
+fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st, bool partials_only)
 {
     if constexpr (std::is_same<R, float>::value)
         if (c.ha.on && c.ha.dual) {
             HaSky ka, kb;
             FM_TRY(sky_of_modes(c, a, xa, va, 0, st, ka));
             FM_TRY(sky_of_modes(c, b, xb, vb, 1, st, kb));
-            return launch_vis_ha_dual(c, ka, kb);
+            return launch_vis_ha_dual(c, ka, kb, partials_only);
         }
+    if (partials_only) {
+        set_error("unfinished visibilities of two skies exist only in the two-sky forward");
+        return FM_ERR_STATE;
+    }
     FM_TRY(vis_of_modes<R>(c, a, xa, va, st));
     return vis_of_modes<R>(c, b, xb, vb, st);
 }
-template fm_status vis_of_two<float>(Ctx &, const float *, float *, float *, const float *, float *, float *, cudaStream_t);
+template fm_status vis_of_two<float>(Ctx &, const float *, float *, float *, const float *, float *, float *, cudaStream_t,
+                                     bool);
 template fm_status vis_of_two<double>(Ctx &, const double *, double *, double *, const double *, double *, double *,
-                                      cudaStream_t);
+                                      cudaStream_t, bool);
 template fm_status vis_of_modes<float>(Ctx &, const float *, float *, float *, cudaStream_t, bool);
 template fm_status vis_of_modes<double>(Ctx &, const double *, double *, double *, cudaStream_t, bool);
 
@@ -420,8 +425,6 @@ static fm_status run_hvp(Ctx &c, const R *theta, const R *v, R *hv, int full, cu
     if (!c.have_data) { set_error("fm_set_data has not been called"); return FM_ERR_STATE; }
     if (c.df_on) { set_error("Hessian-vector products with the delay filter are not implemented"); return FM_ERR_UNSUPPORTED; }
     R *x = (R *)c.x, *xv = (R *)c.xv;
-    FM_TRY(launch_gains<R>(c, theta + c.n_sky, (R *)c.gains, st));
-    FM_TRY(launch_gains<R>(c, v + c.n_sky, (R *)c.dgains, st));
     const R *sky = theta, *vsky = v;
     if (c.K > 0) {
         FM_TRY(launch_freq_expand<R>(c, theta, (R *)c.ax, st));
@@ -429,13 +432,28 @@ static fm_status run_hvp(Ctx &c, const R *theta, const R *v, R *hv, int full, cu
         sky = (const R *)c.ax;
         vsky = (const R *)c.avx;
     }
-    FM_TRY(vis_of_two<R>(c, sky, x, (R *)c.vis, vsky, xv, (R *)c.dvis, st));
-    FM_TRY(launch_hvp_mid<R>(c, (R *)c.vis, (R *)c.dvis, (R *)c.gains, (R *)c.dgains, full, (R *)c.omega,
-                             (R *)c.zpart, st));
-    FM_TRY(run_adjoint<R>(c, (R *)c.omega, (R *)c.xbar, st));
+    // hour-angle form with the two-sky forward: one epilogue from the partial sums (as the gradient's)
+    bool fused = false;
+    if constexpr (std::is_same<R, float>::value) {
+        HaVSrc sv, sd;
+        fused = ha_vsrc_dual(c, c.dc_split ? sky : nullptr, c.nk, 0, sv) &&
+                ha_vsrc_dual(c, c.dc_split ? vsky : nullptr, c.nk, 1, sd) && launch_hvp_ft_fits(c);
+        if (fused) {
+            FM_TRY(vis_of_two<R>(c, sky, x, nullptr, vsky, xv, nullptr, st, true));
+            FM_TRY(launch_hvp_ft(c, theta + c.n_sky, v + c.n_sky, full, (R *)c.zpart, sv, sd, st));
+        }
+    }
+    if (!fused) {
+        FM_TRY(launch_gains<R>(c, theta + c.n_sky, (R *)c.gains, st));
+        FM_TRY(launch_gains<R>(c, v + c.n_sky, (R *)c.dgains, st));
+        FM_TRY(vis_of_two<R>(c, sky, x, (R *)c.vis, vsky, xv, (R *)c.dvis, st));
+        FM_TRY(launch_hvp_mid<R>(c, (R *)c.vis, (R *)c.dvis, (R *)c.gains, (R *)c.dgains, full, (R *)c.omega,
+                                 (R *)c.zpart, st));
+    }
+    FM_TRY(run_adjoint<R>(c, (R *)c.omega, (R *)c.xbar, st, fused));
     FM_TRY(launch_modes_adjoint<R>(c, (R *)c.xbar, c.K > 0 ? (R *)c.gx : hv, st));
     if (c.K > 0) FM_TRY(launch_freq_contract<R>(c, (const R *)c.gx, hv, st));
-    FM_TRY(launch_gain_reduce<R>(c, (R *)c.zpart, hv + c.n_sky, st));
+    FM_TRY(launch_gain_reduce_chan<R>(c, (R *)c.zpart, hv + c.n_sky, st));
     return launch_prior_hvp<R>(c, v, hv, st);
 }
 
@@ -529,6 +547,12 @@ fm_status fm_forward(fm_handle h, const void *dev_theta, void *dev_vis_out, fm_s
     if (c.K > 0) {
         FM_TRY(launch_freq_expand<float>(c, th, (float *)c.ax, stream));
         sky = (const float *)c.ax;
+    }
+    if (c.ha.on) {                          // the gains are applied where V is finished
+        HaSky k;
+        FM_TRY(sky_of_modes(c, sky, (float *)c.x, (float *)dev_vis_out, 0, stream, k));
+        k.gamma = th + c.n_sky;
+        return launch_vis_ha(c, k);
     }
     FM_TRY(launch_gains<float>(c, th + c.n_sky, (float *)c.gains, stream));
     FM_TRY(vis_of_modes<float>(c, sky, (float *)c.x, (float *)c.vis, stream));

@@ -403,9 +403,6 @@ fm_status launch_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st);  // 
 template <typename R>
 fm_status launch_apply_gains(Ctx &c, const R *vis, const R *g, R *out, cudaStream_t st);
 template <typename R>
-fm_status launch_chi2_mid(Ctx &c, const R *vis, const R *g, R *omega, R *zpart, double *chi2p,
-                          cudaStream_t st);
-template <typename R>
 fm_status launch_hvp_mid(Ctx &c, const R *vis, const R *dvis, const R *g, const R *dg, int full, R *omega,
                          R *zpart, cudaStream_t st);
 template <typename R>
@@ -432,6 +429,13 @@ struct HaVSrc {
 // fills v when the epilogue can form V from the partials (hour-angle form on, one LST pass,
 // the groups' monopole visibilities present when dc != nullptr)
 bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v);
+// the same for sky `slot` of the two-sky forward
+bool ha_vsrc_dual(const Ctx &c, const float *dc, long long dcs, int slot, HaVSrc &v);
+// the Hessian-vector product's epilogue from the two-sky forward's partial sums (group sums of the
+// weights formed inside)
+bool launch_hvp_ft_fits(const Ctx &c);
+fm_status launch_hvp_ft(Ctx &c, const float *gamma, const float *dgamma, int full, float *zpart, const HaVSrc &hv,
+                        const HaVSrc &hd, cudaStream_t st);
 
 template <typename R>
 fm_status launch_chi2_chan(Ctx &c, const R *vis, const R *gamma, R *omega, R *zpart, double *chi2p, bool groups,
@@ -457,7 +461,8 @@ template <typename R>
 fm_status vis_of_modes(Ctx &c, const R *a, R *xbuf, R *vis, cudaStream_t st, bool partials_only = false);
 // the same for two skies a and b (into xa, va and xb, vb), in one forward pass where the handle has it
 template <typename R>
-fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st);
+fm_status vis_of_two(Ctx &c, const R *a, R *xa, R *va, const R *b, R *xb, R *vb, cudaStream_t st,
+                     bool partials_only = false);
 
 // tensor-core contraction (sm_103a tcgen05); returns FM_ERR_UNSUPPORTED when the
 // shape does not fit its tiles
@@ -524,13 +529,14 @@ struct HaSky {
     const float *dc = nullptr;
     long long dcs = 0;
     int slot = 0;
+    const float *gamma = nullptr;    // gain coefficients [A][NG][2]: vis = g_p conj(g_q) V instead of V
     bool xmax_ready = false, strips_ready = false;
 };
 // partials_only: V is not finished (the forward's partial sums stay in c.ha.vpart for the chi^2
 // epilogue, HaVSrc)
 fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only = false);
 // two skies (slots 0 and 1) in one pass over the responses; needs c.ha.dual
-fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b);
+fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b, bool partials_only = false);
 // q_ready: the group sums q32 / qmax_ft were already formed from omega (by the chi^2 epilogue)
 fm_status launch_adjoint_ha(Ctx &c, const float *omega, float *xbar, cudaStream_t st, bool q_ready = false);
 

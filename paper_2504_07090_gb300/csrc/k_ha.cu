@@ -734,19 +734,31 @@ done:
 // CTA (segment, LST block of HA_VF_T): the contributors' partials of the segment's 128
 // rows are added into shared memory, then every baseline of the segment's groups gets
 // its (possibly conjugated) value, written coalesced over baselines.  With dc != nullptr
-// the monopole term c_f U[f][t][b] (c_f = dc[f * dcs]) is added in the same write.
+// the monopole term c_f U[f][t][b] (c_f = dc[f * dcs]) is added in the same write, and with gamma !=
+// nullptr the gains are applied.
 constexpr int HA_VF_T = 8;
 
 __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float *__restrict__ vpart,
                                                     const int *__restrict__ ncontrib, const int *__restrict__ bmap,
                                                     const unsigned *__restrict__ xmax, float sp,
                                                     const float *__restrict__ dc, long long dcs,
-                                                    const float *__restrict__ U, float *__restrict__ vis)
+                                                    const float *__restrict__ U, DevGeom g,
+                                                    const float *__restrict__ gamma, float *__restrict__ vis)
 {
     __shared__ float sv[128][HA_VF_T];
+    extern __shared__ float2 sg[];                  // [A] gains of the channel, when gamma is given
     const int seg = blockIdx.x, mt = seg / h.F, f = seg % h.F;
     const int t0 = blockIdx.y * HA_VF_T, tn = min(HA_VF_T, h.T - t0);
     const int nc = ncontrib[seg];
+    if (gamma)                                      // as k_gains
+        for (int i = threadIdx.x; i < g.A; i += blockDim.x) {
+            float re = 0.f, im = 0.f;
+            for (int k = 0; k < g.NG; ++k) {
+                re += g.gleg32[f * g.NG + k] * gamma[(i * g.NG + k) * 2];
+                im += g.gleg32[f * g.NG + k] * gamma[(i * g.NG + k) * 2 + 1];
+            }
+            sg[i] = make_float2(re, im);
+        }
     for (int e = threadIdx.x; e < 128 * HA_VF_T; e += blockDim.x) {
         const int row = e % 128, tl = e / 128;
         float a = 0.f;
@@ -772,6 +784,11 @@ __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float 
         if ((u >> 6) != mt) continue;
         const int row = 2 * (u & 63);
         const float sgn = (code & 1) ? -1.f : 1.f;
+        float2 gg = make_float2(1.f, 0.f);          // g_i conj(g_j)
+        if (gamma) {
+            const float2 gi = sg[g.bl_i[b]], gj = sg[g.bl_j[b]];
+            gg = make_float2(gi.x * gj.x + gi.y * gj.y, gi.y * gj.x - gi.x * gj.y);
+        }
         for (int tl = 0; tl < tn; ++tl) {
             const size_t e = ((size_t)f * h.Tt + h.t0 + t0 + tl) * B + b;
             // explicit roundings: the chi^2 epilogue forms the same values (HaVSrc)
@@ -781,6 +798,7 @@ __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float 
                 v.x = __fmaf_rn(cf, u2.x, v.x);
                 v.y = __fmaf_rn(cf, u2.y, v.y);
             }
+            if (gamma) v = make_float2(gg.x * v.x - gg.y * v.y, gg.x * v.y + gg.y * v.x);
             reinterpret_cast<float2 *>(vis)[e] = v;
         }
     }
@@ -1344,9 +1362,9 @@ fm_status fwd_pass(Ctx &c, const HaDev &h, const HaLayout &L, cudaStream_t st)
 fm_status fwd_finish(Ctx &c, const HaDev &h, const HaSky &k)
 {
     const HaState &s = c.ha;
-    k_ha_vfinish<<<dim3(s.nmt * c.F, cdiv(h.T, HA_VF_T)), 256, 0, k.st>>>(
+    k_ha_vfinish<<<dim3(s.nmt * c.F, cdiv(h.T, HA_VF_T)), 256, k.gamma ? sizeof(float2) * c.A : 0, k.st>>>(
         h, c.B, s.vpart + (size_t)(h.dual ? k.slot : 0) * s.npad * 128, s.ncontrib, s.bmap,
-        s.xmax + (size_t)k.slot * c.F, s.sp, k.dc, k.dcs, c.dc_u, k.vis);
+        s.xmax + (size_t)k.slot * c.F, s.sp, k.dc, k.dcs, c.dc_u, c.g, k.gamma, k.vis);
     FM_CK_LAUNCH();
     return FM_OK;
 }
@@ -1380,7 +1398,7 @@ fm_status vis_ha_launch(Ctx &c, const HaDev &h, const HaSky &k, bool partials_on
 
 // two skies in one pass (s.dual)
 template <int ET, bool X3>
-fm_status vis_ha_dual_launch(Ctx &c, const HaDev &h, const HaSky &a, const HaSky &b)
+fm_status vis_ha_dual_launch(Ctx &c, const HaDev &h, const HaSky &a, const HaSky &b, bool partials_only)
 {
     HaState &s = c.ha;
     HaLayout L;
@@ -1394,6 +1412,7 @@ fm_status vis_ha_dual_launch(Ctx &c, const HaDev &h, const HaSky &a, const HaSky
     hc.N = 2 * s.npad;
     hc.dual = 1;
     FM_TRY((fwd_pass<ET, X3, true>(c, hc, L, a.st)));
+    if (partials_only) return FM_OK;
     FM_TRY(fwd_finish(c, hc, a));
     return fwd_finish(c, hc, b);
 }
@@ -1688,12 +1707,12 @@ fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only)
     return x3 ? vis_ha_launch<0, true>(c, h, k, po) : vis_ha_launch<0, false>(c, h, k, po);
 }
 
-fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b)
+fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b, bool po)
 {
     const HaDev h = make_dev(c);
     const bool x3 = x3_of(c.prec);
-    if (f16_of(c.prec)) return x3 ? vis_ha_dual_launch<1, true>(c, h, a, b) : vis_ha_dual_launch<1, false>(c, h, a, b);
-    return x3 ? vis_ha_dual_launch<0, true>(c, h, a, b) : vis_ha_dual_launch<0, false>(c, h, a, b);
+    if (f16_of(c.prec)) return x3 ? vis_ha_dual_launch<1, true>(c, h, a, b, po) : vis_ha_dual_launch<1, false>(c, h, a, b, po);
+    return x3 ? vis_ha_dual_launch<0, true>(c, h, a, b, po) : vis_ha_dual_launch<0, false>(c, h, a, b, po);
 }
 
 bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
@@ -1714,6 +1733,16 @@ bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
     v.npad = s.npf;
     v.nmt = s.nmt;
     v.F = c.F;
+    return true;
+}
+
+bool ha_vsrc_dual(const Ctx &c, const float *dc, long long dcs, int slot, HaVSrc &v)
+{
+    const HaState &s = c.ha;
+    if (!s.dual || !ha_vsrc(c, dc, dcs, v)) return false;
+    v.npad = 2 * s.npad;
+    v.vpart = s.vpart + (size_t)slot * s.npad * 128;
+    v.xmax = s.xmax + (size_t)slot * c.F;
     return true;
 }
 

@@ -7,6 +7,7 @@
 //   - gains, residual, chi^2 partials in FP64 and the adjoint weights (Eq. likelihood);
 //   - the pixel adjoint xbar_p = dOmega A sum_{p<q} Re[conj(omega_pq) K_pq];
 //   - deterministic reductions (fixed order, no floating-point atomics).
+#include <algorithm>
 #include <type_traits>
 
 #include "fm_internal.cuh"
@@ -412,67 +413,124 @@ __device__ void block_sum_double(double v, double *out, double *sred)
     if (threadIdx.x == 0) *out = sred[0];
 }
 
-// One CTA per (channel, LST): model, residual, chi^2 partial (FP64), the adjoint
-// weights omega_pq = conj(g_p) g_q r_pq / sigma^2 and the per-antenna gain-gradient
-// partials Z_a (gradient w.r.t. gamma_ak is X_k(nu) (Re Z_a, Im Z_a)).
-template <typename R>
-__global__ void __launch_bounds__(256) k_chi2_mid(DevGeom g, const R *__restrict__ vis, const R *__restrict__ data,
-                                                  const R *__restrict__ gains, R *__restrict__ omega,
-                                                  R *__restrict__ zpart, double *__restrict__ chi2p)
+// ---- pieces of the per-(channel, LST) epilogues k_chi2_ft and k_hvp_ft
+
+// sS[row], row < 128 nmt: the contributors' partial rows of the forward at LST t of channel f, in rank
+// order; sc and cf: the scale of the sum and the monopole's coefficient
+template <int NT>
+__device__ __forceinline__ void hv_rows(const HaVSrc &hv, int f, int t, float *sS, float &sc, float &cf)
 {
-    using C2 = typename V2<R>::t;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *sred = reinterpret_cast<double *>(smem_raw);            // [256]
-    C2 *sG = reinterpret_cast<C2 *>(sred + 256);                      // [A]
-    C2 *sV = sG + g.A;                                                // [B]
-    C2 *sRr = sV + g.B;                                               // [B]
-    const int ft = blockIdx.x, f = ft / g.T;
-    for (int i = threadIdx.x; i < g.A; i += blockDim.x) {
-        sG[i].x = gains[2 * (f * g.A + i)];
-        sG[i].y = gains[2 * (f * g.A + i) + 1];
+    for (int e = threadIdx.x; e < hv.nmt * 128; e += NT) {
+        const int seg = (e >> 7) * hv.F + f, row = e & 127, nc = hv.ncontrib[seg];
+        // the contributors' rows in rank order, four loads ahead
+        const float *src = hv.vpart + ((size_t)seg * hv.J * hv.npad + t) * 128 + row;
+        const size_t js = (size_t)hv.npad * 128;
+        float a = 0.f;
+        for (int j0 = 0; j0 < nc; j0 += 4) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = j0 + u < nc ? src[(size_t)(j0 + u) * js] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (j0 + u < nc) a += v[u];
+        }
+        sS[e] = a;
     }
-    __syncthreads();
-    const R is2 = (R)g.inv_sigma2;
-    double c2 = 0.0;
-    for (int b = threadIdx.x; b < g.B; b += blockDim.x) {
-        int i = g.bl_i[b], j = g.bl_j[b];
-        size_t o = ((size_t)ft * g.B + b) * 2;
-        C2 V, gi = sG[i], gj = sG[j];
-        V.x = vis[o]; V.y = vis[o + 1];
-        R ggr = gi.x * gj.x + gi.y * gj.y, ggi = gi.y * gj.x - gi.x * gj.y;     // g_i conj(g_j)
-        R rr = ggr * V.x - ggi * V.y - data[o];
-        R ri = ggr * V.y + ggi * V.x - data[o + 1];
-        c2 += (double)rr * (double)rr + (double)ri * (double)ri;
-        // omega = conj(g_i) g_j r / sigma^2 = conj(g_i conj(g_j)) r / sigma^2
-        omega[o] = (ggr * rr + ggi * ri) * is2;
-        omega[o + 1] = (ggr * ri - ggi * rr) * is2;
-        sV[b] = V;
-        sRr[b].x = rr; sRr[b].y = ri;
+    const float mx = __uint_as_float(hv.xmax[f]);
+    float s2 = 1.f;
+    if (mx > 0.f && isfinite(mx)) {
+        int ex;
+        frexpf(mx, &ex);
+        s2 = ldexpf(1.f, 14 - ex);
     }
-    block_sum_double<R>(c2, chi2p + ft, sred);
-    if (threadIdx.x == 0) chi2p[ft] *= g.inv_sigma2;
-    __syncthreads();
-    for (int a = threadIdx.x; a < g.A; a += blockDim.x) {
-        R zr = 0, zi = 0;
-        for (int j = 0; j < g.A; ++j) {
-            if (j == a) continue;
-            if (j > a) {   // pair (a, j): t = conj(r) conj(g_j) V; Z += conj(t)
-                int b = pair_index(a, j, g.A);
-                C2 r = sRr[b], V = sV[b], gj = sG[j];
-                R cr = r.x * gj.x - r.y * gj.y, ci = -(r.x * gj.y + r.y * gj.x);   // conj(r) conj(g_j)
-                R tr = cr * V.x - ci * V.y, ti = cr * V.y + ci * V.x;
-                zr += tr; zi -= ti;
-            } else {       // pair (j, a): t = conj(r) g_j V; Z += t
-                int b = pair_index(j, a, g.A);
-                C2 r = sRr[b], V = sV[b], gj = sG[j];
-                R cr = r.x * gj.x + r.y * gj.y, ci = r.x * gj.y - r.y * gj.x;      // conj(r) g_j
-                zr += cr * V.x - ci * V.y;
-                zi += cr * V.y + ci * V.x;
+    sc = 1.f / (hv.sp * s2);
+    cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
+}
+
+// V of a baseline with code = 2 u + reversed, with the roundings of k_ha_vfinish, so that it equals the
+// finished forward's bitwise
+__device__ __forceinline__ float2 hv_value(const HaVSrc &hv, const float *sS, size_t ft, int U, int code, float sc,
+                                           float cf)
+{
+    const int u = code >> 1, row = 128 * (u >> 6) + 2 * (u & 63);
+    const float sgn = (code & 1) ? -1.f : 1.f;
+    float vx = __fmul_rn(sS[row], sc), vy = __fmul_rn(sgn * sS[row + 1], sc);
+    if (hv.dc) {
+        const float2 u2 = reinterpret_cast<const float2 *>(hv.ug)[ft * U + u];
+        vx = __fmaf_rn(cf, u2.x, vx);
+        vy = __fmaf_rn(cf, sgn * u2.y, vy);
+    }
+    return make_float2(vx, vy);
+}
+
+// q32[ft][u] = the groups' sums of sW (conjugated for reversed members); returns the largest |Re|, |Im| that
+// this thread stored.  Four lanes a group, each every fourth member, added in a fixed order: one lane a
+// group left three quarters of the threads idle over up to 126 members.
+template <int NT, typename C2>
+__device__ __forceinline__ float group_sums(const C2 *sW, int ft, int U, const int *__restrict__ moff,
+                                            const int *__restrict__ mem, float *__restrict__ q32)
+{
+    const int tid = threadIdx.x;
+    float qm = 0.f;
+    for (int u0 = 0; u0 < U; u0 += NT / 4) {
+        const int u = u0 + (tid >> 2);
+        float qr = 0.f, qi = 0.f;
+        if (u < U) {
+            const int m1 = moff[u + 1];
+#pragma unroll 2
+            for (int m = moff[u] + (tid & 3); m < m1; m += 4) {
+                const int code = mem[m], b = code >> 1;
+                qr += (float)sW[b].x;
+                qi += (code & 1) ? -(float)sW[b].y : (float)sW[b].y;
             }
         }
-        zpart[((size_t)ft * g.A + a) * 2] = zr * is2;
-        zpart[((size_t)ft * g.A + a) * 2 + 1] = zi * is2;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            qr += __shfl_xor_sync(0xffffffffu, qr, o);
+            qi += __shfl_xor_sync(0xffffffffu, qi, o);
+        }
+        if (u < U && (tid & 3) == 0) {
+            *reinterpret_cast<float2 *>(q32 + ((size_t)ft * U + u) * 2) = make_float2(qr, qi);
+            qm = fmaxf(qm, fmaxf(fabsf(qr), fabsf(qi)));
+        }
     }
+    return qm;
+}
+
+// sZ[tid]: chunk c = tid mod nc, nc = NT / A, of Z_a, a = tid div nc: partners j = c, c + nc, ... (j != a);
+// pair_index(a, j) = rowa + j for j > a
+template <int NT, typename C2>
+__device__ __forceinline__ void antenna_chunks(const C2 *sTi, const C2 *sTj, int A, C2 *sZ)
+{
+    using R = decltype(C2::x);
+    const int tid = threadIdx.x, nc = NT / A;
+    if (tid >= nc * A) return;
+    const int a = tid / nc, c = tid - a * nc;
+    const int rowa = a * A - (a * (a + 1)) / 2 - a - 1;
+    R zr = 0, zi = 0;
+    for (int j = c; j < A; j += nc) {
+        if (j == a) continue;
+        const C2 t = j > a ? sTi[rowa + j] : sTj[pair_index(j, a, A)];
+        zr += t.x;
+        zi += t.y;
+    }
+    sZ[tid].x = zr;
+    sZ[tid].y = zi;
+}
+
+// after a barrier: zpart[ft][a] = the chunks of Z_a in order, over sigma^2
+template <int NT, typename R, typename C2>
+__device__ __forceinline__ void antenna_totals(const C2 *sZ, int A, int ft, R is2, R *__restrict__ zpart)
+{
+    const int tid = threadIdx.x, nc = NT / A;
+    if (tid >= A) return;
+    R zr = 0, zi = 0;
+    for (int c = 0; c < nc; ++c) {
+        zr += sZ[tid * nc + c].x;
+        zi += sZ[tid * nc + c].y;
+    }
+    zpart[((size_t)ft * A + tid) * 2] = zr * is2;
+    zpart[((size_t)ft * A + tid) * 2 + 1] = zi * is2;
 }
 
 // One CTA per (channel, LST): model, residual, chi^2 partial (a warp's terms summed in the
@@ -524,34 +582,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1
         }
     }
     float hsc = 0.f, hcf = 0.f;
-    if (hv.vpart) {     // the partial rows of every M-tile at this LST, summed in rank order
-        const int t = ft - f * g.T;
-        for (int e = tid; e < hv.nmt * 128; e += NT) {
-            const int seg = (e >> 7) * hv.F + f, row = e & 127, nc = hv.ncontrib[seg];
-            // the contributors' rows in rank order, four loads ahead
-            const float *src = hv.vpart + ((size_t)seg * hv.J * hv.npad + t) * 128 + row;
-            const size_t js = (size_t)hv.npad * 128;
-            float a = 0.f;
-            for (int j0 = 0; j0 < nc; j0 += 4) {
-                float v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = j0 + u < nc ? src[(size_t)(j0 + u) * js] : 0.f;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (j0 + u < nc) a += v[u];
-            }
-            sS[e] = a;
-        }
-        const float mx = __uint_as_float(hv.xmax[f]);
-        float s2 = 1.f;
-        if (mx > 0.f && isfinite(mx)) {
-            int ex;
-            frexpf(mx, &ex);
-            s2 = ldexpf(1.f, 14 - ex);
-        }
-        hsc = 1.f / (hv.sp * s2);
-        hcf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
-    }
+    if (hv.vpart) hv_rows<NT>(hv, f, ft - f * g.T, sS, hsc, hcf);
     __syncthreads();
     const R is2 = (R)g.inv_sigma2;
     const C2 *vrow = vis ? reinterpret_cast<const C2 *>(vis) + (size_t)ft * g.B : nullptr;
@@ -564,17 +595,9 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1
         const int i = g.bl_i[b], j = g.bl_j[b];
         C2 V;
         if (hv.vpart) {
-            const int code = hv.bmap[b], u = code >> 1, row = 128 * (u >> 6) + 2 * (u & 63);
-            const float sgn = (code & 1) ? -1.f : 1.f;
-            // the roundings of k_ha_vfinish, so that V equals the finished forward's bitwise
-            float vx = __fmul_rn(sS[row], hsc), vy = __fmul_rn(sgn * sS[row + 1], hsc);
-            if (hv.dc) {
-                const float2 u2 = reinterpret_cast<const float2 *>(hv.ug)[(size_t)ft * U + u];
-                vx = __fmaf_rn(hcf, u2.x, vx);
-                vy = __fmaf_rn(hcf, sgn * u2.y, vy);
-            }
-            V.x = (R)vx;
-            V.y = (R)vy;
+            const float2 v = hv_value(hv, sS, (size_t)ft, U, hv.bmap[b], hsc, hcf);
+            V.x = (R)v.x;
+            V.y = (R)v.y;
         } else {
             V = vrow[b];
         }
@@ -615,65 +638,19 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1
         chi2p[ft] = a * g.inv_sigma2;
     }
     if (q32) {
-        // four lanes a group, each every fourth member, added in a fixed order: one lane a group left three
-        // quarters of the threads idle over up to 126 members
-        float qm = 0.f;
-        for (int u0 = 0; u0 < U; u0 += NT / 4) {
-            const int u = u0 + (tid >> 2);
-            float qr = 0.f, qi = 0.f;
-            if (u < U) {
-                const int m1 = moff[u + 1];
-#pragma unroll 2
-                for (int m = moff[u] + (tid & 3); m < m1; m += 4) {
-                    const int code = mem[m], b = code >> 1;
-                    qr += (float)sW[b].x;
-                    qi += (code & 1) ? -(float)sW[b].y : (float)sW[b].y;
-                }
-            }
-#pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
-                qr += __shfl_xor_sync(0xffffffffu, qr, o);
-                qi += __shfl_xor_sync(0xffffffffu, qi, o);
-            }
-            if (u < U && (tid & 3) == 0) {
-                *reinterpret_cast<float2 *>(q32 + ((size_t)ft * U + u) * 2) = make_float2(qr, qi);
-                qm = fmaxf(qm, fmaxf(fabsf(qr), fabsf(qi)));
-            }
-        }
+        float qm = group_sums<NT>(sW, ft, U, moff, mem, q32);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) qm = fmaxf(qm, __shfl_xor_sync(0xffffffffu, qm, o));
         if (lane == 0) fred[w] = qm;
     }
-    // Z_a, chunk c: partners j = c, c + nc, ... (j != a); pair_index(a, j) = rowa + j for j > a
-    const int nc = NT / g.A;
-    if (tid < nc * g.A) {
-        const int a = tid / nc, c = tid - a * nc;
-        const int rowa = a * g.A - (a * (a + 1)) / 2 - a - 1;
-        R zr = 0, zi = 0;
-        for (int j = c; j < g.A; j += nc) {
-            if (j == a) continue;
-            const C2 t = j > a ? sTi[rowa + j] : sTj[pair_index(j, a, g.A)];
-            zr += t.x;
-            zi += t.y;
-        }
-        sZ[tid].x = zr;
-        sZ[tid].y = zi;
-    }
+    antenna_chunks<NT>(sTi, sTj, g.A, sZ);
     __syncthreads();
     if (q32 && tid == 0) {
         float m = 0.f;
         for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, fred[k]);
         qmax_ft[ft] = m;
     }
-    if (tid < g.A) {
-        R zr = 0, zi = 0;
-        for (int c = 0; c < nc; ++c) {
-            zr += sZ[tid * nc + c].x;
-            zi += sZ[tid * nc + c].y;
-        }
-        zpart[((size_t)ft * g.A + tid) * 2] = zr * is2;
-        zpart[((size_t)ft * g.A + tid) * 2 + 1] = zi * is2;
-    }
+    antenna_totals<NT>(sZ, g.A, ft, is2, zpart);
 }
 
 // grad_gamma[a][k][c] = sum_{f,t} X_k(nu_f) zpart[f][t][a][c]: one CTA per (a, c); thread
@@ -689,16 +666,17 @@ __global__ void __launch_bounds__(GR_THREADS) k_gain_reduce_ft(DevGeom g, const 
     __shared__ double red[GR_THREADS / 32][GR_NGMAX];
     const int a = blockIdx.x >> 1, c = blockIdx.x & 1, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const R *gl = Tab<R>::gleg(g);
+    const int nthr = blockDim.x;
     R acc[GR_NGMAX];
 #pragma unroll
     for (int k = 0; k < GR_NGMAX; ++k) acc[k] = 0;
     const int nft = g.F * g.T;
-    for (int base = 0; base < nft; base += GR_THREADS * GR_U) {
+    for (int base = 0; base < nft; base += nthr * GR_U) {
         R z[GR_U];
         int f[GR_U];
 #pragma unroll
         for (int u = 0; u < GR_U; ++u) {
-            const int ft = base + u * GR_THREADS + (int)threadIdx.x;
+            const int ft = base + u * nthr + (int)threadIdx.x;
             z[u] = ft < nft ? zpart[((size_t)ft * g.A + a) * 2 + c] : (R)0;
             f[u] = ft < nft ? ft / g.T : 0;
         }
@@ -710,6 +688,7 @@ __global__ void __launch_bounds__(GR_THREADS) k_gain_reduce_ft(DevGeom g, const 
     }
 #pragma unroll
     for (int k = 0; k < GR_NGMAX; ++k) {
+        if (k >= g.NG) break;
         R v = acc[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -718,7 +697,7 @@ __global__ void __launch_bounds__(GR_THREADS) k_gain_reduce_ft(DevGeom g, const 
     __syncthreads();
     if (threadIdx.x < g.NG) {
         double t = 0.0;
-        for (int k = 0; k < GR_THREADS / 32; ++k) t += red[k][threadIdx.x];
+        for (int k = 0; k < nthr / 32; ++k) t += red[k][threadIdx.x];
         out[(a * g.NG + threadIdx.x) * 2 + c] = (R)t;
     }
 }
@@ -750,18 +729,9 @@ template <typename R>
 fm_status launch_gain_reduce_chan(Ctx &c, const R *zpart, R *grad_gain, cudaStream_t st)
 {
     if (c.NG > GR_NGMAX) return launch_gain_reduce<R>(c, zpart, grad_gain, st);
-    k_gain_reduce_ft<R><<<2 * c.A, GR_THREADS, 0, st>>>(c.g, zpart, grad_gain);
-    FM_CK_LAUNCH();
-    return FM_OK;
-}
-
-template <typename R>
-fm_status launch_chi2_mid(Ctx &c, const R *vis, const R *g, R *omega, R *zpart, double *chi2p, cudaStream_t st)
-{
-    size_t smem = 256 * sizeof(double) + (c.A + 2 * (size_t)c.B) * 2 * sizeof(R);
-    if (smem > 227 * 1024) return FM_ERR_UNSUPPORTED;
-    FM_CK(smem_opt_in(k_chi2_mid<R>));
-    k_chi2_mid<R><<<c.F * c.T, 256, smem, st>>>(c.g, vis, (const R *)c.data, g, omega, zpart, chi2p);
+    // no more warps than there are terms: their FP64 shuffles alone took 20 us
+    const int nthr = std::min(GR_THREADS, (c.F * c.T + 31) / 32 * 32);
+    k_gain_reduce_ft<R><<<2 * c.A, nthr, 0, st>>>(c.g, zpart, grad_gain);
     FM_CK_LAUNCH();
     return FM_OK;
 }
@@ -833,6 +803,99 @@ __global__ void __launch_bounds__(256) k_hvp_mid(DevGeom g, const R *__restrict_
         zpart[((size_t)ft * g.A + a) * 2] = z.x * is2;
         zpart[((size_t)ft * g.A + a) * 2 + 1] = z.y * is2;
     }
+}
+
+// The same in one pass for the hour-angle form after its two-sky forward: V and dV are formed from the
+// partial sums (hv, hd), the gains and their tangents from the coefficients, the omega' sums over the
+// baseline groups go to q32 / qmax_ft, and the gain partials are k_chi2_ft's (a warp's or chunk's terms in
+// order).  37 antennas, 64 channels, 60 LSTs: the separate finishing of V and dV, the gains, k_hvp_mid and
+// the group sums took 91 us.  Bound: the latency of a CTA's chain of phases, as k_chi2_ft.
+template <bool FULL>
+__global__ void __launch_bounds__(CF_THREADS, 6) k_hvp_ft(DevGeom g, const float *__restrict__ data,
+                                                          const float *__restrict__ gamma,
+                                                          const float *__restrict__ dgamma, float *__restrict__ zpart,
+                                                          int U, const int *__restrict__ moff,
+                                                          const int *__restrict__ mem, float *__restrict__ q32,
+                                                          float *__restrict__ qmax_ft, HaVSrc hv, HaVSrc hd)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *sG = reinterpret_cast<float2 *>(smem_raw), *sD = sG + g.A;       // [A] gains and tangents
+    float2 *sTi = sD + g.A, *sTj = sTi + g.B, *sW = sTj + g.B;               // [B]
+    float *sS = reinterpret_cast<float *>(sW + g.B), *sS2 = sS + 128 * hv.nmt;
+    __shared__ float2 sZ[CF_THREADS];
+    __shared__ float fred[CF_THREADS / 32];
+    const int ft = blockIdx.x, f = ft / g.T, tid = threadIdx.x, lane = tid & 31;
+    const float *X = g.gleg32 + (size_t)f * g.NG;
+    for (int i = tid; i < 2 * g.A; i += CF_THREADS) {                        // as k_gains
+        const float *c = (i < g.A ? gamma : dgamma) + 2 * (size_t)(i < g.A ? i : i - g.A) * g.NG;
+        float re = 0, im = 0;
+        for (int k = 0; k < g.NG; ++k) {
+            re += X[k] * c[2 * k];
+            im += X[k] * c[2 * k + 1];
+        }
+        sG[i] = make_float2(re, im);
+    }
+    float sc, cf, dsc, dcf;
+    hv_rows<CF_THREADS>(hv, f, ft - f * g.T, sS, sc, cf);
+    hv_rows<CF_THREADS>(hd, f, ft - f * g.T, sS2, dsc, dcf);
+    __syncthreads();
+    const float is2 = (float)g.inv_sigma2;
+    auto mul = [](float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); };
+    auto mulc = [](float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y); };   // a conj(b)
+    auto add = [](float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); };
+    const float2 *drow = reinterpret_cast<const float2 *>(data) + (size_t)ft * g.B;
+    for (int b = tid; b < g.B; b += CF_THREADS) {
+        const int code = hv.bmap[b];
+        const float2 gi = sG[g.bl_i[b]], gj = sG[g.bl_j[b]], di = sD[g.bl_i[b]], dj = sD[g.bl_j[b]];
+        const float2 V = hv_value(hv, sS, (size_t)ft, U, code, sc, cf), dV = hv_value(hd, sS2, (size_t)ft, U, code, dsc, dcf);
+        const float2 gg = mulc(gi, gj);
+        const float2 dm = add(mul(add(mulc(di, gj), mulc(gi, dj)), V), mul(gg, dV));
+        float2 om = mulc(dm, gg);
+        float2 ti = mulc(mul(dm, gj), V);                  // dm g_j conj(V), the term in Z_i
+        float2 tj = mulc(mul(gi, V), dm);                  // conj(dm) g_i V, the term in Z_j
+        if (FULL) {
+            const float2 d = drow[b];
+            float2 r = mul(gg, V);
+            r.x -= d.x;
+            r.y -= d.y;
+            om = add(om, mul(r, add(mulc(gj, di), mulc(dj, gi))));
+            ti = add(ti, mul(r, add(mulc(dj, V), mulc(gj, dV))));
+            tj = add(tj, mulc(add(mul(di, V), mul(gi, dV)), r));
+        }
+        sTi[b] = ti;
+        sTj[b] = tj;
+        sW[b] = make_float2(om.x * is2, om.y * is2);
+    }
+    __syncthreads();
+    float qm = group_sums<CF_THREADS>(sW, ft, U, moff, mem, q32);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) qm = fmaxf(qm, __shfl_xor_sync(0xffffffffu, qm, o));
+    if (lane == 0) fred[tid >> 5] = qm;
+    antenna_chunks<CF_THREADS>(sTi, sTj, g.A, sZ);
+    __syncthreads();
+    if (tid == 0) {
+        float m = 0.f;
+        for (int k = 0; k < CF_THREADS / 32; ++k) m = fmaxf(m, fred[k]);
+        qmax_ft[ft] = m;
+    }
+    antenna_totals<CF_THREADS>(sZ, g.A, ft, is2, zpart);
+}
+
+bool launch_hvp_ft_fits(const Ctx &c)
+{
+    return c.A <= CF_THREADS && (2 * c.A + 3 * (size_t)c.B) * 8 + 1024 * (size_t)c.ha.nmt <= 200 * 1024;
+}
+
+fm_status launch_hvp_ft(Ctx &c, const float *gamma, const float *dgamma, int full, float *zpart, const HaVSrc &hv,
+                        const HaVSrc &hd, cudaStream_t st)
+{
+    const size_t smem = (2 * c.A + 3 * (size_t)c.B) * 8 + 1024 * (size_t)c.ha.nmt;
+    auto *kern = full ? k_hvp_ft<true> : k_hvp_ft<false>;
+    FM_CK(smem_opt_in(kern));
+    kern<<<c.F * c.T, CF_THREADS, smem, st>>>(c.g, (const float *)c.data, gamma, dgamma, zpart, c.ha.U, c.ha.moff, c.ha.mem,
+                                              c.ha.q32, c.ha.qmax_ft, hv, hd);
+    FM_CK_LAUNCH();
+    return FM_OK;
 }
 
 template <typename R>
@@ -1182,7 +1245,6 @@ fm_status launch_d2f(long long n, const double *a, float *b, cudaStream_t st)
     template fm_status launch_vis<R>(Ctx &, const R *, R *, cudaStream_t);                               \
     template fm_status launch_adjoint<R>(Ctx &, const R *, R *, cudaStream_t);                           \
     template fm_status launch_apply_gains<R>(Ctx &, const R *, const R *, R *, cudaStream_t);            \
-    template fm_status launch_chi2_mid<R>(Ctx &, const R *, const R *, R *, R *, double *, cudaStream_t); \
     template fm_status launch_hvp_mid<R>(Ctx &, const R *, const R *, const R *, const R *, int, R *, R *, \
                                          cudaStream_t);                                                  \
     template fm_status launch_gain_reduce<R>(Ctx &, const R *, R *, cudaStream_t);                       \
