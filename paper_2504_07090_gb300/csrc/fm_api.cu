@@ -269,13 +269,22 @@ static fm_status create_impl(const fm_config *cfg, Ctx *c)
             if (s != FM_OK) return s;
             FM_CK(e2);
         }
+        if (c->mm.on && !c->ha.ug) {
+            FM_TRY(dalloc(*c, &c->ha.ug, 2 * (size_t)c->F * c->T * c->fg.U));
+            FM_TRY(mm_group_monopole(*c, c->ha.ug));
+        }
         if (c->g.beam64) {                      // the FP64 beam table of an FP32 handle
             FM_CK(cudaDeviceSynchronize());
             cudaFree(const_cast<double *>(c->g.beam64));
             c->g.beam64 = nullptr;
         }
     }
+    if (c->mm.on) {
+        c->mm.ra.R = c->mm.ld;
+        c->mm.ra.f32 = c->mm.b32;
+    }
     FM_TRY(modes_tc_setup(*c));
+    if (c->mm.on && !c->mm.ra.img) FM_TRY(dalloc(*c, &c->mm.tmp, (size_t)c->F * c->mm.ld * c->N));
     return FM_OK;
 }
 
@@ -317,6 +326,19 @@ static fm_status run_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st, b
     return profiled(c, 1, st, [&]() -> fm_status { return launch_adjoint<R>(c, omega, xbar, st); });
 }
 
+// residual weights -> gradient of the sky modes (q_ready: as launch_adjoint_ha)
+template <typename R>
+static fm_status run_adjoint_modes(Ctx &c, const R *omega, R *abar, cudaStream_t st, bool q_ready = false)
+{
+    if constexpr (std::is_same<R, float>::value)
+        if (c.mm.on) {
+            FM_TRY(launch_adjoint_ha_modes(c, omega, st, q_ready));
+            return launch_mm_to_modes(c, abar, st);
+        }
+    FM_TRY(run_adjoint<R>(c, omega, (R *)c.xbar, st, q_ready));
+    return launch_modes_adjoint<R>(c, (R *)c.xbar, abar, st);
+}
+
 // mode transform of one sky for the hour-angle forward.  After the tensor-core transform the
 // channel maxima of x that scale the sky strip are formed, and with one CTA per channel the strips
 // themselves
@@ -327,6 +349,10 @@ static fm_status sky_of_modes(Ctx &c, const float *a, float *x, float *vis, int 
     k.dc = dc ? a : nullptr;
     k.dcs = dc ? c.nk : 0;
     k.slot = slot;
+    if (c.mm.on) {                         // the sky's hour-angle modes; no pixels are formed
+        k.y_ready = true;
+        return launch_mm_from_modes(c, a, slot, st, dc ? 1 : 0);
+    }
     unsigned *xmax = c.mtc.on ? c.ha.xmax + (size_t)slot * c.F : nullptr;
     StripArgs sa;
     if (xmax) {
@@ -408,8 +434,7 @@ fm_status run_chi2_grad(Ctx &c, const R *theta, double *chi2_out, double *u_out,
     } else {
         FM_TRY(launch_chi2_chan<R>(c, vis, theta + c.n_sky, om, zp, c.chi2p, groups, st));   // gains formed inside
     }
-    FM_TRY(run_adjoint<R>(c, om, (R *)c.xbar, st, groups));
-    FM_TRY(launch_modes_adjoint<R>(c, (R *)c.xbar, c.K > 0 ? (R *)c.gx : grad, st));
+    FM_TRY(run_adjoint_modes<R>(c, om, c.K > 0 ? (R *)c.gx : grad, st, groups));
     if (c.K > 0) FM_TRY(launch_freq_contract<R>(c, (const R *)c.gx, grad, st));
     FM_TRY(launch_gain_reduce_chan<R>(c, zp, grad + c.n_sky, st));
     if (c.df_on)
@@ -450,8 +475,7 @@ static fm_status run_hvp(Ctx &c, const R *theta, const R *v, R *hv, int full, cu
         FM_TRY(launch_hvp_mid<R>(c, (R *)c.vis, (R *)c.dvis, (R *)c.gains, (R *)c.dgains, full, (R *)c.omega,
                                  (R *)c.zpart, st));
     }
-    FM_TRY(run_adjoint<R>(c, (R *)c.omega, (R *)c.xbar, st, fused));
-    FM_TRY(launch_modes_adjoint<R>(c, (R *)c.xbar, c.K > 0 ? (R *)c.gx : hv, st));
+    FM_TRY(run_adjoint_modes<R>(c, (R *)c.omega, c.K > 0 ? (R *)c.gx : hv, st, fused));
     if (c.K > 0) FM_TRY(launch_freq_contract<R>(c, (const R *)c.gx, hv, st));
     FM_TRY(launch_gain_reduce_chan<R>(c, (R *)c.zpart, hv + c.n_sky, st));
     return launch_prior_hvp<R>(c, v, hv, st);
@@ -711,10 +735,10 @@ fm_status fm_contraction_info(fm_handle h, int32_t *out)
     FM_HANDLE_OK(h);
     if (!out) return invalid("out is NULL");
     const Ctx &c = *reinterpret_cast<const Ctx *>(h);
-    out[0] = c.ha.on ? 2 : (c.prec >= FM_PREC_BF16X1 ? 1 : 0);
-    out[1] = c.ha.on ? c.ha.U : c.B;
-    out[2] = c.ha.on ? c.ha.k : 0;
-    out[3] = c.ha.on ? c.ha.nhp : 0;
+    out[0] = c.ha.drift ? 2 : (c.prec >= FM_PREC_BF16X1 ? 1 : 0);
+    out[1] = c.ha.drift ? c.ha.U : c.B;
+    out[2] = c.ha.drift ? c.ha.k : 0;
+    out[3] = c.ha.drift ? c.ha.nhp : 0;
     return FM_OK;
 }
 

@@ -126,6 +126,7 @@ template <> struct Tab<float> {
 // LST t depends on n = t k - r + R - 1 only.
 struct HaState {
     bool on = false;
+    bool drift = false;        // the drift-scan geometry of this form holds (also when k_mm.cu computes it)
     int k = 1;                 // LST step in hour-angle cells
     int q = 1;                 // hour-angle cells per RA pixel (the LST step is k / q pixels)
     int nh = 0, nhp = 0;       // hour-angle indices used, padded to a multiple of 128
@@ -202,6 +203,37 @@ struct GdState {
     void *qsum = nullptr;             // [F][T][U][2] group sums of the residual weights
 };
 
+// RA basis of a mode transform: the pixels' functions, or their Fourier sums (k_mm.cu)
+struct RaBasis {
+    int R = 0;                        // rows
+    const float *f32 = nullptr;       // [R][M]
+    const uint8_t *img = nullptr, *imgt = nullptr;   // tensor-core images of it and of its transpose (nullptr: none)
+};
+
+// Contraction in hour-angle Fourier modes (k_mm.cu), split-precision handles.
+struct MmState {
+    bool on = false;
+    int L = 0, q = 1;                 // cells of the window, per RA pixel
+    int nm = 0, ld = 0;               // modes |m| < nm; floats of a row of Y and G (2 nm, padded)
+    int wmax = 0;                     // widest band
+    int mlo = 0, pw = 0;              // phasor table: first mode, columns (the last is mode 1)
+    long long ne = 0;                 // elements (|m|, group, sign) of all channels
+    int nitem = 0;
+    size_t vis_smem = 0;
+    float4 *tab = nullptr;            // [ne][(D + 1) / 2] (Re, Re, Im, Im) of two declinations, sorted by channel and |m|
+    int *moff = nullptr;              // [F][nm + 1] first element of each |m|
+    int *code = nullptr;              // [nmt F][wmax][64] 2 e + conjugated of each mode of each group's band, or -1
+    int4 *items = nullptr;            // forward work: channel, |m|, first element, elements
+    int2 *band = nullptr;             // [F][U] first mode and number of modes
+    float2 *ph = nullptr;             // [T][pw] e^{2 pi i m tau_t / L}
+    float2 *z = nullptr, *w = nullptr;   // [sky][ne] forward sums, [ne] adjoint weights
+    float *Y = nullptr, *G = nullptr; // [sky][F][D][ld] modes of the sky, [F][D][ld] of the gradient
+    double *b64 = nullptr;            // [ld][M] RA basis in modes
+    float *b32 = nullptr, *pix = nullptr;   // the same in FP32; [ld][R] of single pixels
+    float *tmp = nullptr;             // [F][ld][N] when the transform runs on the CUDA cores
+    RaBasis ra;
+};
+
 // Mode <-> pixel transforms on the tensor cores (k_modes.cu): FP16 hi/lo images of the
 // basis tables, 128-byte-swizzled per 64-wide K atom.
 struct ModesTc {
@@ -275,6 +307,7 @@ struct Ctx {
     HaState ha;
     HsState hs;
     GdState gd;
+    MmState mm;
     ModesTc mtc;
     // leapfrog scratch
     void *lf_q0 = nullptr, *lf_g = nullptr, *lf_z = nullptr;
@@ -505,8 +538,8 @@ fm_status ha_set_grids(Ctx &c, int ctas_fwd, int ctas_adj);
 // tensor-core mode transforms (float handles of the split precisions)
 fm_status modes_tc_setup(Ctx &c);
 fm_status launch_modes_tc_forward(Ctx &c, const float *a, float *x, cudaStream_t st, int skip_dc, unsigned *xmax,
-                                  const StripArgs *strips = nullptr);
-fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaStream_t st);
+                                  const StripArgs *strips = nullptr, const RaBasis *ra = nullptr);
+fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaStream_t st, const RaBasis *ra = nullptr);
 // windows of wider images as pixel maps: map f is the window of R columns from column off[f / per] of
 // image f % per, images [D][ld] (16-byte aligned, ld a multiple of 4 with 4 columns past the last window)
 // whose largest magnitudes are xmax[per] (float bits); per = 0: maps [nmaps][D][R]
@@ -517,7 +550,16 @@ struct MapWindows {
     const unsigned *xmax = nullptr;
 };
 fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st,
-                                       const MapWindows *w = nullptr);
+                                       const MapWindows *w = nullptr, const RaBasis *ra = nullptr);
+// hour-angle modes (k_mm.cu): setup, both contractions from and to the modes c.mm.Y and c.mm.G, and the
+// transforms between sky modes (or pixels) and them (k_simt.cu)
+fm_status mm_setup(Ctx &c);
+fm_status mm_group_monopole(Ctx &c, float *ug);
+fm_status launch_mm_forward(Ctx &c, int nsky, int slot_rows, int N, float *vpart, cudaStream_t st);
+fm_status launch_mm_adjoint(Ctx &c, const float *q32, cudaStream_t st);
+fm_status launch_mm_from_modes(Ctx &c, const float *a, int slot, cudaStream_t st, int skip_dc);
+fm_status launch_mm_from_pixels(Ctx &c, const float *x, int slot, cudaStream_t st);
+fm_status launch_mm_to_modes(Ctx &c, float *abar, cudaStream_t st);
 // One sky of the hour-angle forward: pixels x -> visibilities vis.  dc != nullptr: also adds the
 // monopole visibilities dc[f * dcs] U[f][t][b]; slot: which of the two strip and maxima buffers it uses;
 // xmax_ready: the channel maxima of x are already in c.ha.xmax (formed by the mode transform);
@@ -531,12 +573,15 @@ struct HaSky {
     int slot = 0;
     const float *gamma = nullptr;    // gain coefficients [A][NG][2]: vis = g_p conj(g_q) V instead of V
     bool xmax_ready = false, strips_ready = false;
+    bool y_ready = false;            // hour-angle modes: c.mm.Y of the slot is formed
 };
 // partials_only: V is not finished (the forward's partial sums stay in c.ha.vpart for the chi^2
 // epilogue, HaVSrc)
 fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only = false);
 // two skies (slots 0 and 1) in one pass over the responses; needs c.ha.dual
 fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b, bool partials_only = false);
+// the gradient's hour-angle modes c.mm.G instead of pixels (c.mm.on)
+fm_status launch_adjoint_ha_modes(Ctx &c, const float *omega, cudaStream_t st, bool q_ready = false);
 // q_ready: the group sums q32 / qmax_ft were already formed from omega (by the chi^2 epilogue)
 fm_status launch_adjoint_ha(Ctx &c, const float *omega, float *xbar, cudaStream_t st, bool q_ready = false);
 

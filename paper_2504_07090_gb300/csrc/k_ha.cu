@@ -1497,7 +1497,7 @@ static void ha_partition(Ctx &c, int G, std::vector<int> &ncontrib)
 fm_status ha_set_grids(Ctx &c, int ctas_fwd, int ctas_adj)
 {
     HaState &s = c.ha;
-    if (!s.on) { set_error("the handle does not run the hour-angle form"); return FM_ERR_UNSUPPORTED; }
+    if (!s.drift) { set_error("the handle does not run the hour-angle form"); return FM_ERR_UNSUPPORTED; }
     const int sm = sm_count();
     if (ctas_fwd < 0 || ctas_adj < 0 || ctas_fwd > sm || ctas_adj > sm) {
         set_error("launch grids must be in [0, %d] CTAs (0: one per SM)", sm);
@@ -1506,28 +1506,25 @@ fm_status ha_set_grids(Ctx &c, int ctas_fwd, int ctas_adj)
     std::vector<int> ncontrib;
     const int Jmax = s.J_alloc;
     ha_partition(c, ctas_fwd > 0 ? ctas_fwd : sm, ncontrib);
-    if (s.J > Jmax) {                      // cannot happen for G <= the default; kept as a guard
+    if (s.J > Jmax && !c.mm.on) {                      // cannot happen for G <= the default; kept as a guard
         ha_partition(c, sm, ncontrib);
         set_error("forward grid needs %d partial sums per segment, %d allocated", s.J, Jmax);
         return FM_ERR_INVALID_ARG;
     }
     s.J = Jmax;                            // the buffer's stride stays that of the allocation
-    FM_CK(cudaMemcpy(s.ncontrib, ncontrib.data(), sizeof(int) * ncontrib.size(), cudaMemcpyHostToDevice));
     s.grid_adj = ctas_adj;
+    if (c.mm.on) return FM_OK;             // hour-angle modes: grids of their own, no partition
+    FM_CK(cudaMemcpy(s.ncontrib, ncontrib.data(), sizeof(int) * ncontrib.size(), cudaMemcpyHostToDevice));
     return FM_OK;
 }
 
-fm_status ha_setup(Ctx &c)
+// Geometry, tile and partition fields; true when the drift-scan geometry and the tiles of both kernels fit.
+static bool ha_geometry(Ctx &c, std::vector<int> &ncontrib)
 {
     HaState &s = c.ha;
-    s.on = false;
-    if (c.prec < FM_PREC_BF16X1) return FM_OK;
-    if (const char *e = getenv("FM_HA"))
-        if (atoi(e) == 0) return FM_OK;
-    if (c.A < 2 || c.R > 512) return FM_OK;
-    const double dra = (c.cfg.ra_max - c.cfg.ra_min) / c.R;
+    if (c.R > 512) return false;
     int k = 1, q = 1;
-    if (!drift_step(c, k, q)) return FM_OK;
+    if (!drift_step(c, k, q)) return false;
     s.k = k;
     s.q = q;
     s.nh = (c.R - 1) * q + (c.T - 1) * k + 1;
@@ -1547,24 +1544,20 @@ fm_status ha_setup(Ctx &c)
     image(HA_TCHUNK);
 
     const FringeGroups &fg = c.fg;
-    s.U = fg.U;
-    s.nmt = (s.U + 63) / 64;
-    s.nkq = (s.U + 31) / 32;
     // the table holds at most 63 antennas plus its zero entry
-    if (fg.nant > 63) return FM_OK;
+    if (fg.nant > 63) return false;
     s.nant = fg.nant;
     for (int a = 0; a < s.nant; ++a) s.ant_of[a] = fg.ant_of[a];
 
     // partition of the forward work units over the CTAs (the default grid: one CTA per SM;
     // the partial-sum buffer is sized for it, and a smaller grid needs no more contributors)
-    std::vector<int> ncontrib;
     ha_partition(c, sm_count(), ncontrib);
 
     // both kernels' tiles must fit in shared memory
     {
         HaLayout L1, L2;
         const bool x3 = x3_of(c.prec);
-        if (!make_layout_fwd(c, x3, HaFwd::narrow, L1) || !make_layout_adj(c, x3, s.npad, HA_NSTAGE, L2)) return FM_OK;
+        if (!make_layout_fwd(c, x3, HaFwd::narrow, L1) || !make_layout_adj(c, x3, s.npad, HA_NSTAGE, L2)) return false;
         // more than 64 LSTs: passes of 128 where their image fits; else two skies a pass where theirs does
         s.wide = s.dual = false;
         s.npa = s.npad;
@@ -1587,6 +1580,55 @@ fm_status ha_setup(Ctx &c)
             s.dual = make_layout_fwd(c, x3, HaFwd::dual, L1);
         }
     }
+    return true;
+}
+
+// The contraction in hour-angle modes (k_mm.cu) in this form's place: its results take the place of one
+// contributor's partial sums of all LSTs, in a scale of one, and the finishing kernels and epilogues are shared.
+static fm_status ha_of_modes(Ctx &c)
+{
+    HaState &s = c.ha;
+    s.npad = s.npf = c.T;
+    s.dual = true;
+    s.wide = false;
+    s.J = s.J_alloc = 1;
+    s.sp = 1.f;
+    s.bmap = c.fg.bmap;
+    s.moff = c.fg.moff;
+    s.mem = c.fg.mem;
+    const std::vector<int> one((size_t)s.nmt * c.F, 1);
+    FM_TRY(ha_alloc(c, &s.ncontrib, one.size()));
+    FM_CK(cudaMemcpy(s.ncontrib, one.data(), sizeof(int) * one.size(), cudaMemcpyHostToDevice));
+    FM_TRY(ha_alloc(c, &s.xmax, 2 * (size_t)c.F));
+    FM_CK(cudaMemset(s.xmax, 0, sizeof(unsigned) * 2 * c.F));
+    FM_TRY(ha_alloc(c, &s.vpart, (size_t)s.nmt * c.F * 2 * c.T * 128));
+    FM_TRY(ha_alloc(c, &s.q32, (size_t)c.F * c.T * s.U * 2));
+    FM_TRY(ha_alloc(c, &s.qmax_ft, (size_t)c.F * c.T));
+    s.on = true;
+    return FM_OK;
+}
+
+fm_status ha_setup(Ctx &c)
+{
+    HaState &s = c.ha;
+    s.on = s.drift = false;
+    if (c.prec < FM_PREC_BF16X1) return FM_OK;
+    if (const char *e = getenv("FM_HA"))
+        if (atoi(e) == 0) return FM_OK;
+    const FringeGroups &fg = c.fg;
+    s.U = fg.U;
+    s.nmt = (s.U + 63) / 64;
+    s.nkq = (s.U + 31) / 32;
+    std::vector<int> ncontrib;
+    const bool fits = ha_geometry(c, ncontrib);
+    // the x1 precisions keep the rounding of their products; what has neither this form nor the antenna form
+    // (64 antennas) stays without one
+    if (x3_of(c.prec) && (fits || c.A <= 64)) FM_TRY(mm_setup(c));
+    if (c.mm.on) {
+        s.drift = fits;
+        return ha_of_modes(c);
+    }
+    if (!fits) return FM_OK;
 
     // device memory, all of it within half of what is free
     const size_t e_n = (size_t)c.F * c.D * s.nbc * (s.nant + 1) * HA_EW;
@@ -1633,7 +1675,7 @@ fm_status ha_setup(Ctx &c)
     a.F = c.F; a.D = c.D; a.R = c.R; a.A = s.nant + 1; a.A_all = c.A; a.nh = s.nh; a.nhp = s.nhp; a.nbc = s.nbc;
     a.q = s.q;
     for (int q = 0; q < s.nant; ++q) a.ant[q] = s.ant_of[q];
-    a.lst0 = c.lst[0]; a.ra_min = c.cfg.ra_min; a.dra = dra;
+    a.lst0 = c.lst[0]; a.ra_min = c.cfg.ra_min; a.dra = (c.cfg.ra_max - c.cfg.ra_min) / c.R;
     a.dec_min = c.cfg.dec_min; a.ddec = (c.cfg.dec_max - c.cfg.dec_min) / c.D;
     a.lat = c.cfg.latitude_rad; a.amp_scale = std::ldexp(1.0, e2 / 2);
     a.kap64 = c.g.kap64; a.bcoef64 = c.g.bcoef64; a.domega64 = c.g.domega64;
@@ -1643,7 +1685,7 @@ fm_status ha_setup(Ctx &c)
     k_ha_table<<<2048, 256>>>(a, 0, reinterpret_cast<float *>(s.Ea));
     FM_CK_LAUNCH();
     FM_CK(cudaDeviceSynchronize());
-    s.on = true;
+    s.on = s.drift = true;
     return FM_OK;
 }
 
@@ -1699,8 +1741,25 @@ fm_status ha_monopole(Ctx &c, float *U, cudaStream_t st)
     return rc;
 }
 
+// forward in hour-angle modes: one sky, or both slots'
+static fm_status vis_mm(Ctx &c, const HaSky &k, const HaSky *k2, bool partials_only)
+{
+    HaState &s = c.ha;
+    for (const HaSky *p : {&k, k2})
+        if (p && !p->y_ready) FM_TRY(launch_mm_from_pixels(c, p->x, p->slot, p->st));
+    HaDev h = make_dev(c);
+    h.T = c.T;
+    h.N = k2 ? 2 * s.npad : s.npf;
+    h.dual = k2 != nullptr;
+    FM_TRY(launch_mm_forward(c, k2 ? 2 : 1, s.npad, h.N, s.vpart, k.st));
+    if (partials_only) return FM_OK;
+    FM_TRY(fwd_finish(c, h, k));
+    return k2 ? fwd_finish(c, h, *k2) : FM_OK;
+}
+
 fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only)
 {
+    if (c.mm.on) return vis_mm(c, k, nullptr, partials_only);
     const HaDev h = make_dev(c);
     const bool x3 = x3_of(c.prec), po = partials_only;
     if (f16_of(c.prec)) return x3 ? vis_ha_launch<1, true>(c, h, k, po) : vis_ha_launch<1, false>(c, h, k, po);
@@ -1709,6 +1768,7 @@ fm_status launch_vis_ha(Ctx &c, const HaSky &k, bool partials_only)
 
 fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b, bool po)
 {
+    if (c.mm.on) return vis_mm(c, a, &b, po);
     const HaDev h = make_dev(c);
     const bool x3 = x3_of(c.prec);
     if (f16_of(c.prec)) return x3 ? vis_ha_dual_launch<1, true>(c, h, a, b, po) : vis_ha_dual_launch<1, false>(c, h, a, b, po);
@@ -1718,7 +1778,7 @@ fm_status launch_vis_ha_dual(Ctx &c, const HaSky &a, const HaSky &b, bool po)
 bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
 {
     const HaState &s = c.ha;
-    if (!s.on || c.T > (s.wide ? HA_TWIDE : HA_TCHUNK) || (dc && !s.ug)) return false;
+    if (!s.on || (!c.mm.on && c.T > (s.wide ? HA_TWIDE : HA_TCHUNK)) || (dc && !s.ug)) return false;
     if (const char *e = getenv("FM_HA_FUSED_CHI2"))      // 0: V finished by its own kernel
         if (atoi(e) == 0) return false;
     v.vpart = s.vpart;
@@ -1761,6 +1821,17 @@ bool ha_strip_args(const Ctx &c, StripArgs &sa, int slot)
     return true;
 }
 
+fm_status launch_adjoint_ha_modes(Ctx &c, const float *omega, cudaStream_t st, bool q_ready)
+{
+    const HaState &s = c.ha;
+    if (!q_ready) {
+        k_ha_qsum<<<c.F * c.T, 256, sizeof(float) * 2 * (size_t)c.B, st>>>(make_dev(c), c.B, omega, s.moff, s.mem, s.q32,
+                                                                            s.qmax_ft);
+        FM_CK_LAUNCH();
+    }
+    return launch_mm_adjoint(c, s.q32, st);
+}
+
 fm_status launch_adjoint_ha(Ctx &c, const float *omega, float *xbar, cudaStream_t st, bool q_ready)
 {
     const HaDev h = make_dev(c);
@@ -1792,7 +1863,7 @@ extern "C" fm_status fm_get_launch_grids(fm_handle h, int32_t *out)
         return FM_ERR_INVALID_ARG;
     }
     const Ctx &c = *reinterpret_cast<const Ctx *>(h);
-    out[0] = c.ha.on ? c.ha.grid : 0;
-    out[1] = c.ha.on ? (c.ha.grid_adj > 0 ? c.ha.grid_adj : (sm_count() < c.F * c.D ? sm_count() : c.F * c.D)) : 0;
+    out[0] = c.ha.drift ? c.ha.grid : 0;
+    out[1] = c.ha.drift ? (c.ha.grid_adj > 0 ? c.ha.grid_adj : (sm_count() < c.F * c.D ? sm_count() : c.F * c.D)) : 0;
     return FM_OK;
 }

@@ -682,12 +682,12 @@ k_modes_adj(MdDims z, int ns, const float *__restrict__ xb_all, const uint8_t *_
     md_finish(m, ok, status, tmem, ncols);
 }
 
-MdDims md_dims(const Ctx &c)
+MdDims md_dims(const Ctx &c, const RaBasis *ra = nullptr)
 {
     MdDims z;
-    z.F = c.F; z.M = c.M; z.N = c.N; z.R = c.R; z.D = c.D;
+    z.F = c.F; z.M = c.M; z.N = c.N; z.R = ra ? ra->R : c.R; z.D = c.D;
     z.Mp = (c.M + 63) / 64 * 64; z.Np = (c.N + 63) / 64 * 64;
-    z.Rp = (c.R + 63) / 64 * 64; z.Dp = (c.D + 63) / 64 * 64;
+    z.Rp = (z.R + 63) / 64 * 64; z.Dp = (c.D + 63) / 64 * 64;
     return z;
 }
 
@@ -758,6 +758,22 @@ fm_status modes_tc_setup(Ctx &c)
     }
     k_md_image<<<256, 256>>>(c.g.leg64, c.D, c.N, 1, 0, z.Np, z.Dp, MD_CSCALE, s.legt_img);
     FM_CK_LAUNCH();
+    if (c.mm.on && (c.mm.ld + 63) / 64 * 64 <= 256) {          // the RA basis in hour-angle modes
+        const MdDims y = md_dims(c, &c.mm.ra);
+        const size_t img_n = 2 * (size_t)y.Rp * y.Mp, imgt_n = (size_t)nmt * 2 * 128 * y.Rp;
+        uint8_t *b = nullptr;
+        FM_CK(cudaMalloc(&b, 2 * (img_n + imgt_n)));
+        c.allocs.push_back(b);
+        c.mm.ra.img = b;
+        c.mm.ra.imgt = b + 2 * img_n;
+        k_md_image<<<256, 256>>>(c.mm.b64, y.R, c.M, 0, 0, y.Rp, y.Mp, MD_CSCALE, b);
+        FM_CK_LAUNCH();
+        for (int mt = 0; mt < nmt; ++mt) {
+            k_md_image<<<256, 256>>>(c.mm.b64, y.R, c.M, 1, 128 * mt, 128, y.Rp, MD_CSCALE,
+                                     b + 2 * img_n + (size_t)mt * 2 * 2 * 128 * y.Rp);
+            FM_CK_LAUNCH();
+        }
+    }
     FM_CK(smem_opt_in(k_modes_fwd<MD_THREADS>));
     FM_CK(smem_opt_in(k_modes_fwd<MD_WIDE>));
     FM_CK(smem_opt_in((k_modes_adj<MD_THREADS, false>)));
@@ -769,9 +785,9 @@ fm_status modes_tc_setup(Ctx &c)
 }
 
 fm_status launch_modes_tc_forward(Ctx &c, const float *a, float *x, cudaStream_t st, int skip_dc, unsigned *xmax,
-                                  const StripArgs *strips)
+                                  const StripArgs *strips, const RaBasis *ra)
 {
-    const MdDims z = md_dims(c);
+    const MdDims z = md_dims(c, ra);
     const int ndt = (c.D + 127) / 128, ns = md_slots(c.F * ndt);
     if (strips && (ndt != 1 || !xmax)) {
         set_error("sky strips need one CTA per channel and the channel maxima");
@@ -780,29 +796,29 @@ fm_status launch_modes_tc_forward(Ctx &c, const float *a, float *x, cudaStream_t
     const bool wide = md_wide(ns, z.Mp, z.Np);
     auto *kern = wide ? k_modes_fwd<MD_WIDE> : k_modes_fwd<MD_THREADS>;
     kern<<<dim3(c.F, ndt), wide ? MD_WIDE : MD_THREADS, md_smem_bytes(z.Mp > z.Rp ? z.Mp : z.Rp, ns), st>>>(
-        z, ns, a, skip_dc, c.mtc.leg_img, c.mtc.phi_img, x, c.status, md_cols(z.Mp + z.Rp), xmax,
+        z, ns, a, skip_dc, c.mtc.leg_img, ra ? ra->img : c.mtc.phi_img, x, c.status, md_cols(z.Mp + z.Rp), xmax,
         strips ? *strips : StripArgs{});
     FM_CK_LAUNCH();
     return FM_OK;
 }
 
-fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaStream_t st)
+fm_status launch_modes_tc_adjoint(Ctx &c, const float *xbar, float *abar, cudaStream_t st, const RaBasis *ra)
 {
-    return launch_modes_tc_adjoint_maps(c, xbar, c.F, abar, st);
+    return launch_modes_tc_adjoint_maps(c, xbar, c.F, abar, st, nullptr, ra);
 }
 
 // the same transform for nmaps pixel maps xbar[nmaps][D][R] -> abar[nmaps][M][N], or the windows w of
 // wider images
 fm_status launch_modes_tc_adjoint_maps(Ctx &c, const float *xbar, int nmaps, float *abar, cudaStream_t st,
-                                       const MapWindows *w)
+                                       const MapWindows *w, const RaBasis *ra)
 {
-    MdDims z = md_dims(c);
+    MdDims z = md_dims(c, ra);
     z.F = nmaps;
     const int nmt = (c.M + 127) / 128, ns = md_slots(nmaps * nmt);
     const bool wide = !w && md_wide(ns, z.Dp, z.Rp);
     auto *kern = w ? k_modes_adj<MD_THREADS, true> : wide ? k_modes_adj<MD_WIDE, false> : k_modes_adj<MD_THREADS, false>;
     kern<<<dim3(nmaps, nmt), wide ? MD_WIDE : MD_THREADS, md_smem_bytes(z.Dp > z.Np ? z.Dp : z.Np, ns), st>>>(
-        z, ns, xbar, c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np), w ? *w : MapWindows{});
+        z, ns, xbar, ra ? ra->imgt : c.mtc.phit_img, c.mtc.legt_img, abar, c.status, md_cols(z.Dp + z.Np), w ? *w : MapWindows{});
     FM_CK_LAUNCH();
     return FM_OK;
 }

@@ -154,6 +154,37 @@ fm_status launch_modes_adjoint(Ctx &c, const R *xbar, R *abar, cudaStream_t st)
     return gemm<R>(s2, c.F, tab_phi<R>(c), t2, abar, st);
 }
 
+// the same between sky modes (or pixels) and hour-angle modes (k_mm.cu): Y[f][d][c] with the RA basis B[c][m]
+fm_status launch_mm_from_modes(Ctx &c, const float *a, int slot, cudaStream_t st, int skip_dc)
+{
+    const MmState &s = c.mm;
+    float *y = s.Y + (size_t)slot * c.F * c.D * s.ld;
+    if (s.ra.img) return launch_modes_tc_forward(c, a, y, st, skip_dc, nullptr, nullptr, &s.ra);
+    const long long tn = (long long)s.ld * c.N;
+    GemmArgs s1{s.ld, c.N, c.M, 0, c.M, 1, c.nk, c.N, 1, tn, c.N, 1, skip_dc};
+    FM_TRY(gemm<float>(s1, c.F, s.b32, a, s.tmp, st));
+    GemmArgs s2{c.D, s.ld, c.N, 0, c.N, 1, tn, 1, c.N, (long long)c.D * s.ld, s.ld, 1, 0};
+    return gemm<float>(s2, c.F, tab_leg<float>(c), s.tmp, y, st);
+}
+
+fm_status launch_mm_from_pixels(Ctx &c, const float *x, int slot, cudaStream_t st)
+{
+    const MmState &s = c.mm;
+    GemmArgs g{c.D, s.ld, c.R, c.npix, c.R, 1, 0, 1, c.R, (long long)c.D * s.ld, s.ld, 1, 0};
+    return gemm<float>(g, c.F, x, s.pix, s.Y + (size_t)slot * c.F * c.D * s.ld, st);
+}
+
+fm_status launch_mm_to_modes(Ctx &c, float *abar, cudaStream_t st)
+{
+    const MmState &s = c.mm;
+    if (s.ra.img) return launch_modes_tc_adjoint(c, s.G, abar, st, &s.ra);
+    const long long tn = (long long)s.ld * c.N;
+    GemmArgs s1{s.ld, c.N, c.D, (long long)c.D * s.ld, 1, s.ld, 0, c.N, 1, tn, c.N, 1, 0};
+    FM_TRY(gemm<float>(s1, c.F, s.G, tab_leg<float>(c), s.tmp, st));
+    GemmArgs s2{c.M, c.N, s.ld, 0, 1, c.M, tn, c.N, 1, c.nk, c.N, 1, 0};
+    return gemm<float>(s2, c.F, s.b32, s.tmp, abar, st);
+}
+
 // ---------------------------------------------------------------- gains
 template <typename R>
 __global__ void k_gains(DevGeom g, const R *__restrict__ gamma, R *__restrict__ out)
