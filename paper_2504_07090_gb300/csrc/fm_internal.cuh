@@ -180,6 +180,8 @@ struct FringeGroups {
     int *bmap = nullptr;              // [B] group * 2 + (1 if the baseline is the reversed vector)
     int *moff = nullptr;              // [U + 1] CSR offsets of group members
     int *mem = nullptr;               // [B] members, b * 2 + reversed
+    int2 *pairs = nullptr;            // [B] (i | j << 16, bmap) of every baseline
+    int2 *gmem = nullptr;             // [B] (mem, i | j << 16) of every member
 };
 
 // Drift-scan form of the contraction on the CUDA cores (k_hs.cu), FP64 and FP32 handles.

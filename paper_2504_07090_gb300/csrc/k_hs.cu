@@ -191,6 +191,11 @@ fm_status fringe_setup(Ctx &c)
         FM_CK(cudaMemcpy(*dst, src.data(), n, cudaMemcpyHostToDevice));
         return FM_OK;
     };
+    std::vector<int2> hpair(c.B), hgm(c.B);
+    for (int b = 0; b < c.B; ++b) hpair[b] = make_int2(bi[b] | (bj[b] << 16), bmap[b]);
+    for (int m = 0; m < c.B; ++m) hgm[m] = make_int2(hmem[m], hpair[hmem[m] >> 1].x);
+    FM_TRY(put(&fg.pairs, hpair));
+    FM_TRY(put(&fg.gmem, hgm));
     FM_TRY(put(&fg.uij, huij));
     FM_TRY(put(&fg.ant, fg.ant_of));
     FM_TRY(put(&fg.bmap, bmap));

@@ -478,6 +478,39 @@ __device__ void block_sum_double(double v, double *out, double *sred)
 
 // ---- pieces of the per-(channel, LST) epilogues k_chi2_ft and k_hvp_ft
 
+__device__ __forceinline__ float hv_scale(const HaVSrc &hv, int f)
+{
+    const float mx = __uint_as_float(hv.xmax[f]);
+    float s2 = 1.f;
+    if (mx > 0.f && isfinite(mx)) {
+        int ex;
+        frexpf(mx, &ex);
+        s2 = ldexpf(1.f, 14 - ex);
+    }
+    return 1.f / (hv.sp * s2);
+}
+
+// the contributors' partial rows 2 u, 2 u + 1 of the forward at LST t of channel f, added in rank order
+__device__ __forceinline__ float2 hv_row(const HaVSrc &hv, int f, int t, int u)
+{
+    const int seg = (u >> 6) * hv.F + f, nc = hv.ncontrib[seg];
+    const float2 *src = reinterpret_cast<const float2 *>(hv.vpart + ((size_t)seg * hv.J * hv.npad + t) * 128) + (u & 63);
+    const size_t js = (size_t)hv.npad * 64;
+    float2 a = make_float2(0.f, 0.f);
+    for (int j0 = 0; j0 < nc; j0 += 4) {
+        float2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = j0 + q < nc ? src[(size_t)(j0 + q) * js] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (j0 + q < nc) {
+                a.x += v[q].x;
+                a.y += v[q].y;
+            }
+    }
+    return a;
+}
+
 // sS[row], row < 128 nmt: the contributors' partial rows of the forward at LST t of channel f, in rank
 // order; sc and cf: the scale of the sum and the monopole's coefficient
 template <int NT>
@@ -499,14 +532,7 @@ __device__ __forceinline__ void hv_rows(const HaVSrc &hv, int f, int t, float *s
         }
         sS[e] = a;
     }
-    const float mx = __uint_as_float(hv.xmax[f]);
-    float s2 = 1.f;
-    if (mx > 0.f && isfinite(mx)) {
-        int ex;
-        frexpf(mx, &ex);
-        s2 = ldexpf(1.f, 14 - ex);
-    }
-    sc = 1.f / (hv.sp * s2);
+    sc = hv_scale(hv, f);
     cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
 }
 
@@ -609,12 +635,11 @@ __device__ __forceinline__ void antenna_totals(const C2 *sZ, int A, int ft, R is
 // sums and the groups' monopole visibilities (HaVSrc) instead of being read from vis.  Needs
 // A <= CF_THREADS.
 //
-// NT threads a CTA: 256, eight CTAs an SM, while a (channel, LST)'s terms are small; 1024 where they take
-// so much shared memory (24 bytes a baseline: 192 KB for 127 antennas) that at most three of 256 would
-// fit an SM and its loads would be left uncovered (127 antennas: 3.23 ms with 256).
-constexpr int CF_THREADS = 256, CF_BIG = 1024;
-template <typename R, int NT>
-__global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1) k_chi2_ft(DevGeom g, const R *__restrict__ vis, const R *__restrict__ data,
+// Eight CTAs of 256 threads an SM while a (channel, LST)'s terms (24 bytes a baseline) are small; handles of the
+// hour-angle form run k_chi2_group below where they are not.
+constexpr int CF_THREADS = 256;
+template <typename R>
+__global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(DevGeom g, const R *__restrict__ vis, const R *__restrict__ data,
                                                         const R *__restrict__ gamma, R *__restrict__ omega,
                                                         R *__restrict__ zpart, double *__restrict__ chi2p, int U,
                                                         const int *__restrict__ moff, const int *__restrict__ mem,
@@ -622,6 +647,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1
                                                         const R *__restrict__ rin, HaVSrc hv)
 {
     using C2 = typename V2<R>::t;
+    constexpr int NT = CF_THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2 *sG = reinterpret_cast<C2 *>(smem_raw);            // [A]
     C2 *sTi = sG + g.A;                                    // [B] term of baseline (i, j) in Z_i
@@ -716,6 +742,157 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && NT == CF_THREADS ? 8 : 1
     antenna_totals<NT>(sZ, g.A, ft, is2, zpart);
 }
 
+// The same for large arrays of the hour-angle form, whose visibilities are those of the fringe groups: V_u
+// (finished here from the forward's partial sums, hv, or taken from the finished vis) and the residuals are all
+// that a CTA keeps, 8 bytes a baseline instead of the 24 of both gain terms and omega.  The sums over the groups' members
+// (q32, their largest |Re|, |Im| to qmax_ft) and over the antennas' partners form their terms again from those,
+// the reversed partner of a pair as its conjugate.
+//
+// Bound: latency of the loads and barriers of one (channel, LST), so what counts is the CTAs an SM holds: three
+// of 512 with 127 antennas (64 KB of residuals; 192 KB with 24 bytes a baseline, one CTA).  127 antennas, 128
+// channels, 120 LSTs: 1.68 -> 1.10 ms (two CTAs of 1024: 1.23 ms).  With 37 antennas k_chi2_ft is the faster one
+// (33 against 36 us).
+constexpr int CG_THREADS = 512;
+__global__ void __launch_bounds__(CG_THREADS, 3)
+k_chi2_group(DevGeom g, const float *__restrict__ vis, const float *__restrict__ data, const float *__restrict__ gamma,
+             float *__restrict__ zpart, double *__restrict__ chi2p, int U, const int2 *__restrict__ pairs,
+             const int2 *__restrict__ gmem, const int *__restrict__ moff, float *__restrict__ q32,
+             float *__restrict__ qmax_ft, const float *__restrict__ rin, HaVSrc hv)
+{
+    constexpr int NT = CG_THREADS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *sG = reinterpret_cast<float2 *>(smem_raw);     // [A]
+    float2 *sV = sG + g.A;                                 // [U]
+    float2 *sR = sV + U;                                   // [B] residuals
+    __shared__ float2 sZ[NT];                              // chunk sums of Z_a
+    __shared__ double dred[NT / 32];
+    __shared__ float fred[NT / 32];
+    const int ft = blockIdx.x, f = ft / g.T, t = ft - f * g.T, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    {
+        const float *X = g.gleg32 + (size_t)f * g.NG;
+        for (int i = tid; i < g.A; i += NT) {              // as k_gains
+            float re = 0, im = 0;
+            for (int k = 0; k < g.NG; ++k) {
+                re += X[k] * gamma[(i * g.NG + k) * 2];
+                im += X[k] * gamma[(i * g.NG + k) * 2 + 1];
+            }
+            sG[i] = make_float2(re, im);
+        }
+    }
+    if (hv.vpart) {
+        const float sc = hv_scale(hv, f), cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
+        for (int u = tid; u < U; u += NT) {                // with the roundings of k_ha_vfinish
+            const float2 v = hv_row(hv, f, t, u);
+            float2 V = make_float2(__fmul_rn(v.x, sc), __fmul_rn(v.y, sc));
+            if (hv.dc) {
+                const float2 m = reinterpret_cast<const float2 *>(hv.ug)[(size_t)ft * U + u];
+                V = make_float2(__fmaf_rn(cf, m.x, V.x), __fmaf_rn(cf, m.y, V.y));
+            }
+            sV[u] = V;
+        }
+    } else {
+        const float2 *vrow = reinterpret_cast<const float2 *>(vis) + (size_t)ft * g.B;
+        for (int u = tid; u < U; u += NT) {                // the first member's
+            const int code = gmem[moff[u]].x;
+            const float2 v = vrow[code >> 1];
+            sV[u] = make_float2(v.x, (code & 1) ? -v.y : v.y);
+        }
+    }
+    __syncthreads();
+    const float is2 = (float)g.inv_sigma2;
+    const float2 *drow = reinterpret_cast<const float2 *>(data) + (size_t)ft * g.B;
+    // rin != NULL (delay filter): the residual weights come in precomputed, sigma^2 F^T W F r
+    const float2 *rrow = rin ? reinterpret_cast<const float2 *>(rin) + (size_t)ft * g.B : nullptr;
+    float c2 = 0;
+#pragma unroll 2
+    for (int b = tid; b < g.B; b += NT) {
+        float2 r;
+        if (rrow) {
+            r = rrow[b];
+        } else {
+            const int2 p = __ldg(pairs + b);               // i | j << 16, 2 u + reversed
+            const float2 d = __ldg(drow + b), gi = sG[p.x & 0xffff], gj = sG[p.x >> 16];
+            float2 V = sV[p.y >> 1];
+            if (p.y & 1) V.y = -V.y;
+            const float ggr = gi.x * gj.x + gi.y * gj.y, ggi = gi.y * gj.x - gi.x * gj.y;     // g_i conj(g_j)
+            r.x = ggr * V.x - ggi * V.y - d.x;
+            r.y = ggr * V.y + ggi * V.x - d.y;
+        }
+        c2 += r.x * r.x + r.y * r.y;
+        sR[b] = r;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+    if (lane == 0) dred[w] = (double)c2;
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        for (int k = 0; k < NT / 32; ++k) a += dred[k];
+        chi2p[ft] = a * g.inv_sigma2;
+    }
+    // sums of omega = conj(g_i) g_j r / sigma^2 over the groups' members: four lanes a group, each every fourth
+    // member, added in a fixed order
+    float qm = 0.f;
+    for (int u0 = 0; u0 < U; u0 += NT / 4) {
+        const int u = u0 + (tid >> 2);
+        float qr = 0.f, qi = 0.f;
+        if (u < U) {
+            const int m1 = moff[u + 1];
+#pragma unroll 4
+            for (int m = moff[u] + (tid & 3); m < m1; m += 4) {
+                const int2 p = __ldg(gmem + m);            // 2 b + reversed, i | j << 16
+                const float2 r = sR[p.x >> 1], gi = sG[p.y & 0xffff], gj = sG[p.y >> 16];
+                const float ggr = gi.x * gj.x + gi.y * gj.y, ggi = gi.y * gj.x - gi.x * gj.y;
+                const float oi = ggr * r.y - ggi * r.x;
+                qr += ggr * r.x + ggi * r.y;
+                qi += (p.x & 1) ? -oi : oi;
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            qr += __shfl_xor_sync(0xffffffffu, qr, o);
+            qi += __shfl_xor_sync(0xffffffffu, qi, o);
+        }
+        if (u < U && (tid & 3) == 0) {
+            qr *= is2;
+            qi *= is2;
+            *reinterpret_cast<float2 *>(q32 + ((size_t)ft * U + u) * 2) = make_float2(qr, qi);
+            qm = fmaxf(qm, fmaxf(fabsf(qr), fabsf(qi)));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) qm = fmaxf(qm, __shfl_xor_sync(0xffffffffu, qm, o));
+    if (lane == 0) fred[w] = qm;
+    // chunk c = tid mod nc of Z_a, a = tid div nc: partners j = c, c + nc, ... (j != a) of r g_j conj(V), r and V
+    // conjugated for j < a
+    const int nc = NT / g.A;
+    if (tid < nc * g.A) {
+        const int a = tid / nc, rowa = a * g.A - (a * (a + 1)) / 2 - a - 1;
+        float zr = 0, zi = 0;
+#pragma unroll 4
+        for (int j = tid - a * nc; j < g.A; j += nc) {
+            if (j == a) continue;
+            const int b = j > a ? rowa + j : pair_index(j, a, g.A), code = __ldg(&pairs[b].y);
+            const float sgn = j > a ? 1.f : -1.f;
+            float2 r = sR[b], V = sV[code >> 1];
+            const float2 gj = sG[j];
+            r.y *= sgn;
+            V.y *= (code & 1) ? -sgn : sgn;
+            const float pr = r.x * gj.x - r.y * gj.y, pi = r.x * gj.y + r.y * gj.x;
+            zr += pr * V.x + pi * V.y;
+            zi += pi * V.x - pr * V.y;
+        }
+        sZ[tid] = make_float2(zr, zi);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        float m = 0.f;
+        for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, fred[k]);
+        qmax_ft[ft] = m;
+    }
+    antenna_totals<NT>(sZ, g.A, ft, is2, zpart);
+}
+
 // grad_gamma[a][k][c] = sum_{f,t} X_k(nu_f) zpart[f][t][a][c]: one CTA per (a, c); thread
 // j takes the (channel, LST) pairs j, j + GR_THREADS, ... in batches of GR_U independent
 // loads.  Per thread and across a warp (fixed shuffle order) the sums are in the working
@@ -778,12 +955,20 @@ fm_status launch_chi2_chan(Ctx &c, const R *vis, const R *gamma, R *omega, R *zp
         set_error("chi^2 epilogue: %d antennas (at most %d, %zu bytes of shared memory)", c.A, CF_THREADS, smem);
         return FM_ERR_UNSUPPORTED;
     }
-    const bool big = smem > 56 * 1024 && smem <= 208 * 1024;    // the larger CTA's static arrays take up to 17 KB
-    auto *kern = big ? k_chi2_ft<R, CF_BIG> : k_chi2_ft<R, CF_THREADS>;
-    FM_CK(smem_opt_in(kern));
-    kern<<<c.F * c.T, big ? CF_BIG : CF_THREADS, smem, st>>>(c.g, vis, (const R *)c.data, gamma, omega, zpart, chi2p, c.ha.U,
-                                                c.ha.moff, c.ha.mem, groups ? c.ha.q32 : nullptr, c.ha.qmax_ft, rin,
-                                                hv ? *hv : HaVSrc{});
+    if constexpr (std::is_same<R, float>::value)
+        if (groups && (c.A + 3 * (size_t)c.B) * 2 * sizeof(R) > 56 * 1024) {   // fewer than four CTAs of k_chi2_ft an SM
+            const size_t sm = ((size_t)c.A + c.ha.U + c.B) * sizeof(float2);
+            FM_CK(smem_opt_in(k_chi2_group));
+            k_chi2_group<<<c.F * c.T, CG_THREADS, sm, st>>>(c.g, vis, (const float *)c.data, gamma, zpart, chi2p, c.ha.U,
+                                                            c.fg.pairs, c.fg.gmem, c.ha.moff, c.ha.q32, c.ha.qmax_ft, rin,
+                                                            hv ? *hv : HaVSrc{});
+            FM_CK_LAUNCH();
+            return FM_OK;
+        }
+    FM_CK(smem_opt_in(k_chi2_ft<R>));
+    k_chi2_ft<R><<<c.F * c.T, CF_THREADS, smem, st>>>(c.g, vis, (const R *)c.data, gamma, omega, zpart, chi2p, c.ha.U, c.ha.moff,
+                                                      c.ha.mem, groups ? c.ha.q32 : nullptr, c.ha.qmax_ft, rin,
+                                                      hv ? *hv : HaVSrc{});
     FM_CK_LAUNCH();
     return FM_OK;
 }
