@@ -358,7 +358,7 @@ fm_status gd_setup(Ctx &c)
     s.on = false;
     if (const char *e = getenv("FM_HA_GROUPS"))
         if (atoi(e) == 0) return FM_OK;
-    if (c.ha.on || c.hs.on || fg.U > GD_MAX_U) return FM_OK;
+    if ((c.ha.on && !c.mm.on) || c.hs.on || fg.U > GD_MAX_U) return FM_OK;   // with c.mm: the monopole's sum
     const bool f64 = c.prec == FM_PREC_FP64_SIMT;
     if (c.prec >= FM_PREC_BF16X1) return FM_OK;
     if (std::max(gd_fwd_smem<double>(c), f64 ? gd_adj_smem<double>(c) : gd_adj_smem<float>(c)) > 200 * 1024) return FM_OK;

@@ -1612,13 +1612,18 @@ fm_status ha_setup(Ctx &c)
 {
     HaState &s = c.ha;
     s.on = s.drift = false;
-    if (c.prec < FM_PREC_BF16X1) return FM_OK;
+    if (c.prec == FM_PREC_FP64_SIMT) return FM_OK;
     if (const char *e = getenv("FM_HA"))
         if (atoi(e) == 0) return FM_OK;
     const FringeGroups &fg = c.fg;
     s.U = fg.U;
     s.nmt = (s.U + 63) / 64;
     s.nkq = (s.U + 31) / 32;
+    if (c.prec == FM_PREC_FP32_SIMT) {       // in hour-angle modes, for what the per-baseline sums take
+        if (simt_supports<float>(c, false) != FM_OK || simt_supports<float>(c, true) != FM_OK) return FM_OK;
+        FM_TRY(mm_setup(c));
+        return c.mm.on ? ha_of_modes(c) : FM_OK;
+    }
     std::vector<int> ncontrib;
     const bool fits = ha_geometry(c, ncontrib);
     // the x1 precisions keep the rounding of their products; what has neither this form nor the antenna form

@@ -661,7 +661,7 @@ fm_status hs_fwd_launch(Ctx &c, const HsDev &h, const R *x, cudaStream_t st)
 fm_status hs_setup(Ctx &c)
 {
     c.hs.on = false;
-    if (c.prec >= FM_PREC_BF16X1 || !c.fg.drift) return FM_OK;
+    if (c.prec >= FM_PREC_BF16X1 || c.ha.on || !c.fg.drift) return FM_OK;
     return c.prec == FM_PREC_FP64_SIMT ? hs_setup_t<double>(c) : hs_setup_t<float>(c);
 }
 

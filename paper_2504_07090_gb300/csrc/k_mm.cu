@@ -24,6 +24,8 @@
 // TB/s), adjoint 188 -> 43 us (k_mm_adj 28); LSTs off the grid (12 of them): 10.02 ms -> 82 us; 127 antennas, 128
 // channels, 120 LSTs: 7.26 -> 0.61 ms (k_mm_fwd 477 us, 3.1 GB at 6.5 TB/s) and 4.98 -> 0.65 ms.  The errors against 64 bits fall to
 // those of the mode transforms (V of 7 antennas 1.3e-6 -> 2.6e-7).
+// FP32 handles: 37 antennas, 64 channels, 60 LSTs, chi^2 and gradient 3.13 ms (each distinct fringe on the CUDA
+// cores, k_hs.cu) -> 0.27 ms; gradient against 64 bits 1.2e-7 in the mean of 14 geometries, as before.
 #include <algorithm>
 #include <cmath>
 #include <vector>
