@@ -232,6 +232,8 @@ struct MmState {
     float *Y = nullptr, *G = nullptr; // [sky][F][D][ld] modes of the sky, [F][D][ld] of the gradient
     double *b64 = nullptr;            // [ld][M] RA basis in modes
     float *b32 = nullptr, *pix = nullptr;   // the same in FP32; [ld][R] of single pixels
+    int nf = 0;                       // rows of fac
+    float2 *fac = nullptr;            // [nf][wmax] conj(f): the LSTs' phasors of a band, E^H E = f f^H (mass matrix)
     float *tmp = nullptr;             // [F][ld][N] when the transform runs on the CUDA cores
     RaBasis ra;
 };
@@ -559,6 +561,7 @@ fm_status mm_setup(Ctx &c);
 fm_status mm_group_monopole(Ctx &c, float *ug);
 fm_status launch_mm_forward(Ctx &c, int nsky, int slot_rows, int N, float *vpart, cudaStream_t st);
 fm_status launch_mm_adjoint(Ctx &c, const float *q32, cudaStream_t st);
+fm_status launch_mm_maps(Ctx &c, int f, int j0, int nj, const float *W, float *X, cudaStream_t st);
 fm_status launch_mm_from_modes(Ctx &c, const float *a, int slot, cudaStream_t st, int skip_dc);
 fm_status launch_mm_from_pixels(Ctx &c, const float *x, int slot, cudaStream_t st);
 fm_status launch_mm_to_modes(Ctx &c, float *abar, cudaStream_t st);

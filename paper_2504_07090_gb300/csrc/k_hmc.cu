@@ -799,7 +799,19 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     // baseline groups (once per handle)
     if (!c.pc_grp) {
         std::vector<int> rep, off, mem;
-        pc_groups(c, rep, off, mem);
+        if (c.mm.on) {                       // the groups of the forms (k_hs.cu)
+            off.resize(c.fg.U + 1);
+            mem.resize(c.B);
+            FM_CK(cudaMemcpy(off.data(), c.fg.moff, sizeof(int) * off.size(), cudaMemcpyDeviceToHost));
+            FM_CK(cudaMemcpy(mem.data(), c.fg.mem, sizeof(int) * mem.size(), cudaMemcpyDeviceToHost));
+            for (int &m : mem) m >>= 1;
+            for (int u = 0; u < c.fg.U; ++u) {
+                rep.push_back(c.fg.ant_of[c.fg.rep_i[u]]);
+                rep.push_back(c.fg.ant_of[c.fg.rep_j[u]]);
+            }
+        } else {
+            pc_groups(c, rep, off, mem);
+        }
         c.pc_U = (int)off.size() - 1;
         std::vector<int> all(rep);
         all.insert(all.end(), off.begin(), off.end());
@@ -819,9 +831,12 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     // Drift scans: the channel's cell image serves every LST (PcCells), up to GR_CHAINS chains of four
     // LSTs a launch so that the 2 U TB maps fill whole waves of two CTAs an SM (504 maps leave the second
     // of two waves a third full, 1512 take five full ones) within 128 MB of results.
-    bool cells = tcx && c.fg.drift;
+    // Handles in hour-angle modes: fewer maps than LSTs serve the sum over LSTs (k_mm_maps)
+    const bool modes = tcx && c.mm.on && c.mm.ra.img && 4 * c.mm.nf <= 3 * c.T;
+    const int nT = modes ? c.mm.nf : c.T;
+    bool cells = tcx && c.fg.drift && !modes;
     PcCells pc{};
-    const int chain_t = tcx ? (c.T < 4 ? c.T : 4) : 1;            // LSTs of one FP32 Gram sum
+    const int chain_t = tcx ? (nT < 4 ? nT : 4) : 1;              // LSTs of one FP32 Gram sum
     int TB = chain_t;
     if (cells) {
         pc.q = c.fg.q;
@@ -836,17 +851,17 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
         const size_t img = (size_t)U * c.D * pc.ld;
         cells = img <= (size_t)U * c.npix * 4 || img * 2 * sizeof(R) <= (size_t)1 << 30;
     }
-    if (cells) {
+    if (cells || modes) {
         const long long maps = 2LL * U * cdiv(c.M, 128), slots = 2 * 152;
         double best = 0.0;
-        for (int k = 1; k <= GR_CHAINS && (k - 1) * chain_t < c.T; ++k) {
-            const int tb = std::min(k * chain_t, c.T);
+        for (int k = 1; k <= GR_CHAINS && (k - 1) * chain_t < nT; ++k) {
+            const int tb = std::min(k * chain_t, nT);
             if (k > 1 && 2.0 * U * tb * c.nk * sizeof(R) > 128e6) break;
             const double fill = (double)(maps * tb) / (double)(cdiv(maps * tb, slots) * slots);
             if (fill > best + 0.02) { best = fill; TB = tb; }
         }
     }
-    size_t nX = cells ? 2 * (size_t)U * c.D * pc.ld : 2 * (size_t)U * c.npix * TB, nQ = tcx ? 0 : 2 * (size_t)U * c.D * c.M, nS = 2 * (size_t)U * c.nk * TB;
+    size_t nX = cells ? 2 * (size_t)U * c.D * pc.ld : 2 * (size_t)U * (modes ? (size_t)c.D * c.mm.ld : c.npix) * TB, nQ = tcx ? 0 : 2 * (size_t)U * c.D * c.M, nS = 2 * (size_t)U * c.nk * TB;
     // (counts rounded up to even so that the FP64 scratch after them stays 8-byte aligned)
     size_t nG = ((size_t)c.nk * bs + 1) & ~(size_t)1, nW = ((size_t)c.F * U + 1) & ~(size_t)1;
     R *X = nullptr;
@@ -897,9 +912,11 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                     k_pc_cells<<<dim3(std::max(1u, std::min(cdiv((long long)c.D * pc.ld, 256), 4864u / U)), U), 256, 0, st>>>(
                         c.g, pc, f, U, g_rep, Wg, X, xmax);
                 }
-            for (int t = 0; t < c.T; t += TB) {
-                const int tbn = c.T - t < TB ? c.T - t : TB;
-                if (!cells)
+            for (int t = 0; t < nT; t += TB) {
+                const int tbn = nT - t < TB ? nT - t : TB;
+                if constexpr (std::is_same<R, float>::value)
+                    if (modes && (rc = launch_mm_maps(c, f, t, tbn, Wg, X, st)) != FM_OK) break;
+                if (!cells && !modes)
                     for (int tb = 0; tb < tbn; ++tb)
                         k_pc_fringe<R><<<2048, 256, 0, st>>>(c.g, f, t + tb, U, g_rep, Wg, X + (size_t)tb * 2 * U * c.npix);
                 if (cudaGetLastError() != cudaSuccess) { rc = FM_ERR_CUDA; break; }
@@ -919,7 +936,8 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                 } else if (tcx) {
                     // S[tb,pl,b][m][n] = sum_{d,r} Phi[r][m] X[tb,pl,b][d][r] P[d][n]: the tensor-core
                     // pixel -> mode transform over the 2U response maps of tbn LSTs
-                    if ((rc = launch_modes_tc_adjoint_maps(c, (const float *)X, 2 * U * tbn, (float *)S, st)) != FM_OK)
+                    if ((rc = launch_modes_tc_adjoint_maps(c, (const float *)X, 2 * U * tbn, (float *)S, st, nullptr,
+                                                           modes ? &c.mm.ra : nullptr)) != FM_OK)
                         break;
                 } else {
                     // Q[pl,b][d][m] = sum_r X[pl,b][d][r] Phi[r][m]

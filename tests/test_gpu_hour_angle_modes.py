@@ -60,3 +60,26 @@ def test_hour_angle_modes_match_fp64(name, prec, monkeypatch):
     for k in a:
         err = float((a[k] - b[k]).norm() / b[k].norm())
         assert err < (1e-5 if k in ("V", "Vx") else 1e-4), (k, err)
+
+
+# The mass matrix from fewer maps than LSTs against the responses of every LST: both form FP32 responses from FP16
+# split transforms and agree to 2e-6 (the bound of the drift-scan cell image's test).
+@pytest.mark.parametrize("name", ["half", "one_dec", "lst70", "offgrid16", "uneven", "wide_lst"])
+@pytest.mark.parametrize("block", [64, 1])
+def test_mass_matrix_from_hour_angle_maps(name, block, monkeypatch):
+    import torch
+    from paper_2504_07090_gb300 import fm
+    p = _problem(name)
+    tr = synth.draw_truth(p)
+    mu, lam = (torch.tensor(a.astype(np.float32), device="cuda") for a in synth.prior_for(p, tr.theta))
+    got = []
+    for ha in ("1", "0"):
+        monkeypatch.setenv("FM_HA", ha)
+        h = fm.ForwardModel(p, "fp16x3", sigma=50.0)
+        th = torch.tensor(tr.theta.astype(np.float32), device="cuda")
+        h.set_data(torch.tensor(synth.random_data(p, 1e3, 7).astype(np.float32), device="cuda"))
+        h.set_prior(mu, lam)
+        h.build_precond(th, block)
+        got.append(h.precond_blocks().cpu().numpy()[: p.n_sky_params * block])
+        h.close()
+    assert np.linalg.norm(got[0] - got[1]) < 2e-6 * np.linalg.norm(got[1])
