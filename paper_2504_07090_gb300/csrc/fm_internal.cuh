@@ -455,7 +455,7 @@ fm_status launch_gain_reduce(Ctx &c, const R *zpart, R *grad_gain, cudaStream_t 
 struct HaVSrc {
     const float *vpart = nullptr;    // [nmt F][J][npad][128]
     const int *ncontrib = nullptr;   // [nmt F]
-    const int *bmap = nullptr;       // [B] 2 u + reversed
+    const int2 *pairs = nullptr;     // [B] i | j << 16, 2 u + reversed
     const unsigned *xmax = nullptr;  // [F]
     const float *dc = nullptr;
     long long dcs = 0;

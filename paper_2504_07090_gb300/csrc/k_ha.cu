@@ -1788,7 +1788,7 @@ bool ha_vsrc(const Ctx &c, const float *dc, long long dcs, HaVSrc &v)
         if (atoi(e) == 0) return false;
     v.vpart = s.vpart;
     v.ncontrib = s.ncontrib;
-    v.bmap = s.bmap;
+    v.pairs = c.fg.pairs;
     v.xmax = s.xmax;
     v.dc = dc;
     v.dcs = dcs;

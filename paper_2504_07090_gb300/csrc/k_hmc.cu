@@ -286,7 +286,7 @@ __global__ void k_pc_accum(long long n, const R *__restrict__ G, double *__restr
 // 16-byte shared-memory reads a row.  Rows arrive GR_ROWS a chain at a time by cp.async, two stages; a row
 // keeps 4 words of padding after its first half, which puts the eight 8-word tiles of a row into
 // different banks.  Bound: FP32 multiply-adds (and the shared-memory reads, at the same rate).
-constexpr int GR_ROWS = 8, GR_TILES = 36, GR_CHAINS = 4, GR_LD = 68;
+constexpr int GR_ROWS = 8, GR_TILES = 36, GR_CHAINS = 8, GR_LD = 68;
 
 constexpr int gram_threads(int chains) { return (chains * GR_TILES + 31) / 32 * 32; }
 constexpr int gram_smem(int chains)
@@ -828,7 +828,7 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     // route only), S [TB][2][U][nk], G [nk/bs][bs][bs], group weights W [F][U].  The tensor-core
     // transform takes TB LSTs' response maps per launch.
     const bool tcx = std::is_same<R, float>::value && c.mtc.on;
-    // Drift scans: the channel's cell image serves every LST (PcCells), up to GR_CHAINS chains of four
+    // Drift scans: the channel's cell image serves every LST (PcCells), up to four chains of four
     // LSTs a launch so that the 2 U TB maps fill whole waves of two CTAs an SM (504 maps leave the second
     // of two waves a third full, 1512 take five full ones) within 128 MB of results.
     // Handles in hour-angle modes: fewer maps than LSTs serve the sum over LSTs (k_mm_maps)
@@ -836,7 +836,9 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     const int nT = modes ? c.mm.nf : c.T;
     bool cells = tcx && c.fg.drift && !modes;
     PcCells pc{};
-    const int chain_t = tcx ? (nT < 4 ? nT : 4) : 1;              // LSTs of one FP32 Gram sum
+    // LSTs of one FP32 Gram sum, and most sums a launch: hour-angle maps come a few a channel, and the more chains
+    // a CTA of the Gram holds the more warps an SM has (two of four maps: 86 us a launch)
+    const int chain_t = !tcx ? 1 : std::min(nT, modes ? std::max(1, std::min(4, 64 / (2 * U))) : 4), chains = modes ? GR_CHAINS : 4;
     int TB = chain_t;
     if (cells) {
         pc.q = c.fg.q;
@@ -854,7 +856,7 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     if (cells || modes) {
         const long long maps = 2LL * U * cdiv(c.M, 128), slots = 2 * 152;
         double best = 0.0;
-        for (int k = 1; k <= GR_CHAINS && (k - 1) * chain_t < nT; ++k) {
+        for (int k = 1; k <= chains && (k - 1) * chain_t < nT && k * chain_t <= 16; ++k) {
             const int tb = std::min(k * chain_t, nT);
             if (k > 1 && 2.0 * U * tb * c.nk * sizeof(R) > 128e6) break;
             const double fill = (double)(maps * tb) / (double)(cdiv(maps * tb, slots) * slots);

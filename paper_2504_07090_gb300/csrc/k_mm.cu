@@ -350,15 +350,18 @@ __global__ void __launch_bounds__(256) k_mm_vis(int F, int T, int U, int mlo, in
     const int seg = blockIdx.x, f = seg % F, mt = seg / F, tid = threadIdx.x;
     const int tb = blockIdx.y * MM_TC, nt = min(MM_TC, T - tb);
     const float2 *zz = z + blockIdx.z * zs;
-    for (int e = tid; e < w4 * 64; e += 256) {
-        const int c = e < wmax * 64 ? code[(size_t)seg * wmax * 64 + e] : -1;
-        float2 v = make_float2(0.f, 0.f);
-        if (c >= 0) {
-            v = zz[c >> 1];
-            if (c & 1) v.y = -v.y;
-        }
-        sz[e] = v;
+    for (int e0 = tid; e0 < w4 * 64; e0 += 4 * 256) {            // four gathers in flight
+        int c[4];
+        float2 v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) c[r] = e0 + 256 * r < wmax * 64 ? code[(size_t)seg * wmax * 64 + e0 + 256 * r] : -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = c[r] >= 0 ? zz[c[r] >> 1] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (e0 + 256 * r < w4 * 64) sz[e0 + 256 * r] = make_float2(v[r].x, (c[r] & 1) ? -v[r].y : v[r].y);
     }
+#pragma unroll 4
     for (int e = tid; e < MM_TC * pw; e += 256) sp[e] = e < nt * pw ? ph[(size_t)tb * pw + e] : make_float2(0.f, 0.f);
     __syncthreads();
     const int ul = tid & 63, u = mt * 64 + ul, tl = tid >> 6;
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(256) k_mm_vis(int F, int T, int U, int mlo, in
 // ------------------------------------------------------------ adjoint
 // w_e of every element from the group sums Q_u(t): sum_t conj(Q_u(t)) e^{2 pi i m tau_t / L}, conjugated for
 // the conjugated elements.  CTA = (channel, 8 groups), one warp a group, lanes over the modes of its band, so
-// that the phasors are read in a row; Q is staged MM_QT LSTs at a time and the phasors of five LSTs are in
+// that the phasors are read in a row; Q is staged MM_QT LSTs at a time and the phasors of ten LSTs are in
 // flight.  (Lanes over groups, four modes each, gathered 32 phasors a load: 27 us at 37 antennas, 64 channels,
 // 60 LSTs; Q read word by word from L2: 20 us.)
 constexpr int MM_QT = 60;
@@ -419,16 +422,16 @@ __global__ void __launch_bounds__(256) k_mm_q(int T, int U, int mlo, int pw, int
             }
             __syncthreads();
             if (!one) continue;
-            for (int t = 0; t < nt; t += 5) {
-                float2 x[5], y[5];
+            for (int t = 0; t < nt; t += 10) {
+                float2 x[10], y[10];
 #pragma unroll
-                for (int r = 0; r < 5; ++r) {
+                for (int r = 0; r < 10; ++r) {
                     const float2 *p = pm + (size_t)(tb + min(t + r, nt - 1)) * pw;
                     x[r] = __ldg(p);
                     y[r] = two ? __ldg(p + 32) : make_float2(0.f, 0.f);
                 }
 #pragma unroll
-                for (int r = 0; r < 5; ++r) {
+                for (int r = 0; r < 10; ++r) {
                     const float2 v = sq[t + r][uw];           // zero past the last LST
                     a.x += v.x * x[r].x + v.y * x[r].y;       // conj(Q) e^{...}
                     a.y += v.x * x[r].y - v.y * x[r].x;
@@ -447,7 +450,7 @@ __global__ void __launch_bounds__(256) k_mm_q(int T, int U, int mlo, int pw, int
         }
     }
 }
-static_assert(MM_QT % 5 == 0, "k_mm_q reads LSTs in fives");
+static_assert(MM_QT % 10 == 0, "k_mm_q reads LSTs in tens");
 
 // G[f][d][2 m] = Re, [2 m + 1] = -Im of X(m, d) = sum over the elements of |m| of c_e(d) w_e: one warp per
 // (channel, m, 32 pairs of declinations), eight 16-byte loads of the table in flight a lane.  The channels run
@@ -600,9 +603,11 @@ int mm_window(const Ctx &c, const std::vector<double> &bcoef, const std::vector<
         const double za = sU > 0.0 ? std::acos(sU > 1.0 ? 1.0 : sU) : 0.5 * kPi;   // the step at the horizon
         return domega[d] * std::exp(bc * za * za);
     };
+    // the beam falls with |H|: its maximum in use is at the cell nearest the meridian
+    const double n0 = (c.R - 1) * q + 0.5 * q + (c.cfg.ra_min - lst0) / dh;
+    const int at = (int)std::fmin(std::fmax(std::rint(n0), 0.0), nh - 1.0);
     double top = 0.0;
-    for (int d = 0; d < c.D; ++d)
-        for (int n = 0; n < nh; ++n) top = std::fmax(top, weight(d, n));
+    for (int d = 0; d < c.D; ++d) top = std::fmax(top, weight(d, at));
     for (int L = nh + (nh & 1); L <= 2 * nh + 64 && L <= MM_MAXL && L * dh <= 2.0 * kPi; L += 2) {
         if (!smooth_factors(L, p)) continue;
         const int p0 = (L - nh) / 2;

@@ -511,45 +511,27 @@ __device__ __forceinline__ float2 hv_row(const HaVSrc &hv, int f, int t, int u)
     return a;
 }
 
-// sS[row], row < 128 nmt: the contributors' partial rows of the forward at LST t of channel f, in rank
-// order; sc and cf: the scale of the sum and the monopole's coefficient
+// sV[u]: V of every group at LST t of channel f, with the roundings of k_ha_vfinish, so that a member's value
+// (sV[u], conjugated when reversed) equals the finished forward's bitwise
 template <int NT>
-__device__ __forceinline__ void hv_rows(const HaVSrc &hv, int f, int t, float *sS, float &sc, float &cf)
+__device__ __forceinline__ void group_vis(const HaVSrc &hv, int f, int t, int ft, int U, float2 *sV)
 {
-    for (int e = threadIdx.x; e < hv.nmt * 128; e += NT) {
-        const int seg = (e >> 7) * hv.F + f, row = e & 127, nc = hv.ncontrib[seg];
-        // the contributors' rows in rank order, four loads ahead
-        const float *src = hv.vpart + ((size_t)seg * hv.J * hv.npad + t) * 128 + row;
-        const size_t js = (size_t)hv.npad * 128;
-        float a = 0.f;
-        for (int j0 = 0; j0 < nc; j0 += 4) {
-            float v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = j0 + u < nc ? src[(size_t)(j0 + u) * js] : 0.f;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (j0 + u < nc) a += v[u];
+    const float sc = hv_scale(hv, f), cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
+    for (int u = threadIdx.x; u < U; u += NT) {
+        const float2 v = hv_row(hv, f, t, u);
+        float2 V = make_float2(__fmul_rn(v.x, sc), __fmul_rn(v.y, sc));
+        if (hv.dc) {
+            const float2 m = reinterpret_cast<const float2 *>(hv.ug)[(size_t)ft * U + u];
+            V = make_float2(__fmaf_rn(cf, m.x, V.x), __fmaf_rn(cf, m.y, V.y));
         }
-        sS[e] = a;
+        sV[u] = V;
     }
-    sc = hv_scale(hv, f);
-    cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
 }
 
-// V of a baseline with code = 2 u + reversed, with the roundings of k_ha_vfinish, so that it equals the
-// finished forward's bitwise
-__device__ __forceinline__ float2 hv_value(const HaVSrc &hv, const float *sS, size_t ft, int U, int code, float sc,
-                                           float cf)
+__device__ __forceinline__ float2 member_vis(const float2 *sV, int code)
 {
-    const int u = code >> 1, row = 128 * (u >> 6) + 2 * (u & 63);
-    const float sgn = (code & 1) ? -1.f : 1.f;
-    float vx = __fmul_rn(sS[row], sc), vy = __fmul_rn(sgn * sS[row + 1], sc);
-    if (hv.dc) {
-        const float2 u2 = reinterpret_cast<const float2 *>(hv.ug)[ft * U + u];
-        vx = __fmaf_rn(cf, u2.x, vx);
-        vy = __fmaf_rn(cf, sgn * u2.y, vy);
-    }
-    return make_float2(vx, vy);
+    const float2 v = sV[code >> 1];
+    return make_float2(v.x, (code & 1) ? -v.y : v.y);
 }
 
 // q32[ft][u] = the groups' sums of sW (conjugated for reversed members); returns the largest |Re|, |Im| that
@@ -653,7 +635,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     C2 *sTi = sG + g.A;                                    // [B] term of baseline (i, j) in Z_i
     C2 *sTj = sTi + g.B;                                   // [B] term of baseline (i, j) in Z_j
     C2 *sW = sTj + g.B;                                    // [B] omega (hour-angle form)
-    float *sS = reinterpret_cast<float *>(sW + g.B);       // [nmt][128] forward partial sums (hv)
+    float2 *sV = reinterpret_cast<float2 *>(sW + g.B);     // [U] V of the groups (hv)
     __shared__ C2 sZ[NT];                          // chunk sums of Z_a
     __shared__ double dred[NT / 32];
     __shared__ float fred[NT / 32];
@@ -670,8 +652,7 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
             sG[i].y = im;
         }
     }
-    float hsc = 0.f, hcf = 0.f;
-    if (hv.vpart) hv_rows<NT>(hv, f, ft - f * g.T, sS, hsc, hcf);
+    if (hv.vpart) group_vis<NT>(hv, f, ft - f * g.T, ft, U, sV);
     __syncthreads();
     const R is2 = (R)g.inv_sigma2;
     const C2 *vrow = vis ? reinterpret_cast<const C2 *>(vis) + (size_t)ft * g.B : nullptr;
@@ -681,13 +662,18 @@ __global__ void __launch_bounds__(CF_THREADS, sizeof(R) == 4 ? 8 : 1) k_chi2_ft(
     C2 *orow = reinterpret_cast<C2 *>(omega) + (size_t)ft * g.B;
     R c2 = 0;   // a warp's terms in the working type; FP64 across warps
     for (int b = tid; b < g.B; b += NT) {
-        const int i = g.bl_i[b], j = g.bl_j[b];
+        int i, j;
         C2 V;
         if (hv.vpart) {
-            const float2 v = hv_value(hv, sS, (size_t)ft, U, hv.bmap[b], hsc, hcf);
+            const int2 pr = __ldg(hv.pairs + b);
+            i = pr.x & 0xffff;
+            j = pr.x >> 16;
+            const float2 v = member_vis(sV, pr.y);
             V.x = (R)v.x;
             V.y = (R)v.y;
         } else {
+            i = g.bl_i[b];
+            j = g.bl_j[b];
             V = vrow[b];
         }
         const C2 d = drow[b], gi = sG[i], gj = sG[j];
@@ -780,16 +766,7 @@ k_chi2_group(DevGeom g, const float *__restrict__ vis, const float *__restrict__
         }
     }
     if (hv.vpart) {
-        const float sc = hv_scale(hv, f), cf = hv.dc ? hv.dc[(size_t)f * hv.dcs] : 0.f;
-        for (int u = tid; u < U; u += NT) {                // with the roundings of k_ha_vfinish
-            const float2 v = hv_row(hv, f, t, u);
-            float2 V = make_float2(__fmul_rn(v.x, sc), __fmul_rn(v.y, sc));
-            if (hv.dc) {
-                const float2 m = reinterpret_cast<const float2 *>(hv.ug)[(size_t)ft * U + u];
-                V = make_float2(__fmaf_rn(cf, m.x, V.x), __fmaf_rn(cf, m.y, V.y));
-            }
-            sV[u] = V;
-        }
+        group_vis<NT>(hv, f, t, ft, U, sV);
     } else {
         const float2 *vrow = reinterpret_cast<const float2 *>(vis) + (size_t)ft * g.B;
         for (int u = tid; u < U; u += NT) {                // the first member's
@@ -1069,7 +1046,7 @@ __global__ void __launch_bounds__(CF_THREADS, 6) k_hvp_ft(DevGeom g, const float
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *sG = reinterpret_cast<float2 *>(smem_raw), *sD = sG + g.A;       // [A] gains and tangents
     float2 *sTi = sD + g.A, *sTj = sTi + g.B, *sW = sTj + g.B;               // [B]
-    float *sS = reinterpret_cast<float *>(sW + g.B), *sS2 = sS + 128 * hv.nmt;
+    float2 *sV = sW + g.B, *sdV = sV + 64 * hv.nmt;                          // [U] V and dV of the groups
     __shared__ float2 sZ[CF_THREADS];
     __shared__ float fred[CF_THREADS / 32];
     const int ft = blockIdx.x, f = ft / g.T, tid = threadIdx.x, lane = tid & 31;
@@ -1083,9 +1060,8 @@ __global__ void __launch_bounds__(CF_THREADS, 6) k_hvp_ft(DevGeom g, const float
         }
         sG[i] = make_float2(re, im);
     }
-    float sc, cf, dsc, dcf;
-    hv_rows<CF_THREADS>(hv, f, ft - f * g.T, sS, sc, cf);
-    hv_rows<CF_THREADS>(hd, f, ft - f * g.T, sS2, dsc, dcf);
+    group_vis<CF_THREADS>(hv, f, ft - f * g.T, ft, U, sV);
+    group_vis<CF_THREADS>(hd, f, ft - f * g.T, ft, U, sdV);
     __syncthreads();
     const float is2 = (float)g.inv_sigma2;
     auto mul = [](float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); };
@@ -1093,9 +1069,10 @@ __global__ void __launch_bounds__(CF_THREADS, 6) k_hvp_ft(DevGeom g, const float
     auto add = [](float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); };
     const float2 *drow = reinterpret_cast<const float2 *>(data) + (size_t)ft * g.B;
     for (int b = tid; b < g.B; b += CF_THREADS) {
-        const int code = hv.bmap[b];
-        const float2 gi = sG[g.bl_i[b]], gj = sG[g.bl_j[b]], di = sD[g.bl_i[b]], dj = sD[g.bl_j[b]];
-        const float2 V = hv_value(hv, sS, (size_t)ft, U, code, sc, cf), dV = hv_value(hd, sS2, (size_t)ft, U, code, dsc, dcf);
+        const int2 pr = __ldg(hv.pairs + b);
+        const int i = pr.x & 0xffff, j = pr.x >> 16;
+        const float2 gi = sG[i], gj = sG[j], di = sD[i], dj = sD[j];
+        const float2 V = member_vis(sV, pr.y), dV = member_vis(sdV, pr.y);
         const float2 gg = mulc(gi, gj);
         const float2 dm = add(mul(add(mulc(di, gj), mulc(gi, dj)), V), mul(gg, dV));
         float2 om = mulc(dm, gg);
