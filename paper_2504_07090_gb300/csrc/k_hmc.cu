@@ -281,12 +281,13 @@ __global__ void k_pc_accum(long long n, const R *__restrict__ G, double *__restr
 
 // acc64[j0][c][c'] += sum over rows of S[row][64 j0 + c] S[row][64 j0 + c'], one CTA per 64-block.  The
 // rows form chains of `chain` rows (a few LSTs' responses): a chain's sum is one FP32 multiply-add
-// sequence in row order, the chains join the FP64 total in order.  Thread (tile, chain) holds one of the 36
+// sequence in row order, the chains join the FP64 total in order, `per` of them (four LSTs' responses) added
+// in FP32 first (FP64 conversions and adds run at 2 lanes per SM and clock).  Thread (tile, chain) holds one of the 36
 // 8 x 8 tiles with c >= c' (the block is symmetric): 64 accumulators as 32 packed pairs against four
 // 16-byte shared-memory reads a row.  Rows arrive GR_ROWS a chain at a time by cp.async, two stages; a row
 // keeps 4 words of padding after its first half, which puts the eight 8-word tiles of a row into
 // different banks.  Bound: FP32 multiply-adds (and the shared-memory reads, at the same rate).
-constexpr int GR_ROWS = 8, GR_TILES = 36, GR_CHAINS = 8, GR_LD = 68;
+constexpr int GR_ROWS = 16, GR_TILES = 36, GR_CHAINS = 9, GR_LD = 68;
 
 constexpr int gram_threads(int chains) { return (chains * GR_TILES + 31) / 32 * 32; }
 constexpr int gram_smem(int chains)
@@ -295,7 +296,7 @@ constexpr int gram_smem(int chains)
     return stages > tiles ? stages : tiles;
 }
 
-__global__ void __launch_bounds__(gram_threads(GR_CHAINS)) k_pc_gram(int rows, int chain, int nk,
+__global__ void __launch_bounds__(gram_threads(GR_CHAINS)) k_pc_gram(int rows, int chain, int per, int nk,
                                                                      const float *__restrict__ S,
                                                                      double *__restrict__ acc64)
 {
@@ -368,7 +369,11 @@ __global__ void __launch_bounds__(gram_threads(GR_CHAINS)) k_pc_gram(int rows, i
         const int th = hi >> 3, tl = lo >> 3;
         const float *o = st + (size_t)(th * (th + 1) / 2 + tl) * 64 + 8 * (hi & 7) + (lo & 7);
         double a = out[e];
-        for (int k = 0; k < nch; ++k) a += (double)o[(size_t)k * GR_TILES * 64];
+        for (int k = 0; k < nch; k += per) {
+            float v = o[(size_t)k * GR_TILES * 64];
+            for (int i = k + 1; i < min(k + per, nch); ++i) v += o[(size_t)i * GR_TILES * 64];
+            a += (double)v;
+        }
         out[e] = a;
     }
 }
@@ -837,7 +842,8 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
     bool cells = tcx && c.fg.drift && !modes;
     PcCells pc{};
     // LSTs of one FP32 Gram sum, and most sums a launch: hour-angle maps come a few a channel, and the more chains
-    // a CTA of the Gram holds the more warps an SM has (two of four maps: 86 us a launch)
+    // a CTA of the Gram holds the more warps an SM has (17 maps in launches of nine chains of one: 11.1 -> 8.6 ms
+    // against two chains of four, 37 antennas, 64 channels)
     const int chain_t = !tcx ? 1 : std::min(nT, modes ? std::max(1, std::min(4, 64 / (2 * U))) : 4), chains = modes ? GR_CHAINS : 4;
     int TB = chain_t;
     if (cells) {
@@ -853,10 +859,15 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
         const size_t img = (size_t)U * c.D * pc.ld;
         cells = img <= (size_t)U * c.npix * 4 || img * 2 * sizeof(R) <= (size_t)1 << 30;
     }
-    if (cells || modes) {
+    if (modes) {                       // equal launches, within 256 MB of results
+        const long long fit = (long long)(256e6 / (2.0 * U * c.nk * sizeof(R))) / chain_t;
+        const int most = (int)std::max(1LL, std::min({(long long)chains, 16LL / chain_t, fit})) * chain_t;
+        TB = (int)cdiv(cdiv(nT, cdiv(nT, most)), chain_t) * chain_t;
+    }
+    if (cells) {
         const long long maps = 2LL * U * cdiv(c.M, 128), slots = 2 * 152;
         double best = 0.0;
-        for (int k = 1; k <= chains && (k - 1) * chain_t < nT && k * chain_t <= 16; ++k) {
+        for (int k = 1; k <= chains && (k - 1) * chain_t < nT; ++k) {
             const int tb = std::min(k * chain_t, nT);
             if (k > 1 && 2.0 * U * tb * c.nk * sizeof(R) > 128e6) break;
             const double fill = (double)(maps * tb) / (double)(cdiv(maps * tb, slots) * slots);
@@ -954,7 +965,7 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                 if (bs > 1 && std::is_same<R, float>::value) {
                     const int nch = (int)cdiv(tbn, chain_t);
                     k_pc_gram<<<(unsigned)(c.nk / 64), gram_threads(nch), gram_smem(nch), st>>>(
-                        2 * U * tbn, 2 * U * chain_t, c.nk, (const float *)S, accf);
+                        2 * U * tbn, 2 * U * chain_t, std::max(1, 4 / chain_t), c.nk, (const float *)S, accf);
                 } else if (bs > 1) {
                     // G[j0][c][c'] = sum_{tb,pl,b} S[tb,pl,b][j0*bs+c] S[tb,pl,b][j0*bs+c']
                     GemmArgsH q3{bs, bs, 2 * U * tbn, bs, 1, c.nk, bs, c.nk, 1, (long long)bs * bs, bs, 1};
