@@ -452,19 +452,21 @@ __global__ void __launch_bounds__(256) k_mm_q(int T, int U, int mlo, int pw, int
 }
 static_assert(MM_QT % 10 == 0, "k_mm_q reads LSTs in tens");
 
-// G[f][d][2 m] = Re, [2 m + 1] = -Im of X(m, d) = sum over the elements of |m| of c_e(d) w_e: one warp per
-// (channel, m, 32 pairs of declinations), eight 16-byte loads of the table in flight a lane.  The channels run
-// against the forward's order, so that what the forward read last is still in L2.
+// G[f][d][2 m] = Re, [2 m + 1] = -Im of X(m, d) = sum over the elements of |m| of c_e(d) w_e: two warps per
+// (channel, m, 32 pairs of declinations), one for each half of the elements (their numbers differ tenfold between
+// modes, and with one warp each the longest ran alone at the end: 27.7 -> 26.0 us for 37 antennas), eight 16-byte loads of the table in flight a
+// lane.  The channels run against the forward's order, so that what the forward read last is still in L2.
 __global__ void __launch_bounds__(256) k_mm_adj(int F, int D, int nm, int ld, const int *__restrict__ moff,
                                                 const float4 *__restrict__ tab, const float2 *__restrict__ w,
                                                 float *__restrict__ G)
 {
+    __shared__ float4 half[4][32];
     const int np = (D + 1) / 2, nchunk = (np + 31) / 32, nmc = ld / 2;
-    const int wi = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int wl = threadIdx.x >> 5, second = wl >> 2, lane = threadIdx.x & 31;
+    const int wi = blockIdx.x * 4 + (wl & 3);
     const int m = wi % nmc, fc = wi / nmc, ch = fc % nchunk, f = F - 1 - fc / nchunk;
-    if (f < 0) return;
     const int i = ch * 32 + lane;
-    if (i >= np) return;
+    const bool on = f >= 0 && i < np;
     float2 re = make_float2(0.f, 0.f), im = re;
     auto add = [&](const float4 &c, const float2 &x) {
         const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
@@ -472,9 +474,10 @@ __global__ void __launch_bounds__(256) k_mm_adj(int F, int D, int nm, int ld, co
         re = __ffma2_rn(ci, ny, __ffma2_rn(cr, wx, re));
         im = __ffma2_rn(ci, wx, __ffma2_rn(cr, wy, im));
     };
-    if (m < nm) {
-        const int e1 = moff[f * (nm + 1) + m + 1];
-        int e = moff[f * (nm + 1) + m];
+    if (on && m < nm) {
+        const int e0 = moff[f * (nm + 1) + m], e2 = moff[f * (nm + 1) + m + 1], mid = e0 + (e2 - e0 + 1) / 2;
+        const int e1 = second ? e2 : mid;
+        int e = second ? mid : e0;
         const float4 *tp = tab + (size_t)e * np + i;
         const float2 *wp = w + e;
         for (; e + 8 <= e1; e += 8, tp += (size_t)8 * np, wp += 8) {
@@ -485,24 +488,28 @@ __global__ void __launch_bounds__(256) k_mm_adj(int F, int D, int nm, int ld, co
             for (int r = 0; r < 8; ++r) add(c[r], __ldg(wp + r));
         }
         if (e < e1) {
-            float4 c[8];
+            float4 c[7];
 #pragma unroll
             for (int r = 0; r < 7; ++r) c[r] = e + r < e1 ? __ldg(tp + (size_t)r * np) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int r = 0; r < 7; ++r) add(c[r], e + r < e1 ? __ldg(wp + r) : make_float2(0.f, 0.f));
         }
     }
+    if (second) half[wl & 3][lane] = make_float4(re.x, re.y, im.x, im.y);
+    __syncthreads();
+    if (second || !on) return;
+    const float4 o = half[wl & 3][lane];
     float *g = G + ((size_t)f * D + 2 * i) * ld + 2 * m;
-    *reinterpret_cast<float2 *>(g) = make_float2(re.x, -im.x);
-    if (2 * i + 1 < D) *reinterpret_cast<float2 *>(g + ld) = make_float2(re.y, -im.y);
+    *reinterpret_cast<float2 *>(g) = make_float2(re.x + o.x, -(im.x + o.z));
+    if (2 * i + 1 < D) *reinterpret_cast<float2 *>(g + ld) = make_float2(re.y + o.y, -(im.y + o.w));
 }
 
 // Response maps of the mass matrix in hour-angle modes.  Its blocks sum conj(R) R over the LSTs, where a
 // group's responses at the LSTs are R = E Y (E the phasors of its band, Y its modes, at every declination), and
 // E^H E = f f^H with nf columns, fewer than there are LSTs (17 for 60 within 15 degrees): the maps conj(f_j) Y serve as
 // nf LSTs.  X[j][plane][u][d][c] = sqrt(W_u) / sigma times the real (plane 0) and imaginary part of map j0 + j, in the
-// columns of launch_mm_to_modes.  Mass matrix of 37 antennas, 64 channels, 60 LSTs: 83.1 -> 37.6 ms (maps of every
-// LST: transforms 39.8, Gram 27.1 ms; these: 10.4 and 11.1, and 2.4 for the maps, bound by their 8 GB).
+// columns of launch_mm_to_modes.  Mass matrix of 37 antennas, 64 channels, 60 LSTs: 83.1 -> 34.9 ms (maps of every
+// LST: transforms 39.8, Gram 27.1 ms; these: 10.3 and 8.6, and 2.3 for the maps, bound by their 8 GB).
 constexpr int MM_JMAX = 16, MM_MAPP = 4;
 __global__ void __launch_bounds__(256) k_mm_maps(int f, int F, int D, int U, int L, int wmax, int ld, int nj,
                                                  const float2 *__restrict__ fac, const int *__restrict__ code,
@@ -896,7 +903,7 @@ fm_status launch_mm_adjoint(Ctx &c, const float *q32, cudaStream_t st)
         k_mm_q<<<dim3(cdiv(U, 8), c.F), 256, 0, st>>>(
             c.T, U, s.mlo, s.pw, s.wmax, s.code, s.band, s.ph, reinterpret_cast<const float2 *>(q32), s.w);
         FM_CK_LAUNCH();
-        k_mm_adj<<<cdiv(c.F * nchunk * (s.ld / 2), 8), 256, 0, st>>>(c.F, c.D, s.nm, s.ld, s.moff, s.tab, s.w, s.G);
+        k_mm_adj<<<cdiv((long long)c.F * nchunk * (s.ld / 2), 4), 256, 0, st>>>(c.F, c.D, s.nm, s.ld, s.moff, s.tab, s.w, s.G);
         FM_CK_LAUNCH();
         return FM_OK;
     });
