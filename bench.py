@@ -699,6 +699,10 @@ def measure(args, name, K, W, rank, world, dist, local, forms_on=True, err_mode=
         names = ("forward contraction (k_vis_tc)", "adjoint contraction (k_adj_tc)")
         exe = (None, None)
     fwd_dom = fwd_ms >= adj_ms
+    table = h.mode_table_bytes()
+    if table:
+        names = ("forward contraction (k_mm_fwd, k_mm_vis)", "adjoint contraction (k_mm_q, k_mm_adj)")
+        exe = (None, None)
     dom = names[0] if fwd_dom else names[1]
     dom_ms1, dom_n = (fwd_ms1, fwd_n) if fwd_dom else (adj_ms1, adj_n)
     achieved = flops_launch / (dom_ms1 / 1000.0) / 1e12 if dom_n else None
@@ -713,6 +717,12 @@ def measure(args, name, K, W, rank, world, dist, local, forms_on=True, err_mode=
                 "launches": {"forward": fwd_n, "adjoint": adj_n},
                 "timing": "CUDA events around every contraction launch on its stream, in an untimed pass of "
                           f"{min(K, 5)} steps after the timed region"}
+    if table and dom_n:
+        # in hour-angle modes: one pass over the table of modes
+        gbs = table / (dom_ms1 / 1000.0) / 1e9
+        roofline.update(bound="hbm", achieved=gbs, peak=pk["hbm_gbs"], unit="GB/s", frac=gbs / pk["hbm_gbs"], traffic=None,
+                        peak_source=f"{pk_src} copy bandwidth; bytes per launch = the table of hour-angle modes, {table}",
+                        algorithmic_tflops=achieved)
     if exe[0] is not None and dom_n:
         e_dom = exe[0] if fwd_dom else exe[1]
         roofline["tensor_executed_tflops"] = e_dom / (dom_ms1 / 1000.0) / 1e12

@@ -311,6 +311,10 @@ FM_API fm_status fm_sky_pixels_noalloc(int n_freq, int n_ra, int n_dec, int n_mo
  * disables form 2 and FM_HA_GROUPS=0 makes it compute every baseline separately. */
 FM_API fm_status fm_contraction_info(fm_handle h, int32_t *out);
 
+/* Bytes of the table of hour-angle modes that every contraction of the handle reads once; 0 when the handle does
+ * not compute in hour-angle modes, -1 for a NULL handle. */
+FM_API int64_t fm_mode_table_bytes(fm_handle h);
+
 /* Launch grids of the hour-angle contraction kernels (the knobs of the autotuner,
  * paper_2504_07090_gb300/autotune.py; the paper has no counterpart): ctas_fwd CTAs for the
  * forward contraction (its work units are re-partitioned over them) and ctas_adj for the

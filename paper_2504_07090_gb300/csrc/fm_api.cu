@@ -742,6 +742,13 @@ fm_status fm_contraction_info(fm_handle h, int32_t *out)
     return FM_OK;
 }
 
+int64_t fm_mode_table_bytes(fm_handle h)
+{
+    if (!h) return -1;
+    const Ctx &c = *reinterpret_cast<Ctx *>(h);
+    return c.mm.on ? c.mm.ne * ((c.D + 1) / 2) * 16 : 0;
+}
+
 int64_t fm_kernel_launches(void) { return __atomic_load_n(&g_launches, __ATOMIC_RELAXED); }
 
 fm_status fm_sync_status(fm_handle h, fm_stream stream)

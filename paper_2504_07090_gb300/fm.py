@@ -33,7 +33,8 @@ EXPORTS = ["fm_create", "fm_destroy", "fm_num_params", "fm_num_vis", "fm_set_dat
            "fm_contraction_info", "fm_kernel_launches", "fm_sky_pixels_noalloc", "fm_sync_status",
            "fm_last_error", "fm_create_batch", "fm_batch_create", "fm_batch_leapfrog", "fm_batch_kernels",
            "fm_batch_destroy", "fm_diag_bounded_wait", "fm_hmc_chain", "fm_chain_kernels", "fm_draw_normal",
-           "fm_draw_accept_uniform", "fm_set_delay_filter", "fm_set_launch_grids", "fm_get_launch_grids"]
+           "fm_draw_accept_uniform", "fm_set_delay_filter", "fm_set_launch_grids", "fm_get_launch_grids",
+           "fm_mode_table_bytes"]
 CONTRACTION_FORMS = {0: "direct", 1: "antenna", 2: "hour_angle"}
 
 
@@ -86,6 +87,8 @@ def load(path: str = LIB_PATH):
     L.fm_get_precond_blocks.argtypes = [vp, vp, vp]
     L.fm_precond_size.argtypes = [vp]
     L.fm_precond_size.restype = c_int64
+    L.fm_mode_table_bytes.argtypes = [vp]
+    L.fm_mode_table_bytes.restype = c_int64
     L.fm_leapfrog.argtypes = [vp, vp, vp, c_double, c_int, c_double, vp, vp, vp]
     L.fm_sync_status.argtypes = [vp, vp]
     L.fm_precond_apply.argtypes = [vp, c_int, vp, vp, vp]
@@ -111,7 +114,8 @@ def load(path: str = LIB_PATH):
     L.fm_draw_normal.argtypes = [ctypes.c_uint64, ctypes.c_uint64, c_int64, vp, c_int, vp]
     L.fm_draw_accept_uniform.argtypes = [ctypes.c_uint64, ctypes.c_uint64, c_int64, vp, vp]
     for name in EXPORTS:
-        if name not in ("fm_num_params", "fm_num_vis", "fm_precond_size", "fm_last_error", "fm_kernel_launches"):
+        if name not in ("fm_num_params", "fm_num_vis", "fm_precond_size", "fm_last_error", "fm_kernel_launches",
+                        "fm_mode_table_bytes"):
             getattr(L, name).restype = c_int
     _lib = L
     return L
@@ -153,12 +157,13 @@ def _check(status: int, where: str):
         raise FmError(status, where, last_error())
 
 
-def _stream():
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    # the current stream's handle without the Stream object around it (every call passes it)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: torch.Tensor | None):
-    return c_void_p(0) if t is None else c_void_p(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def make_config(prob, precision: str | int = "fp32", sigma: float | None = None):
@@ -246,7 +251,7 @@ class ForwardModel:
         grad = torch.empty(self.n_params, dtype=self.dtype, device="cuda") if grad is None else grad
         scal = torch.empty(2, dtype=torch.float64, device="cuda") if scal is None else scal
         _check(self.lib.fm_chi2_grad(self.h, self._t(theta, self.n_params, "theta"), _ptr(scal),
-                                     c_void_p(scal.data_ptr() + 8), self._t(grad, self.n_params, "grad"), _stream()),
+                                     scal.data_ptr() + 8, self._t(grad, self.n_params, "grad"), _stream()),
                "fm_chi2_grad")
         return scal, grad
 
@@ -332,6 +337,10 @@ class ForwardModel:
         return {"form": CONTRACTION_FORMS[int(out[0])], "fringes": int(out[1]), "lst_step_cells": int(out[2]),
                 "hour_angle_cells": int(out[3])}
 
+    def mode_table_bytes(self) -> int:
+        """Bytes of the table of hour-angle modes a contraction reads (fm_mode_table_bytes); 0: another form."""
+        return int(self.lib.fm_mode_table_bytes(self.h))
+
     def sync_status(self):
         _check(self.lib.fm_sync_status(self.h, _stream()), "fm_sync_status")
 
@@ -339,7 +348,7 @@ class ForwardModel:
 class _Chi2Fn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, theta, model):
-        scal, grad = model.chi2_grad(theta.detach().contiguous())
+        scal, grad = model.chi2_grad(theta.contiguous())
         ctx.save_for_backward(grad)
         return scal[1].to(theta.dtype)
 

@@ -35,6 +35,7 @@ def _outputs(p, prec):
     import torch
     from paper_2504_07090_gb300 import fm
     h = fm.ForwardModel(p, prec, sigma=1.0)
+    assert (h.mode_table_bytes() > 0) == (prec != "fp64")
     th = torch.tensor(synth.draw_truth(p).theta.astype(np.float32), device="cuda").to(h.dtype)
     h.set_data(torch.tensor(synth.random_data(p, 1e4, 3).astype(np.float32), device="cuda").to(h.dtype))
     x = np.random.default_rng(2).standard_normal(h.n_pix_total).astype(np.float32)
