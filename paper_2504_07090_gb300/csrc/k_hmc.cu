@@ -458,55 +458,78 @@ __global__ void k_pc_gain_block(DevGeom g, const double *__restrict__ s2, const 
     }
 }
 
-// Cholesky of one block held in shared memory (n <= 64), FP64, with prior inflation:
-// M = (H - diag(lam)) + c diag(lam), c = 1, 1.1, 1.21, ...  Writes L (lower) in R.
+// Cholesky of every 64 x 64 sky block in FP64 with prior inflation on failure: H + (c - 1) lam on the diagonal,
+// c *= 1.1 per attempt.  Right-looking in registers: warp w holds the rows w + 8 i, a lane the columns lane and
+// lane + 32; per column the raw column goes through shared memory (two buffers, one barrier), its pivot's
+// reciprocal is formed once, and the factor is scaled at the end.  Bound: the FP64 pipe (2 lanes per SM and clock): 3008
+// warp multiply-adds a block, where a thread per row took 2.2 times as many.  FIGURES
 template <typename R>
-__global__ void __launch_bounds__(64) k_pc_chol_small(int n, const double *__restrict__ H, const R *__restrict__ lam,
-                                                      long long lam_off, int have_prior, R *__restrict__ L,
-                                                      int *__restrict__ status)
+__global__ void __launch_bounds__(256) k_pc_chol_small(const double *__restrict__ H, const R *__restrict__ lam,
+                                                       int have_prior, R *__restrict__ L, int *__restrict__ status)
 {
-    __shared__ double sM[64][65];
-    __shared__ int bad;
-    const int blk = blockIdx.x, tid = threadIdx.x;
-    const double *Hb = H + (size_t)blk * n * n;
-    double c = 1.0;
+    __shared__ double sc[2][65], sd[64];                 // raw column and, at [64], the reciprocal of its pivot
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double *Hb = H + (size_t)blockIdx.x * 4096;
+    double a[8][2], c = 1.0;
     for (int attempt = 0; attempt < 200; ++attempt) {
-        for (int e = tid; e < n * n; e += blockDim.x) {
-            int r = e / n, q = e % n;
-            double v = Hb[e];
-            if (r == q && have_prior) {
-                double l = (double)lam[lam_off + (size_t)blk * n + r];
-                v += (c - 1.0) * l;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = w + 8 * i, q = lane + 32 * h;
+                double v = q <= r ? Hb[r * 64 + q] : 0.0;
+                if (q == r && have_prior) v += (c - 1.0) * (double)lam[(size_t)blockIdx.x * 64 + r];
+                a[i][h] = v;
             }
-            sM[r][q] = v;
-        }
-        if (tid == 0) bad = 0;
-        __syncthreads();
-        for (int k = 0; k < n; ++k) {
-            if (tid == 0) {
-                double d = sM[k][k];
-                if (!(d > 0.0) || !isfinite(d)) bad = 1;
-                sM[k][k] = bad ? 1.0 : sqrt(d);
-            }
-            __syncthreads();
+        bool bad = false;
+#pragma unroll
+        for (int kb = 0; kb < 8; ++kb) {
             if (bad) break;
-            double dk = sM[k][k];
-            for (int r = k + 1 + tid; r < n; r += blockDim.x) sM[r][k] /= dk;
-            __syncthreads();
-            for (int r = k + 1 + tid; r < n; r += blockDim.x)
-                for (int q = k + 1; q <= r; ++q) sM[r][q] -= sM[r][k] * sM[q][k];
-            __syncthreads();
+            for (int kk = 0; kk < 8; ++kk) {
+                const int k = 8 * kb + kk;
+                double *col = sc[k & 1];
+                if (lane == (k & 31)) {
+#pragma unroll
+                    for (int i = kb; i < 8; ++i) col[w + 8 * i] = a[i][kb >> 2];
+                    if (w == kk) {
+                        col[64] = 1.0 / a[kb][kb >> 2];
+                        sd[k] = a[kb][kb >> 2];
+                    }
+                }
+                __syncthreads();
+                const double d = col[k], inv = col[64];
+                if (!(d > 0.0) || !isfinite(d)) {        // the same for every thread
+                    bad = true;
+                    break;
+                }
+                const double t0 = kb < 4 && lane > k ? col[lane] * inv : 0.0, t1 = 32 + lane > k ? col[32 + lane] * inv : 0.0;
+#pragma unroll
+                for (int i = kb; i < 8; ++i) {
+                    const int r = w + 8 * i;
+                    if (r > k) {
+                        const double x = col[r];
+                        if (kb < 4) a[i][0] -= x * t0;
+                        if (i >= 4) a[i][1] -= x * t1;
+                    }
+                }
+            }
         }
         __syncthreads();
         if (!bad) break;
         c *= 1.1;
-        __syncthreads();
-        if (attempt == 199 && tid == 0) atomicExch(status, (int)FM_ERR_NOT_SPD);
+        if (attempt == 199) {
+            if (threadIdx.x == 0) atomicExch(status, (int)FM_ERR_NOT_SPD);
+            for (int k = threadIdx.x; k < 64; k += 256) sd[k] = 1.0;
+            __syncthreads();
+        }
     }
-    R *Lb = L + (size_t)blk * n * n;
-    for (int e = tid; e < n * n; e += blockDim.x) {
-        int r = e / n, q = e % n;
-        Lb[e] = (q <= r) ? (R)sM[r][q] : R(0);
+    const double s0 = 1.0 / sqrt(sd[lane]), s1 = 1.0 / sqrt(sd[lane + 32]);
+    R *Lb = L + (size_t)blockIdx.x * 4096;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = w + 8 * i;
+        Lb[r * 64 + lane] = lane <= r ? (R)(a[i][0] * s0) : R(0);
+        Lb[r * 64 + lane + 32] = lane + 32 <= r ? (R)(a[i][1] * s1) : R(0);
     }
 }
 
@@ -722,35 +745,62 @@ __host__ __device__ constexpr int tri_block_elems()
 static_assert(tri_row_start<float>(64) == 544 && tri_row_start<double>(64) == 1056, "packed block size");
 static_assert(tri_row_start<float>(5) == 6 && tri_row_start<float>(4) == 4, "packed row start");
 
-// Inverses of the stored 64 x 64 sky-block factors (one CTA of 64 threads per block):
-// the factor, as stored in the working type, is read into FP64 shared memory and thread
-// j solves L x = e_j by forward substitution; Linv[r][j] = x_r, stored packed (above).
-// Inverting the stored factor keeps L^-1 (L z) = z to FP64 rounding before the final store.
+// Inverses of the stored 64 x 64 sky-block factors (one CTA a block): the factor, as stored in the working type, is
+// read into FP64 shared memory and L X = 1 is solved column of L by column, with X in registers (warp w the rows
+// w + 8 i, a lane the columns lane and lane + 32); Linv[r][j] = X[r][j], stored packed (above).  Inverting the
+// stored factor keeps L^-1 (L z) = z to FP64 rounding before the final store.  Bound: the FP64 pipe: 2512 warp
+// multiply-adds a block, where a thread per column took 4032, most lanes idle.  FIGURES
 template <typename R>
-__global__ void __launch_bounds__(64) k_pc_blk_inv(const R *__restrict__ L, R *__restrict__ Linv)
+__global__ void __launch_bounds__(256) k_pc_blk_inv(const R *__restrict__ L, R *__restrict__ Linv)
 {
-    extern __shared__ double sd[];
-    double *sL = sd;                  // [64][65]
-    double *sX = sd + 64 * 65;        // [64 columns][65]
+    extern __shared__ double sL[];                       // [64][64]
+    __shared__ double sx[2][64], rd[64];
     const R *Lb = L + (size_t)blockIdx.x * 4096;
-    for (int e = threadIdx.x; e < 4096; e += 64) sL[(e >> 6) * 65 + (e & 63)] = (double)Lb[e];
+    for (int e = threadIdx.x; e < 4096; e += 256) sL[e] = (double)Lb[e];
     __syncthreads();
-    const int j = threadIdx.x;
-    double *x = sX + j * 65;
-    for (int r = 0; r < 64; ++r) {
-        double v = 0.0;
-        if (r == j) v = 1.0 / sL[r * 65 + r];
-        else if (r > j) {
-            double a = 0.0;
-            for (int cc = j; cc < r; ++cc) a += sL[r * 65 + cc] * x[cc];
-            v = -a / sL[r * 65 + r];
-        }
-        x[r] = v;
+    if (threadIdx.x < 64) rd[threadIdx.x] = 1.0 / sL[threadIdx.x * 65];
+    __syncthreads();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v[8][2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        v[i][0] = w + 8 * i == lane ? 1.0 : 0.0;
+        v[i][1] = w + 8 * i == lane + 32 ? 1.0 : 0.0;
     }
+#pragma unroll
+    for (int kb = 0; kb < 8; ++kb)
+        for (int kk = 0; kk < 8; ++kk) {
+            const int k = 8 * kb + kk;
+            double *x = sx[k & 1];
+            if (w == kk) {
+                v[kb][0] *= rd[k];
+                x[lane] = v[kb][0];
+                if (kb >= 4) {
+                    v[kb][1] *= rd[k];
+                    x[lane + 32] = v[kb][1];
+                }
+            }
+            __syncthreads();
+            const double x0 = x[lane], x1 = kb >= 4 ? x[lane + 32] : 0.0;
+#pragma unroll
+            for (int i = kb; i < 8; ++i) {
+                const int r = w + 8 * i;
+                if (r > k) {
+                    const double l = sL[r * 64 + k];
+                    v[i][0] -= l * x0;
+                    if (kb >= 4) v[i][1] -= l * x1;
+                }
+            }
+        }
     R *Ib = Linv + (size_t)blockIdx.x * tri_block_elems<R>();
     constexpr int PER = 16 / sizeof(R);
-    for (int r = 0; r < 64; ++r)
-        if (j < tri_row_pieces<R>(r) * PER) Ib[tri_row_start<R>(r) * PER + j] = (R)x[r];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = w + 8 * i, n = tri_row_pieces<R>(r) * PER;
+        R *o = Ib + tri_row_start<R>(r) * PER;
+        if (lane < n) o[lane] = (R)v[i][0];
+        if (lane + 32 < n) o[lane + 32] = (R)v[i][1];
+    }
 }
 
 // Sky prior on the block diagonals: blocks[k/bs][k%bs][k%bs] += lam[k]
@@ -997,8 +1047,8 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
         // factorise every block (prior inflation on failure)
         R *Lf = (R *)c.pc_chol;
         if (bs > 1) {
-            k_pc_chol_small<R><<<(unsigned)nsky_blk, 64, 0, st>>>(bs, c.pc_blocks, (const R *)c.lam, 0,
-                                                                  c.have_prior ? 1 : 0, Lf, c.status);
+            k_pc_chol_small<R><<<(unsigned)nsky_blk, 256, 0, st>>>(c.pc_blocks, (const R *)c.lam, c.have_prior ? 1 : 0,
+                                                                   Lf, c.status);
             if (ng > 0 && !c.pc_ginv) {
                 if (cudaMalloc(&c.pc_ginv, 4 * sizeof(double) * (size_t)ng * ng) != cudaSuccess ||
                     cudaMalloc(&c.pc_tmp, sizeof(double) * (size_t)ng * ng) != cudaSuccess) {
@@ -1028,8 +1078,7 @@ fm_status run_build_precond(Ctx &c, const R *theta, int block, cudaStream_t st)
                 }
                 c.allocs.push_back(c.pc_linv);
             }
-            smem_opt_in(k_pc_blk_inv<R>);
-            k_pc_blk_inv<R><<<(unsigned)nsky_blk, 64, 2 * 64 * 65 * sizeof(double), st>>>(Lf, (R *)c.pc_linv);
+            k_pc_blk_inv<R><<<(unsigned)nsky_blk, 256, 64 * 64 * sizeof(double), st>>>(Lf, (R *)c.pc_linv);
             if (ng > 0) {
                 k_pc_tri_inv<<<ng, 32, sizeof(double) * ng, st>>>(ng, W, c.pc_tmp, G64 + (size_t)ng * ng,
                                                             G64 + 2 * (size_t)ng * ng);
