@@ -25,7 +25,7 @@
 // channels, 120 LSTs: 7.26 -> 0.61 ms (k_mm_fwd 477 us, 3.1 GB at 6.5 TB/s) and 4.98 -> 0.65 ms.  The errors against 64 bits fall to
 // those of the mode transforms (V of 7 antennas 1.3e-6 -> 2.6e-7).
 // FP32 handles: 37 antennas, 64 channels, 60 LSTs, chi^2 and gradient 3.13 ms (each distinct fringe on the CUDA
-// cores, k_hs.cu) -> 0.27 ms; gradient against 64 bits 1.2e-7 in the mean of 14 geometries, as before.
+// cores, k_hs.cu) -> 0.27 ms; gradient against 64 bits 1.0e-7 in the mean of 14 geometries (1.2e-7 before), V 1.7e-7 (2.8e-7).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -567,30 +567,30 @@ __global__ void k_mm_ug(long long FT, int U, int B, const int *__restrict__ moff
     }
 }
 
-template <typename T>
-fm_status mm_alloc(Ctx &c, T **p, size_t count)
-{
-    void *q = nullptr;
-    cudaError_t e = cudaMalloc(&q, count * sizeof(T) > 0 ? count * sizeof(T) : 16);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (hour-angle modes)", __FILE__, __LINE__);
-    c.allocs.push_back(q);
-    *p = reinterpret_cast<T *>(q);
-    return FM_OK;
-}
+// several buffers from one allocation (a cudaMalloc takes tens of microseconds, and small handles are made often)
+struct MmArena {
+    size_t bytes = 0;
+    std::vector<std::pair<void **, size_t>> at;
+    template <typename T> void add(T **p, size_t count)
+    {
+        at.push_back({reinterpret_cast<void **>(p), bytes});
+        bytes += (count * sizeof(T) + 255) / 256 * 256;
+    }
+    fm_status get(std::vector<void *> &owner)
+    {
+        char *q = nullptr;
+        cudaError_t e = cudaMalloc(&q, bytes > 0 ? bytes : 16);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (hour-angle modes)", __FILE__, __LINE__);
+        owner.push_back(q);
+        for (auto &x : at) *x.first = q + x.second;
+        return FM_OK;
+    }
+};
 
 // device buffers that live until the handle is complete
 struct MmTemp {
     std::vector<void *> p;
     ~MmTemp() { for (void *q : p) cudaFree(q); }
-    template <typename T> fm_status get(T **d, size_t n)
-    {
-        void *q = nullptr;
-        cudaError_t e = cudaMalloc(&q, n * sizeof(T));
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (hour-angle modes)", __FILE__, __LINE__);
-        p.push_back(q);
-        *d = reinterpret_cast<T *>(q);
-        return FM_OK;
-    }
 };
 
 // Smallest window of L cells around the nh in use (from LST lst0, q cells a pixel) whose ends the beam does not
@@ -697,9 +697,12 @@ fm_status mm_setup(Ctx &c)
     MmDir *geo = nullptr;
     float *wt = nullptr;
     int2 *band = nullptr;
-    FM_TRY(tmp.get(&tw, L));
-    FM_TRY(tmp.get(&geo, (size_t)c.D * L));
-    FM_TRY(tmp.get(&band, (size_t)c.F * U));
+    MmArena ta;
+    ta.add(&tw, L);
+    ta.add(&geo, (size_t)c.D * L);
+    ta.add(&band, (size_t)c.F * U);
+    ta.add(&wt, (size_t)c.F * c.D * L);
+    FM_TRY(ta.get(tmp.p));
     FM_CK(cudaMemcpy(tw, htw.data(), sizeof(double2) * L, cudaMemcpyHostToDevice));
     MmGeo ga;
     ga.lst0 = lst0; ga.ra_min = c.cfg.ra_min; ga.dra = dra;
@@ -812,21 +815,23 @@ fm_status mm_setup(Ctx &c)
     std::vector<float2> hfac((size_t)s.nf * s.wmax);
     for (int j = 0; j < s.nf; ++j)
         for (int i = 0; i < s.wmax; ++i) hfac[(size_t)j * s.wmax + i] = make_float2((float)fr_[j][i], (float)-fi_[j][i]);
-    FM_TRY(mm_alloc(c, &s.fac, hfac.size()));
+    MmArena pa;
+    pa.add(&s.fac, hfac.size());
+    pa.add(&s.tab, (size_t)s.ne * np);
+    pa.add(&s.moff, moff.size());
+    pa.add(&s.code, code.size());
+    pa.add(&s.items, items.size());
+    pa.add(&s.band, hb.size());
+    pa.add(&s.ph, hph.size());
+    pa.add(&s.z, 2 * (size_t)s.ne);
+    pa.add(&s.w, s.ne);
+    pa.add(&s.Y, 2 * (size_t)c.F * c.D * s.ld);
+    pa.add(&s.G, (size_t)c.F * c.D * s.ld);
+    pa.add(&s.b64, (size_t)s.ld * c.M);
+    pa.add(&s.b32, (size_t)s.ld * c.M);
+    pa.add(&s.pix, (size_t)s.ld * c.R);
+    FM_TRY(pa.get(c.allocs));
     FM_CK(cudaMemcpy(s.fac, hfac.data(), sizeof(float2) * hfac.size(), cudaMemcpyHostToDevice));
-    FM_TRY(mm_alloc(c, &s.tab, (size_t)s.ne * np));
-    FM_TRY(mm_alloc(c, &s.moff, moff.size()));
-    FM_TRY(mm_alloc(c, &s.code, code.size()));
-    FM_TRY(mm_alloc(c, &s.items, items.size()));
-    FM_TRY(mm_alloc(c, &s.band, hb.size()));
-    FM_TRY(mm_alloc(c, &s.ph, hph.size()));
-    FM_TRY(mm_alloc(c, &s.z, 2 * (size_t)s.ne));
-    FM_TRY(mm_alloc(c, &s.w, s.ne));
-    FM_TRY(mm_alloc(c, &s.Y, 2 * (size_t)c.F * c.D * s.ld));
-    FM_TRY(mm_alloc(c, &s.G, (size_t)c.F * c.D * s.ld));
-    FM_TRY(mm_alloc(c, &s.b64, (size_t)s.ld * c.M));
-    FM_TRY(mm_alloc(c, &s.b32, (size_t)s.ld * c.M));
-    FM_TRY(mm_alloc(c, &s.pix, (size_t)s.ld * c.R));
     FM_CK(cudaMemcpy(s.moff, moff.data(), sizeof(int) * moff.size(), cudaMemcpyHostToDevice));
     FM_CK(cudaMemcpy(s.code, code.data(), sizeof(int) * code.size(), cudaMemcpyHostToDevice));
     FM_CK(cudaMemcpy(s.items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
@@ -835,7 +840,6 @@ fm_status mm_setup(Ctx &c)
 
     // the basis holds sums of R values of at most 1: stored over 2^e >= R, which the table takes up
     const int e2 = (int)std::ceil(std::log2((double)c.R));
-    FM_TRY(tmp.get(&wt, (size_t)c.F * c.D * L));
     k_mm_basis<<<1024, 128>>>(c.R, c.M, q, L, s.ld, std::ldexp(1.0, -e2), tw, c.g.phi64, s.b64, s.b32, s.pix);
     FM_CK_LAUNCH();
     k_mm_weight<<<2048, 256>>>(c.F, c.D, L, geo, c.g.bcoef64, c.g.domega64, wt);

@@ -29,8 +29,9 @@ struct GemmArgs {
 
 // FP32: 64 x 64 tiles, 128 threads of 8 x 4 sums (packed FMAs on column pairs: three 16-byte shared loads for 16
 // of them), the next 16 K values on their way in registers while the last are summed.  Each sum runs over K in
-// order.  The four products of the mode transforms of 127 antennas, 128 channels, 256 x 256 modes: 1.10 (256
-// threads of 4 x 4 sums, no prefetch) -> 0.58 ms, 45 TFLOP/s.
+// order, 16 terms at a time (their rounding errors grow with K / 16 + 16, not K).  The four products of the mode transforms of 127 antennas, 128 channels, 256 x 256 modes: 1.10 (256
+// threads of 4 x 4 sums, no prefetch) -> 0.65 ms, 40 TFLOP/s (0.58 ms with one running sum, whose errors were up to
+// twice as large: FP32 gradient of 37 antennas against 64 bits 1.3e-7, now 5e-8).
 constexpr int GM_LD = 68;
 __global__ void __launch_bounds__(128) k_gemm(GemmArgs a, const float *__restrict__ A, const float *__restrict__ B,
                                               float *__restrict__ C)
@@ -82,6 +83,9 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a, const float *__restric
     for (int k0 = 0, s = 0; k0 < a.K; k0 += 16, s ^= 1) {
         const bool more = k0 + 16 < a.K;
         if (more) fetch(k0 + 16);
+        float2 t[8][2];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u][0] = t[u][1] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
             const float4 p = *reinterpret_cast<const float4 *>(&sA[s][k][8 * ty]),
@@ -92,10 +96,14 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a, const float *__restric
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const float2 w = make_float2(av[u], av[u]);
-                acc[u][0] = __ffma2_rn(w, b0, acc[u][0]);
-                acc[u][1] = __ffma2_rn(w, b1, acc[u][1]);
+                t[u][0] = __ffma2_rn(w, b0, t[u][0]);
+                t[u][1] = __ffma2_rn(w, b1, t[u][1]);
             }
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) acc[u][q] = make_float2(acc[u][q].x + t[u][q].x, acc[u][q].y + t[u][q].y);
         if (more) stage(s ^ 1);                 // last read before the previous barrier
         __syncthreads();
     }
