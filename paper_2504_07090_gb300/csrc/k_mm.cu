@@ -611,7 +611,9 @@ int mm_window(const Ctx &c, const std::vector<double> &bcoef, const std::vector<
         return domega[d] * std::exp(bc * za * za);
     };
     // the beam falls with |H|: its maximum in use is at the cell nearest the meridian
-    const double n0 = (c.R - 1) * q + 0.5 * q + (c.cfg.ra_min - lst0) / dh;
+    const double turn = 2.0 * kPi / dh;
+    double n0 = (c.R - 1) * q + 0.5 * q + (c.cfg.ra_min - lst0) / dh;
+    n0 -= turn * std::rint((n0 - 0.5 * nh) / turn);
     const int at = (int)std::fmin(std::fmax(std::rint(n0), 0.0), nh - 1.0);
     double top = 0.0;
     for (int d = 0; d < c.D; ++d) top = std::fmax(top, weight(d, at));

@@ -17,7 +17,7 @@ GEOMETRIES = {
     "one_dec": (2, 2, 17, 1, 40, None), "lst70": (2, 1, 70, 3, 224, None), "dec130": (2, 1, 5, 130, 32, None),
     "hex61": (5, 1, 5, 3, 32, None), "offgrid": (3, 6, 3, 7, 41, None), "offgrid16": (4, 3, 16, 6, 70, None),
     "uneven": (4, 2, 9, 5, 64, "uneven"), "backwards": (3, 2, 6, 5, 64, "backwards"), "wide_lst": (2, 2, 65, 4, 100, "uneven"),
-    "hex127": (7, 1, 120, 3, 384, None),
+    "hex127": (7, 1, 120, 3, 384, None), "turn": (3, 2, 6, 5, 64, "turn"),
 }
 
 
@@ -28,6 +28,8 @@ def _problem(name):
         p.lst_rad = p.lst_rad + 1e-3 * np.random.default_rng(8).standard_normal(nt)
     if lst == "backwards":
         p.lst_rad = np.ascontiguousarray(p.lst_rad[::-1])
+    if lst == "turn":             # hour angles around -2 pi: right ascensions a turn ahead of the LSTs
+        p.ra_min, p.ra_max = p.ra_min + 2 * np.pi, p.ra_max + 2 * np.pi
     return p
 
 
