@@ -356,6 +356,21 @@ extern long long g_launches;     // kernels launched by the library (relaxed cou
         FM_CK(cudaGetLastError());                                          \
     } while (0)
 
+// Visibilities are written into the caller's buffer, which need only be aligned for one real of them: both
+// parts at once where the buffer is aligned for the pair (pair_aligned, the same for a whole launch).
+template <typename C2, typename R>
+__device__ __forceinline__ bool pair_aligned(const R *p) { return (reinterpret_cast<uintptr_t>(p) & (sizeof(C2) - 1)) == 0; }
+template <typename C2, typename R>
+__device__ __forceinline__ void put_pair(R *p, const C2 &v, bool aligned)
+{
+    if (aligned) {
+        *reinterpret_cast<C2 *>(p) = v;
+    } else {
+        p[0] = v.x;
+        p[1] = v.y;
+    }
+}
+
 // Lets kernel `fn` launch with up to the device's opt-in shared memory per block (less its
 // static shared memory).  The limit
 // is an attribute of the function, shared by every handle in the process, so it is raised to

@@ -779,6 +779,7 @@ __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float 
     __syncthreads();
     const float sc = 1.f / (sp * pow2_scale(__uint_as_float(xmax[f])));
     const float cf = dc ? dc[(size_t)f * dcs] : 0.f;
+    const bool pair = pair_aligned<float2>(vis);
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
         const int code = bmap[b], u = code >> 1;
         if ((u >> 6) != mt) continue;
@@ -799,7 +800,7 @@ __global__ void __launch_bounds__(256) k_ha_vfinish(HaDev h, int B, const float 
                 v.y = __fmaf_rn(cf, u2.y, v.y);
             }
             if (gamma) v = make_float2(gg.x * v.x - gg.y * v.y, gg.x * v.y + gg.y * v.x);
-            reinterpret_cast<float2 *>(vis)[e] = v;
+            put_pair(vis + 2 * e, v, pair);
         }
     }
 }

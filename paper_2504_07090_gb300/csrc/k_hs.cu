@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int n
 {
     using C2 = typename C2of<R>::t;
     const long long n = (long long)F * T * U;
+    const bool pair = pair_aligned<C2>(vis);
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const int u = (int)(e % U);
         const long long ft = e / U;
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int n
                 v.x += cf * (R)Udc[o];
                 v.y += cf * (R)Udc[o + 1];
             }
-            *reinterpret_cast<C2 *>(vis + o) = v;
+            put_pair(vis + o, v, pair);
         }
     }
 }
