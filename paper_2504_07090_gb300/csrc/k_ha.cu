@@ -1418,6 +1418,16 @@ fm_status vis_ha_dual_launch(Ctx &c, const HaDev &h, const HaSky &a, const HaSky
     return fwd_finish(c, hc, b);
 }
 
+// group sums of omega; a (channel, LST)'s baselines pass the default 48 KB from 111 antennas on
+fm_status launch_qsum(Ctx &c, const HaDev &h, const float *omega, cudaStream_t st)
+{
+    const HaState &s = c.ha;
+    FM_CK(smem_opt_in(k_ha_qsum));
+    k_ha_qsum<<<c.F * c.T, 256, sizeof(float) * 2 * (size_t)c.B, st>>>(h, c.B, omega, s.moff, s.mem, s.q32, s.qmax_ft);
+    FM_CK_LAUNCH();
+    return FM_OK;
+}
+
 template <int ET, bool X3>
 fm_status adj_ha_launch(Ctx &c, const HaDev &h, const float *omega, float *xbar, cudaStream_t st, bool q_ready)
 {
@@ -1427,11 +1437,7 @@ fm_status adj_ha_launch(Ctx &c, const HaDev &h, const float *omega, float *xbar,
         set_error("hour-angle adjoint tiles exceed shared memory");
         return FM_ERR_UNSUPPORTED;
     }
-    if (!q_ready) {
-        k_ha_qsum<<<c.F * c.T, 256, sizeof(float) * 2 * (size_t)c.B, st>>>(h, c.B, omega, s.moff, s.mem, s.q32,
-                                                                            s.qmax_ft);
-        FM_CK_LAUNCH();
-    }
+    if (!q_ready) FM_TRY(launch_qsum(c, h, omega, st));
     int grid = s.grid_adj > 0 ? s.grid_adj : sm_count();
     if (grid > c.F * c.D) grid = c.F * c.D;
     const bool wide = s.npa > HA_TCHUNK;
@@ -1829,13 +1835,8 @@ bool ha_strip_args(const Ctx &c, StripArgs &sa, int slot)
 
 fm_status launch_adjoint_ha_modes(Ctx &c, const float *omega, cudaStream_t st, bool q_ready)
 {
-    const HaState &s = c.ha;
-    if (!q_ready) {
-        k_ha_qsum<<<c.F * c.T, 256, sizeof(float) * 2 * (size_t)c.B, st>>>(make_dev(c), c.B, omega, s.moff, s.mem, s.q32,
-                                                                            s.qmax_ft);
-        FM_CK_LAUNCH();
-    }
-    return launch_mm_adjoint(c, s.q32, st);
+    if (!q_ready) FM_TRY(launch_qsum(c, make_dev(c), omega, st));
+    return launch_mm_adjoint(c, c.ha.q32, st);
 }
 
 fm_status launch_adjoint_ha(Ctx &c, const float *omega, float *xbar, cudaStream_t st, bool q_ready)
