@@ -935,13 +935,15 @@ fm_status launch_chi2_chan(Ctx &c, const R *vis, const R *gamma, R *omega, R *zp
         set_error("V from the forward's partial sums: hour-angle form, FP32, no delay filter");
         return FM_ERR_STATE;
     }
-    const size_t smem = (c.A + 3 * (size_t)c.B) * 2 * sizeof(R) + (hv ? sizeof(float) * 128 * (size_t)hv->nmt : 0);
-    if (smem > 227 * 1024 || c.A > CF_THREADS) {
-        set_error("chi^2 epilogue: %d antennas (at most %d, %zu bytes of shared memory)", c.A, CF_THREADS, smem);
+    // the limit of k_chi2_ft without V of the groups holds for either kernel: k_chi2_group takes less (V of at most B
+    // groups and the residuals), and k_chi2_ft runs with V of the groups only up to 56 KB without it
+    const size_t base = (c.A + 3 * (size_t)c.B) * 2 * sizeof(R);
+    if (base > 227 * 1024 || c.A > CF_THREADS) {
+        set_error("chi^2 epilogue: %d antennas (at most %d, %zu bytes of shared memory)", c.A, CF_THREADS, base);
         return FM_ERR_UNSUPPORTED;
     }
     if constexpr (std::is_same<R, float>::value)
-        if (groups && (c.A + 3 * (size_t)c.B) * 2 * sizeof(R) > 56 * 1024) {   // fewer than four CTAs of k_chi2_ft an SM
+        if (groups && base > 56 * 1024) {              // fewer than four CTAs of k_chi2_ft an SM
             const size_t sm = ((size_t)c.A + c.ha.U + c.B) * sizeof(float2);
             FM_CK(smem_opt_in(k_chi2_group));
             k_chi2_group<<<c.F * c.T, CG_THREADS, sm, st>>>(c.g, vis, (const float *)c.data, gamma, zpart, chi2p, c.ha.U,
@@ -950,6 +952,7 @@ fm_status launch_chi2_chan(Ctx &c, const R *vis, const R *gamma, R *omega, R *zp
             FM_CK_LAUNCH();
             return FM_OK;
         }
+    const size_t smem = base + (hv ? sizeof(float) * 128 * (size_t)hv->nmt : 0);
     FM_CK(smem_opt_in(k_chi2_ft<R>));
     k_chi2_ft<R><<<c.F * c.T, CF_THREADS, smem, st>>>(c.g, vis, (const R *)c.data, gamma, omega, zpart, chi2p, c.ha.U, c.ha.moff,
                                                       c.ha.mem, groups ? c.ha.q32 : nullptr, c.ha.qmax_ft, rin,

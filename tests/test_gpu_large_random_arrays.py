@@ -1,6 +1,7 @@
 """FP32 handles of large arrays without redundancy (every baseline a fringe of its own) in hour-angle modes against the
-per-baseline sums: Hessian-vector products from where a baseline list passes 48 KB (111 antennas) to the largest that
-the tangent epilogue takes (120).  Bound: that of the large-array epilogue's gradients (1e-4)."""
+per-baseline sums: gradients up to the largest array whose per-baseline epilogue fits a CTA (138 antennas), and
+Hessian-vector products from where a baseline list passes 48 KB (111 antennas) to the largest that the tangent
+epilogue takes (120).  Bounds: those of the large-array epilogue (chi^2 2e-5, gradients and products 1e-4)."""
 import numpy as np
 import pytest
 
@@ -33,6 +34,16 @@ def _both(p, monkeypatch, call):
 
 def _err(a, b):
     return float((a.double() - b.double()).norm() / b.double().norm())
+
+
+@pytest.mark.parametrize("n_ant", [120, 121, 138])
+def test_gradient_matches_per_baseline_sums(n_ant, monkeypatch):
+    def call(h, th):
+        scal, grad = h.chi2_grad(th)
+        return float(scal[0]), grad.clone()
+    (ca, ga), (cb, gb) = _both(_problem(n_ant), monkeypatch, call)
+    assert abs(ca - cb) < 2e-5 * cb
+    assert _err(ga, gb) < 1e-4
 
 
 @pytest.mark.parametrize("n_ant", [110, 111, 120])
