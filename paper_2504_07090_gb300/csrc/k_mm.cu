@@ -12,7 +12,11 @@
 // basis functions replaced by their Fourier sums, so the pixels are never formed.  Cells outside 0 .. nh - 1 meet no
 // pixel: there P_u is continued by its own formula, to where the beam is below MM_EDGE of its maximum, so that
 // the window has no step and the band ends; what a band leaves out is below MM_EPS of the response's l2 norm,
-// far under the FP32 rounding (6e-8) of the table that keeps it.
+// far under the FP32 rounding (6e-8) of the table that keeps it.  All of these are relative to the largest response
+// in the window, and a grid whose hour angles stay off the meridian has it in cells that meet no pixel: what is
+// left in those in use is then wrong by 3e-8 times the ratio of the two (a beam of 4.2 degrees FWHM, the nearest
+// cell in use 5 degrees off the meridian: 2e-6; 10 degrees off: 1e-2).  The form is taken up to a ratio of MM_PEAK = 4,
+// where that is 1e-7, below the FP32 sums' own 2.8e-7.
 //
 // The sky is real, so modes m and -m share Y: an element e = (|m|, u, sign) keeps c_u(m) or conj(c_u(-m)).
 // The table [e][declination] is sorted by |m|: the forward is one dot product over declinations per element, the
@@ -37,6 +41,7 @@ namespace {
 
 constexpr double MM_EDGE = 4e-9;       // beam at the window's ends, relative to its maximum
 constexpr double MM_EPS = 1e-9;        // l2 share of a response outside its band
+constexpr double MM_PEAK = 4.0;        // beam in the cells around those in use, relative to its maximum in them
 constexpr int MM_MAXL = 2048;
 constexpr int MM_MAXQ = 8;             // cells per RA pixel, LSTs off the pixel grid
 constexpr int MM_ROWS = 8;             // forward: elements a warp sums at a time
@@ -594,27 +599,44 @@ struct MmTemp {
 };
 
 // Smallest window of L cells around the nh in use (from LST lst0, q cells a pixel) whose ends the beam does not
-// reach; 0 when there is none below 2 nh cells or a turn of hour angle.
+// reach; 0 when there is none below 2 nh cells or a turn of hour angle, or when the beam is larger in the cells
+// around those in use by more than MM_PEAK.
 int mm_window(const Ctx &c, const std::vector<double> &bcoef, const std::vector<double> &domega, double lst0, int q,
               int nh, MmFft &p)
 {
     const double dh = (c.cfg.ra_max - c.cfg.ra_min) / c.R / q, ddec = (c.cfg.dec_max - c.cfg.dec_min) / c.D;
-    double bc = bcoef[0];
-    for (double b : bcoef) bc = std::fmax(bc, b);
+    double bc = bcoef[0], bn = bcoef[0];           // of the widest and the narrowest beam
+    for (double b : bcoef) {
+        bc = std::fmax(bc, b);
+        bn = std::fmin(bn, b);
+    }
     if (!(bc < 0.0)) return 0;
     const double sl = std::sin(c.cfg.latitude_rad), cl = std::cos(c.cfg.latitude_rad);
-    auto weight = [&](int d, int n) {
+    auto zenith_angle = [&](int d, int n) {        // of cell n; pi / 2 below the horizon (the step there)
         const double H = lst0 - (c.cfg.ra_min + ((double)((c.R - 1) * q - n) + 0.5 * q) * dh);
         const double dec = c.cfg.dec_min + (d + 0.5) * ddec;
         const double sU = sl * std::sin(dec) + cl * std::cos(dec) * std::cos(H);
-        const double za = sU > 0.0 ? std::acos(sU > 1.0 ? 1.0 : sU) : 0.5 * kPi;   // the step at the horizon
+        return sU > 0.0 ? std::acos(sU > 1.0 ? 1.0 : sU) : 0.5 * kPi;
+    };
+    auto weight = [&](int d, int n) {
+        const double za = zenith_angle(d, n);
         return domega[d] * std::exp(bc * za * za);
+    };
+    // log of the narrowest beam's maximum over the declinations at cell n; none below the horizon
+    auto narrow = [&](int n) {
+        double t = -INFINITY;
+        for (int d = 0; d < c.D; ++d) {
+            const double za = zenith_angle(d, n);
+            if (za < 0.5 * kPi && domega[d] > 0.0) t = std::fmax(t, std::log(domega[d]) + bn * za * za);
+        }
+        return t;
     };
     // the beam falls with |H|: its maximum in use is at the cell nearest the meridian
     const double turn = 2.0 * kPi / dh;
     double n0 = (c.R - 1) * q + 0.5 * q + (c.cfg.ra_min - lst0) / dh;
     n0 -= turn * std::rint((n0 - 0.5 * nh) / turn);
     const int at = (int)std::fmin(std::fmax(std::rint(n0), 0.0), nh - 1.0);
+    const double used = narrow(at);
     double top = 0.0;
     for (int d = 0; d < c.D; ++d) top = std::fmax(top, weight(d, at));
     for (int L = nh + (nh & 1); L <= 2 * nh + 64 && L <= MM_MAXL && L * dh <= 2.0 * kPi; L += 2) {
@@ -622,7 +644,10 @@ int mm_window(const Ctx &c, const std::vector<double> &bcoef, const std::vector<
         const int p0 = (L - nh) / 2;
         double edge = 0.0;
         for (int d = 0; d < c.D; ++d) edge = std::fmax(edge, std::fmax(weight(d, -p0), weight(d, L - 1 - p0)));
-        if (edge <= MM_EDGE * top) return L;
+        if (edge <= MM_EDGE * top) {
+            const int near = (int)std::fmin(std::fmax(std::rint(n0), -p0), L - 1 - p0);    // as `at`, in the window
+            return narrow(near) - used <= std::log(MM_PEAK) ? L : 0;
+        }
     }
     return 0;
 }
