@@ -322,7 +322,8 @@ FM_API int64_t fm_mode_table_bytes(fm_handle h);
  * independent handles (the batched schedule) run side by side on the GPU.  The results change
  * only by the order of the partial sums.  FM_ERR_UNSUPPORTED when the handle does not run the
  * hour-angle form.  fm_get_launch_grids writes the grids in use to out[2] (host int32; 0 when
- * the form is off).  Not to be called while work of the handle is in flight or captured. */
+ * the form is off).  Not to be called while work of the handle is in flight or captured.  A handle that
+ * computes in hour-angle modes (fm_mode_table_bytes > 0) keeps the grids set and does not use them. */
 FM_API fm_status fm_set_launch_grids(fm_handle h, int ctas_fwd, int ctas_adj);
 FM_API fm_status fm_get_launch_grids(fm_handle h, int32_t *out);
 

@@ -17,6 +17,10 @@ use runs longer.  The tuner
 
 All of it is host-side scheduling: the kernels and their arithmetic are unchanged (a grid
 change only regroups the forward's partial sums).
+
+A handle that computes in hour-angle modes takes the grids and does not use them (its kernels have
+grids of their own): it is timed at one grid for all candidates, under a key of its own, and
+`tune_batch` leaves it at the default.
 """
 from __future__ import annotations
 
@@ -38,11 +42,17 @@ def default_cache_path() -> str:
     return os.path.join(os.path.expanduser("~"), ".cache", "paper_2504_07090_gb300", "launch_grids.json")
 
 
+def uses_grids(model: "fm.ForwardModel") -> bool:
+    """Whether the model's contraction kernels run on the grids set (hour-angle form, not in modes)."""
+    return model.contraction_info()["form"] == "hour_angle" and model.mode_table_bytes() == 0
+
+
 def shape_key(model: "fm.ForwardModel") -> str:
+    # the last part tells the kernels: the same sizes run either ("cells": the grids matter)
     info = model.contraction_info()
     p = model.prob
     return (f"A{p.n_ant}-U{info['fringes']}-F{p.n_freq}-D{p.n_dec}-R{p.n_ra}-H{info['hour_angle_cells']}"
-            f"-T{p.n_lst}-k{info['lst_step_cells']}-{model.precision}")
+            f"-T{p.n_lst}-k{info['lst_step_cells']}-{model.precision}-{'cells' if uses_grids(model) else 'modes'}")
 
 
 def load_cache(path: str) -> dict:
@@ -65,13 +75,15 @@ def save_cache(path: str, cache: dict) -> None:
 
 def measure(model: "fm.ForwardModel", theta: torch.Tensor, candidates=CANDIDATES, reps: int = 5) -> dict:
     """Milliseconds per chi^2 + gradient evaluation of `model` at each candidate grid (the same
-    count of CTAs for the forward and the adjoint), after one untimed evaluation per grid."""
+    count of CTAs for the forward and the adjoint), after one untimed evaluation per grid; a model
+    that does not use the grids is timed once for all of them."""
     sm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     st = torch.cuda.current_stream()
     scal = torch.empty(2, dtype=torch.float64, device="cuda")
     grad = torch.empty_like(theta)
     out = {}
-    for g in sorted({min(int(c), sm) for c in candidates}):
+    grids = sorted({min(int(c), sm) for c in candidates})
+    for g in grids if uses_grids(model) else grids[-1:]:
         model.set_launch_grids(g, g)
         model.chi2_grad(theta, grad, scal)
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -82,7 +94,7 @@ def measure(model: "fm.ForwardModel", theta: torch.Tensor, candidates=CANDIDATES
         torch.cuda.synchronize()
         out[str(g)] = a.elapsed_time(b) / reps
     model.set_launch_grids(0, 0)
-    return out
+    return {str(g): out.get(str(g), out[str(grids[-1])]) for g in grids}
 
 
 def choose(times: dict, slack: float) -> int:
@@ -130,25 +142,26 @@ def tune_batch(models, thetas, run_step, slacks=(1.0, 1.25, 1.5, 2.0, 3.0), cach
     """Pick the slack whose grids give the shortest batch step.  run_step() must build the batch
     for the models' current grids, run it and return its milliseconds per step.  Returns a
     report: the slack chosen, the step time of each slack and of the default grids, and the
-    number of shapes that had to be timed."""
+    number of shapes that had to be timed.  No slack is tried when no model uses its grids."""
     t0 = time.perf_counter()
     tables, timed = shape_times(models, thetas, cache_path, candidates)
     for m, tab in zip(models, tables):
         if tab is not None:
             m.set_launch_grids(0, 0)
     default_ms = run_step()
+    live = [tab if tab is not None and uses_grids(m) else None for m, tab in zip(models, tables)]
     steps = {}
-    for s in slacks:
-        apply(models, tables, s)
+    for s in slacks if any(tab is not None for tab in live) else ():
+        apply(models, live, s)
         steps[str(s)] = run_step()
-    best = min(steps, key=steps.get)
-    if steps[best] >= default_ms:
+    best = min(steps, key=steps.get, default=None)
+    if best is None or steps[best] >= default_ms:
         for m, tab in zip(models, tables):
             if tab is not None:
                 m.set_launch_grids(0, 0)
         chosen = "default"
     else:
-        apply(models, tables, float(best))
+        apply(models, live, float(best))
         chosen = float(best)
     grids = [m.launch_grids()[0] if tab is not None else None for m, tab in zip(models, tables)]
     return {"slack": chosen, "ms_per_step": {"default": default_ms, **steps}, "shapes_timed": timed,
