@@ -358,7 +358,8 @@ fm_status gd_setup(Ctx &c)
     s.on = false;
     if (const char *e = getenv("FM_HA_GROUPS"))
         if (atoi(e) == 0) return FM_OK;
-    if ((c.ha.on && !c.mm.on) || c.hs.on || fg.U > GD_MAX_U) return FM_OK;   // with c.mm: the monopole's sum
+    // with c.mm: only the monopole's sum off the pixel grid, which has a buffer of its own (launch_vis_gd)
+    if ((c.ha.on && !c.mm.on) || c.hs.on || (c.mm.on && fg.drift) || fg.U > GD_MAX_U) return FM_OK;
     const bool f64 = c.prec == FM_PREC_FP64_SIMT;
     if (c.prec >= FM_PREC_BF16X1) return FM_OK;
     if (std::max(gd_fwd_smem<double>(c), f64 ? gd_adj_smem<double>(c) : gd_adj_smem<float>(c)) > 200 * 1024) return FM_OK;
@@ -372,9 +373,11 @@ fm_status gd_setup(Ctx &c)
     std::sort(ord.begin(), ord.end(), [](const int4 &a, const int4 &b) { return a.x != b.x ? a.x < b.x : a.y < b.y; });
     FM_TRY(gd_alloc(c, &s.ord, sizeof(int4) * ord.size()));
     FM_CK(cudaMemcpy(s.ord, ord.data(), sizeof(int4) * ord.size(), cudaMemcpyHostToDevice));
-    const size_t v = (size_t)c.F * c.T * fg.U * 2 * c.rsz;
-    FM_TRY(gd_alloc(c, &s.part, v * s.nsplit));
-    FM_TRY(gd_alloc(c, &s.qsum, v));
+    if (!c.mm.on) {
+        const size_t v = (size_t)c.F * c.T * fg.U * 2 * c.rsz;
+        FM_TRY(gd_alloc(c, &s.part, v * s.nsplit));
+        FM_TRY(gd_alloc(c, &s.qsum, v));
+    }
     s.on = true;
     return FM_OK;
 }
