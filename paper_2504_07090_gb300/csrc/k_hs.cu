@@ -22,8 +22,11 @@
 // 16 channels, 20 LSTs, 32 x 96 pixels in FP64 10.08 -> 0.44 ms.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdlib>
+#include <cstring>
 #include <type_traits>
+#include <unordered_map>
 #include <vector>
 
 #include "fm_internal.cuh"
@@ -65,6 +68,55 @@ bool drift_step(const Ctx &c, int &k, int &q)
     return false;
 }
 
+// Groups by the cell of 1 um their vectors fall into; a vector on the edge of cells is looked for in all of them.  (Every
+// vector against every group took 19 ms for 4950 baselines, and grew with their square.)
+class FringeCells {
+public:
+    explicit FringeCells(double tol) : tol_(tol) {}
+    void add(const double *v, int u)
+    {
+        double q[3];
+        for (int c = 0; c < 3; ++c) q[c] = cell(v[c]);
+        map_[key(q)].push_back(u);
+    }
+    // f(u) for every group within tol of v, and perhaps others
+    template <typename F> void around(const double *v, F f) const
+    {
+        double lo[3], hi[3], q[3];
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = cell(v[c] - 2.0 * tol_);
+            hi[c] = cell(v[c] + 2.0 * tol_);
+        }
+        for (int s = 0; s < 8; ++s) {
+            bool again = false;
+            for (int c = 0; c < 3; ++c) {
+                q[c] = s >> c & 1 ? hi[c] : lo[c];
+                again = again || (s >> c & 1 && hi[c] == lo[c]);
+            }
+            if (again) continue;
+            const auto it = map_.find(key(q));
+            if (it == map_.end()) continue;
+            for (int u : it->second) f(u);
+        }
+    }
+
+private:
+    static double cell(double x) { return std::floor(x * 1e6) + 0.0; }      // no negative zero
+    static uint64_t key(const double *q)
+    {
+        uint64_t h = 0;
+        for (int c = 0; c < 3; ++c) {
+            uint64_t b;
+            std::memcpy(&b, q + c, sizeof b);
+            h = (h ^ b) * 0x9e3779b97f4a7c15ull;
+            h ^= h >> 32;
+        }
+        return h;
+    }
+    double tol_;
+    std::unordered_map<uint64_t, std::vector<int>> map_;
+};
+
 // Groups, covering antenna subset (greedy: add the antenna that completes the most groups, ties
 // broken by partial coverage; each group's representative is a member pair inside it) and the
 // device tables.  FM_HA_GROUPS=0 keeps every baseline a group of its own; FM_HA=0 switches the
@@ -87,29 +139,32 @@ fm_status fringe_setup(Ctx &c)
     std::vector<int> rep_i, rep_j, bmap(c.B), bi(c.B), bj(c.B);
     std::vector<double> rep_b;
     std::vector<std::vector<int>> members;
+    FringeCells cells(tol);
     for (int i = 0, b = 0; i < c.A; ++i)
         for (int j = i + 1; j < c.A; ++j, ++b) {
             bi[b] = i;
             bj[b] = j;
-            const double v0 = c.ant[3 * i] - c.ant[3 * j], v1 = c.ant[3 * i + 1] - c.ant[3 * j + 1],
-                         v2 = c.ant[3 * i + 2] - c.ant[3 * j + 2];
-            int found = -1, cj = 0;
-            if (group)
-                for (size_t u = 0; u < rep_i.size() && found < 0; ++u) {
+            const double v[3] = {c.ant[3 * i] - c.ant[3 * j], c.ant[3 * i + 1] - c.ant[3 * j + 1],
+                                 c.ant[3 * i + 2] - c.ant[3 * j + 2]};
+            int found = -1, cj = 0;       // the first group whose vector is v, or -v
+            for (int flip = 0; flip < 2 && group; ++flip) {
+                const double w[3] = {flip ? -v[0] : v[0], flip ? -v[1] : v[1], flip ? -v[2] : v[2]};
+                cells.around(w, [&](int u) {
                     const double *r = &rep_b[3 * u];
-                    const double dp = std::fmax(std::fabs(v0 - r[0]), std::fmax(std::fabs(v1 - r[1]), std::fabs(v2 - r[2])));
-                    const double dm = std::fmax(std::fabs(v0 + r[0]), std::fmax(std::fabs(v1 + r[1]), std::fabs(v2 + r[2])));
-                    if (dp < tol) { found = (int)u; cj = 0; }
-                    else if (dm < tol) { found = (int)u; cj = 1; }
-                }
+                    if ((found >= 0 && u >= found) ||
+                        !(std::fmax(std::fabs(w[0] - r[0]), std::fmax(std::fabs(w[1] - r[1]), std::fabs(w[2] - r[2]))) < tol))
+                        return;
+                    found = u;
+                    cj = flip;
+                });
+            }
             if (found < 0) {
                 found = (int)rep_i.size();
                 rep_i.push_back(i);
                 rep_j.push_back(j);
-                rep_b.push_back(v0);
-                rep_b.push_back(v1);
-                rep_b.push_back(v2);
+                rep_b.insert(rep_b.end(), v, v + 3);
                 members.emplace_back();
+                cells.add(v, found);
             }
             bmap[b] = 2 * found + cj;
             members[found].push_back(2 * b + cj);
@@ -125,26 +180,37 @@ fm_status fringe_setup(Ctx &c)
         for (int a = 0; a < c.A; ++a) in_s[a] = 1;
         n_unc = 0;
     }
+    std::vector<long long> full(c.A), part(c.A);
+    std::vector<int> full_of(c.A), part_of(c.A);        // the last group counted
     while (n_unc > 0) {
-        int best = -1;
-        long long bfull = -1, bpart = -1;
-        for (int a = 0; a < c.A; ++a) {
-            if (in_s[a]) continue;
-            long long full = 0, part = 0;
-            for (int u = 0; u < fg.U; ++u) {
-                if (!uncovered[u]) continue;
-                bool f1 = false, p1 = false;
-                for (int m : members[u]) {
-                    const int b = m >> 1, i = bi[b], j = bj[b];
-                    const bool hi = in_s[i] || i == a, hj = in_s[j] || j == a;
-                    if (hi && hj) { f1 = true; break; }
-                    if (hi || hj) p1 = true;
-                }
-                full += f1;
-                part += p1;
+        // per antenna: groups it completes, and partly covers (less those that every antenna does: the groups with a
+        // member of one antenna in S, which only the antenna that completes the first such member may not)
+        std::fill(full.begin(), full.end(), 0);
+        std::fill(part.begin(), part.end(), 0);
+        std::fill(full_of.begin(), full_of.end(), -1);
+        std::fill(part_of.begin(), part_of.end(), -1);
+        for (int u = 0; u < fg.U; ++u) {
+            if (!uncovered[u]) continue;
+            const std::vector<int> &mu = members[u];
+            size_t first = 0;
+            while (first < mu.size() && !in_s[bi[mu[first] >> 1]] && !in_s[bj[mu[first] >> 1]]) ++first;
+            for (size_t k = 0; k < first; ++k)
+                for (int a : {bi[mu[k] >> 1], bj[mu[k] >> 1]})
+                    if (part_of[a] != u) {
+                        part_of[a] = u;
+                        if (first == mu.size()) ++part[a];
+                    }
+            for (size_t k = first; k < mu.size(); ++k) {
+                const int i = bi[mu[k] >> 1], j = bj[mu[k] >> 1], a = in_s[i] ? j : i;
+                if ((!in_s[i] && !in_s[j]) || full_of[a] == u) continue;
+                full_of[a] = u;
+                ++full[a];
+                if (k == first && part_of[a] != u) --part[a];
             }
-            if (full > bfull || (full == bfull && part > bpart)) { best = a; bfull = full; bpart = part; }
         }
+        int best = -1;
+        for (int a = 0; a < c.A; ++a)
+            if (!in_s[a] && (best < 0 || full[a] > full[best] || (full[a] == full[best] && part[a] > part[best]))) best = a;
         in_s[best] = 1;
         for (int u = 0; u < fg.U; ++u) {
             if (!uncovered[u]) continue;
