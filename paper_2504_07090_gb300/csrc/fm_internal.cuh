@@ -359,7 +359,7 @@ extern long long g_launches;     // kernels launched by the library (relaxed cou
 // Visibilities are written into the caller's buffer, which need only be aligned for one real of them: both
 // parts at once where the buffer is aligned for the pair (pair_aligned, the same for a whole launch).
 template <typename C2, typename R>
-__device__ __forceinline__ bool pair_aligned(const R *p) { return (reinterpret_cast<uintptr_t>(p) & (sizeof(C2) - 1)) == 0; }
+__host__ __device__ __forceinline__ bool pair_aligned(const R *p) { return (reinterpret_cast<uintptr_t>(p) & (sizeof(C2) - 1)) == 0; }
 template <typename C2, typename R>
 __device__ __forceinline__ void put_pair(R *p, const C2 &v, bool aligned)
 {

@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(256) k_hs_fwd(HsDev h, const typename C2of<R>:
 
 // V of every member of a group: the splits' partial sums in order, conjugated for reversed
 // members, plus the monopole dc[f dcs] Udc[f][t][b]
-template <typename R>
+template <typename R, bool PAIR>
 __global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int nsplit, int B, const typename C2of<R>::t *__restrict__ part,
                                                    const int *__restrict__ moff, const int *__restrict__ mem,
                                                    const R *__restrict__ dc, long long dcs,
@@ -489,7 +489,6 @@ __global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int n
 {
     using C2 = typename C2of<R>::t;
     const long long n = (long long)F * T * U;
-    const bool pair = pair_aligned<C2>(vis);
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const int u = (int)(e % U);
         const long long ft = e / U;
@@ -513,7 +512,7 @@ __global__ void __launch_bounds__(128) k_group_finish(int F, int T, int U, int n
                 v.x += cf * (R)Udc[o];
                 v.y += cf * (R)Udc[o + 1];
             }
-            put_pair(vis + o, v, pair);
+            put_pair(vis + o, v, PAIR);
         }
     }
 }
@@ -740,8 +739,10 @@ static unsigned group_blocks(const Ctx &c)
 template <typename R>
 fm_status launch_group_finish(Ctx &c, int nsplit, const void *part, R *vis, cudaStream_t st, const R *dc, long long dcs)
 {
-    k_group_finish<R><<<2 * group_blocks(c), 128, 0, st>>>(c.F, c.T, c.fg.U, nsplit, c.B, (const typename C2of<R>::t *)part,
-                                                       c.fg.moff, c.fg.mem, dc, dcs, c.dc_u, vis);
+    using C2 = typename C2of<R>::t;
+    auto *kern = pair_aligned<C2>(vis) ? k_group_finish<R, true> : k_group_finish<R, false>;
+    kern<<<2 * group_blocks(c), 128, 0, st>>>(c.F, c.T, c.fg.U, nsplit, c.B, (const C2 *)part, c.fg.moff, c.fg.mem, dc, dcs,
+                                              c.dc_u, vis);
     FM_CK_LAUNCH();
     return FM_OK;
 }
