@@ -212,7 +212,7 @@ struct RaBasis {
     const uint8_t *img = nullptr, *imgt = nullptr;   // tensor-core images of it and of its transpose (nullptr: none)
 };
 
-// Contraction in hour-angle Fourier modes (k_mm.cu), split-precision handles.
+// Contraction in hour-angle Fourier modes (k_mm.cu): handles of the three-product splits and of FP32.
 struct MmState {
     bool on = false;
     int L = 0, q = 1;                 // cells of the window, per RA pixel
@@ -359,7 +359,10 @@ extern long long g_launches;     // kernels launched by the library (relaxed cou
 // Visibilities are written into the caller's buffer, which need only be aligned for one real of them: both
 // parts at once where the buffer is aligned for the pair (pair_aligned, the same for a whole launch).
 template <typename C2, typename R>
-__host__ __device__ __forceinline__ bool pair_aligned(const R *p) { return (reinterpret_cast<uintptr_t>(p) & (sizeof(C2) - 1)) == 0; }
+__host__ __device__ __forceinline__ bool pair_aligned(const R *p)
+{
+    return (reinterpret_cast<uintptr_t>(p) & (sizeof(C2) - 1)) == 0;
+}
 template <typename C2, typename R>
 __device__ __forceinline__ void put_pair(R *p, const C2 &v, bool aligned)
 {

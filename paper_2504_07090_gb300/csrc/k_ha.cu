@@ -1474,10 +1474,6 @@ static fm_status ha_alloc(Ctx &c, T **p, size_t count)
     return FM_OK;
 }
 
-// Geometry test, fringe groups, work partition and the per-handle phasor table.  The
-// path is used for the tensor-core precisions when the LSTs are equally spaced by
-// k = 1 .. 32 RA pixels, n_ant <= 64, n_lst <= 64, n_ra <= 512 and the buffers take at most half of
-// the free device memory; otherwise c.ha.on stays false and the antenna form runs.
 // CTAs contributing to each (M-tile, channel) segment when the forward's Q work units are cut
 // into G contiguous ranges; sets s.grid and s.J (the most contributors of any segment)
 static void ha_partition(Ctx &c, int G, std::vector<int> &ncontrib)
@@ -1615,6 +1611,10 @@ static fm_status ha_of_modes(Ctx &c)
     return FM_OK;
 }
 
+// Chooses the form: hour-angle modes (k_mm.cu) for the three-product splits and FP32 where their table is made;
+// else, for the tensor-core precisions, this file's form where the LSTs are equally spaced by k / q RA pixels (q <= 4,
+// k <= 32), n_ra <= 512, the table's antennas are at most 63, the tiles fit and the buffers take at most half of the
+// free device memory; otherwise c.ha.on stays false and the antenna form (or the CUDA-core sums) runs.
 fm_status ha_setup(Ctx &c)
 {
     HaState &s = c.ha;

@@ -7,29 +7,30 @@
 // rate, where the cells in use number nh = 251 (37 antennas) or 503 (127 antennas).  With
 //   P_u(n, d) = sum_m c_u(m, d) e^{2 pi i m n / L},   Y(m, d) = sum_j y(j, d) e^{2 pi i m j / L},
 //   V_u(t) = sum_{m in band(u)} e^{2 pi i m tau_t / L} sum_d c_u(m, d) Y(m, d),
-// and the transpose gives the pixel gradient.  tau_t need not be a whole number where the cells sample the
-// fringes above their Nyquist rate: LSTs off the pixel grid take the same path.  Y comes from the mode transform of k_modes.cu with the RA
-// basis functions replaced by their Fourier sums, so the pixels are never formed.  Cells outside 0 .. nh - 1 meet no
-// pixel: there P_u is continued by its own formula, to where the beam is below MM_EDGE of its maximum, so that
-// the window has no step and the band ends; what a band leaves out is below MM_EPS of the response's l2 norm,
-// far under the FP32 rounding (6e-8) of the table that keeps it.  All of these are relative to the largest response
-// in the window, and a grid whose hour angles stay off the meridian has it in cells that meet no pixel: what is
-// left in those in use is then wrong by 3e-8 times the ratio of the two (a beam of 4.2 degrees FWHM, the nearest
-// cell in use 5 degrees off the meridian: 2e-6; 10 degrees off: 1e-2).  The form is taken up to a ratio of MM_PEAK = 4,
-// where that is 1e-7, below the FP32 sums' own 2.8e-7.
+// and the transpose gives the pixel gradient.  tau_t need not be a whole number where the cells sample the fringes
+// above their Nyquist rate: LSTs off the pixel grid take the same path.  Y comes from the mode transform of
+// k_modes.cu with the RA basis functions replaced by their Fourier sums, so the pixels are never formed.  Cells
+// outside 0 .. nh - 1 meet no pixel: there P_u is continued by its own formula, to where the beam is below MM_EDGE
+// of its maximum, so that the window has no step and the band ends; what a band leaves out is below MM_EPS of the
+// response's l2 norm, far under the FP32 rounding (6e-8) of the table that keeps it.  All of these are relative to
+// the largest response in the window, and a grid whose hour angles stay off the meridian has it in cells that meet
+// no pixel: what is left in those in use is then wrong by 3e-8 times the ratio of the two (a beam of 4.2 degrees
+// FWHM, the nearest cell in use 5 degrees off the meridian: 2e-6; 10 degrees off: 1e-2).  The form is taken up to a
+// ratio of MM_PEAK = 4, where that is 1e-7, below the FP32 sums' own 2.8e-7.
 //
 // The sky is real, so modes m and -m share Y: an element e = (|m|, u, sign) keeps c_u(m) or conj(c_u(-m)).
 // The table [e][declination] is sorted by |m|: the forward is one dot product over declinations per element, the
 // adjoint one sum over the elements of |m| per declination, both bound by one pass over the table in HBM.
 //
-// The tensor-core forms make the response of every cell anew from antenna phasors (bound by the producers and
-// the MMA issue of N = 64: k_ha.cu, k_tc.cu).  Measured with FP16 x3, their time first, the figures of chi^2 and
-// gradient: 37 antennas, 64 channels, 60 LSTs: forward 189 -> 38 us (k_mm_fwd 28 of them, 142 MB of table at 5.0
-// TB/s), adjoint 188 -> 43 us (k_mm_adj 28); LSTs off the grid (12 of them): 10.02 ms -> 82 us; 127 antennas, 128
-// channels, 120 LSTs: 7.26 -> 0.61 ms (k_mm_fwd 477 us, 3.1 GB at 6.5 TB/s) and 4.98 -> 0.65 ms.  The errors against 64 bits fall to
-// those of the mode transforms (V of 7 antennas 1.3e-6 -> 2.6e-7).
+// The tensor-core forms make the response of every cell anew from antenna phasors (bound by the producers and the
+// MMA issue of N = 64: k_ha.cu, k_tc.cu).  Measured with FP16 x3, their time first, the figures of chi^2 and
+// gradient: 37 antennas, 64 channels, 60 LSTs: forward 189 -> 36 us (k_mm_fwd 28 of them, 142 MB of table at 5.1
+// TB/s), adjoint 188 -> 40 us (k_mm_adj 26); LSTs off the grid (12 of them): 10.02 ms -> 82 us; 127 antennas, 128
+// channels, 120 LSTs: 7.26 -> 0.61 ms (k_mm_fwd 477 us, 3.1 GB at 6.5 TB/s) and 4.98 -> 0.65 ms.  The errors against
+// 64 bits fall to those of the mode transforms (V of 7 antennas 1.3e-6 -> 2.6e-7).
 // FP32 handles: 37 antennas, 64 channels, 60 LSTs, chi^2 and gradient 3.13 ms (each distinct fringe on the CUDA
-// cores, k_hs.cu) -> 0.27 ms; gradient against 64 bits 1.0e-7 in the mean of 14 geometries (1.2e-7 before), V 1.7e-7 (2.8e-7).
+// cores, k_hs.cu) -> 0.27 ms; gradient against 64 bits 1.0e-7 in the mean of 14 geometries (1.2e-7 before), V 1.7e-7
+// (2.8e-7).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -459,8 +460,9 @@ static_assert(MM_QT % 10 == 0, "k_mm_q reads LSTs in tens");
 
 // G[f][d][2 m] = Re, [2 m + 1] = -Im of X(m, d) = sum over the elements of |m| of c_e(d) w_e: two warps per
 // (channel, m, 32 pairs of declinations), one for each half of the elements (their numbers differ tenfold between
-// modes, and with one warp each the longest ran alone at the end: 27.7 -> 26.0 us for 37 antennas), eight 16-byte loads of the table in flight a
-// lane.  The channels run against the forward's order, so that what the forward read last is still in L2.
+// modes, and with one warp each the longest ran alone at the end: 27.7 -> 26.0 us for 37 antennas), eight 16-byte
+// loads of the table in flight a lane.  The channels run against the forward's order, so that what the forward read
+// last is still in L2.
 __global__ void __launch_bounds__(256) k_mm_adj(int F, int D, int nm, int ld, const int *__restrict__ moff,
                                                 const float4 *__restrict__ tab, const float2 *__restrict__ w,
                                                 float *__restrict__ G)

@@ -27,11 +27,12 @@ struct GemmArgs {
     int zero_b00;      // read B[0][0] of every batch as zero (drops the monopole mode a_00)
 };
 
-// FP32: 64 x 64 tiles, 128 threads of 8 x 4 sums (packed FMAs on column pairs: three 16-byte shared loads for 16
-// of them), the next 16 K values on their way in registers while the last are summed.  Each sum runs over K in
-// order, 16 terms at a time (their rounding errors grow with K / 16 + 16, not K).  The four products of the mode transforms of 127 antennas, 128 channels, 256 x 256 modes: 1.10 (256
-// threads of 4 x 4 sums, no prefetch) -> 0.65 ms, 40 TFLOP/s (0.58 ms with one running sum, whose errors were up to
-// twice as large: FP32 gradient of 37 antennas against 64 bits 1.3e-7, now 5e-8).
+// FP32: 64 x 64 tiles, 128 threads of 8 x 4 sums (packed FMAs on column pairs: three 16-byte shared loads for 16 of
+// them), the next 16 K values on their way in registers while the last are summed.  Each sum runs over K in order,
+// 16 terms at a time (their rounding errors grow with K / 16 + 16, not K).  The four products of the mode transforms
+// of 127 antennas, 128 channels, 256 x 256 modes: 1.10 (256 threads of 4 x 4 sums, no prefetch) -> 0.65 ms, 40
+// TFLOP/s (0.58 ms with one running sum, whose errors were up to twice as large: FP32 gradient of 37 antennas
+// against 64 bits 1.3e-7, now 5e-8).
 constexpr int GM_LD = 68;
 __global__ void __launch_bounds__(128) k_gemm(GemmArgs a, const float *__restrict__ A, const float *__restrict__ B,
                                               float *__restrict__ C)
