@@ -477,8 +477,8 @@ static fm_status run_hvp(Ctx &c, const R *theta, const R *v, R *hv, int full, cu
     }
     FM_TRY(run_adjoint_modes<R>(c, (R *)c.omega, c.K > 0 ? (R *)c.gx : hv, st, fused));
     if (c.K > 0) FM_TRY(launch_freq_contract<R>(c, (const R *)c.gx, hv, st));
-    // the products' gain block is summed in FP64 throughout (k_gain_reduce_ft's FP32 sums over a warp take 8 us less
-    // of a 214 us product of 37 antennas)
+    // the products' gain block is summed in FP64 throughout (k_gain_reduce_ft's FP32 sums over a warp take 1.3 us less
+    // of a 207 us product of 37 antennas)
     FM_TRY(launch_gain_reduce<R>(c, (R *)c.zpart, hv + c.n_sky, st));
     return launch_prior_hvp<R>(c, v, hv, st);
 }

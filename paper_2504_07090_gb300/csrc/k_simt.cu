@@ -473,18 +473,6 @@ fm_status launch_vis(Ctx &c, const R *x, R *vis, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------- chi^2 epilogue
-template <typename R>
-__device__ void block_sum_double(double v, double *out, double *sred)
-{
-    sred[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sred[threadIdx.x] += sred[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = sred[0];
-}
-
 // ---- pieces of the per-(channel, LST) epilogues k_chi2_ft and k_hvp_ft
 
 __device__ __forceinline__ float hv_scale(const HaVSrc &hv, int f)
@@ -1213,33 +1201,48 @@ fm_status launch_adjoint(Ctx &c, const R *omega, R *xbar, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------- reductions
-// grad_gamma[a][k][re, im] = sum_{f,t} X_k(nu_f) Z[f][t][a]   (FP64, fixed order)
+// grad_gamma[a][k][c] = sum_f X_k(nu_f) sum_t Z[f][t][a][c]   (FP64, fixed order).  CTA (a, c): 16 lanes a channel sum
+// its LSTs, lane k multiplies by X_k, warp k adds the channels.  Bound: the FP64 pipe (2 lanes per SM and clock),
+// where summing over the LSTs first leaves a conversion and an addition a term, and the products a channel; and the
+// latency of the loads, four in flight a thread.  Product of 37 antennas, 64 channels, 60 LSTs: 214.3 (256 threads an
+// antenna and coefficient, a product a term) -> 207.2 us.
+constexpr int GN_MAX = 16, GN_FC = 64;     // most gain coefficients (fm_create's limit); channels at a time
 template <typename R>
-__global__ void __launch_bounds__(256) k_gain_reduce(DevGeom g, const R *__restrict__ zpart, R *__restrict__ out)
+__global__ void __launch_bounds__(GN_MAX * GN_FC) k_gain_reduce(DevGeom g, const R *__restrict__ zpart, R *__restrict__ out)
 {
-    __shared__ double sred[256];
-    const int a = blockIdx.x, k = blockIdx.y;
-    double sr = 0.0, si = 0.0;
-    for (int ft = threadIdx.x; ft < g.F * g.T; ft += blockDim.x) {
-        int f = ft / g.T;
-        double X = (double)Tab<R>::gleg(g)[(size_t)f * g.NG + k];
-        sr += X * (double)zpart[((size_t)ft * g.A + a) * 2];
-        si += X * (double)zpart[((size_t)ft * g.A + a) * 2 + 1];
+    __shared__ double red[GN_MAX][GN_FC + 1];
+    const int a = blockIdx.x, c = blockIdx.y, tid = threadIdx.x, q = tid % GN_MAX, fl = tid / GN_MAX;
+    double acc = 0.0;                      // warp k < NG: the channels fl = lane, lane + 32 of coefficient k
+    for (int f0 = 0; f0 < g.F; f0 += GN_FC) {
+        const int f = f0 + fl;
+        double s = 0.0;
+        if (f < g.F) {
+            const R *z = zpart + ((size_t)f * g.T * g.A + a) * 2 + c;
+            for (int t0 = q; t0 < g.T; t0 += 4 * GN_MAX) {
+                R v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = t0 + u * GN_MAX < g.T ? z[(size_t)(t0 + u * GN_MAX) * g.A * 2] : R(0);
+                s += ((double)v[0] + (double)v[1]) + ((double)v[2] + (double)v[3]);
+            }
+        }
+#pragma unroll
+        for (int o = GN_MAX / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (f0) __syncthreads();           // the last channels are read
+        if (q < g.NG) red[q][fl] = f < g.F ? (double)Tab<R>::gleg(g)[(size_t)f * g.NG + q] * s : 0.0;
+        __syncthreads();
+        if (tid / 32 < g.NG) acc += red[tid / 32][tid % 32] + red[tid / 32][tid % 32 + 32];
     }
-    double tot;
-    block_sum_double<R>(sr, &tot, sred);
-    __syncthreads();
-    if (threadIdx.x == 0) out[(a * g.NG + k) * 2] = (R)tot;
-    __syncthreads();
-    block_sum_double<R>(si, &tot, sred);
-    if (threadIdx.x == 0) out[(a * g.NG + k) * 2 + 1] = (R)tot;
+    if (tid / 32 < g.NG) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (tid % 32 == 0) out[(a * g.NG + tid / 32) * 2 + c] = (R)acc;
+    }
 }
 
 template <typename R>
 fm_status launch_gain_reduce(Ctx &c, const R *zpart, R *grad_gain, cudaStream_t st)
 {
-    dim3 grid(c.A, c.NG);
-    k_gain_reduce<R><<<grid, 256, 0, st>>>(c.g, zpart, grad_gain);
+    k_gain_reduce<R><<<dim3(c.A, 2), GN_MAX * GN_FC, 0, st>>>(c.g, zpart, grad_gain);
     FM_CK_LAUNCH();
     return FM_OK;
 }
