@@ -307,7 +307,9 @@ FM_API fm_status fm_sky_pixels_noalloc(int n_freq, int n_ra, int n_dec, int n_mo
  * With a Gaussian beam the x3 precisions (forms 1 and 2) and FP32 compute in hour-angle Fourier modes, from one table per
  * channel of each distinct fringe's band of modes, where the table fits and the grid reaches the beam's maximum
  * (fm_mode_table_bytes > 0 tells); the form written here, and what the launch grids below may be set to, are those
- * of the geometry.  The x1 precisions do not, and with that beam are slower and less exact than x3.
+ * of the geometry.  Their responses are exact to 3e-8 of the largest in use, not of each cell's own: a sky that is
+ * bright only where the beam is 1e-3 keeps five figures.  The x1 precisions do not compute so, and with that beam
+ * are slower and less exact than x3.
  * The form is fixed at fm_create; the environment variable FM_HA=0 read there
  * disables form 2 and FM_HA_GROUPS=0 makes it compute every baseline separately. */
 FM_API fm_status fm_contraction_info(fm_handle h, int32_t *out);
