@@ -308,7 +308,7 @@ FM_API fm_status fm_sky_pixels_noalloc(int n_freq, int n_ra, int n_dec, int n_mo
  * channel of each distinct fringe's band of modes, where the table fits and the grid reaches the beam's maximum
  * (fm_mode_table_bytes > 0 tells); the form written here, and what the launch grids below may be set to, are those
  * of the geometry.  Their responses are exact to 3e-8 of the largest in use, not of each cell's own: a sky that is
- * bright only where the beam is 1e-3 keeps five figures.  The x1 precisions do not compute so, and with that beam
+ * bright only where the beam is 1e-3 keeps four figures.  The x1 precisions do not compute so, and with that beam
  * are slower and less exact than x3.
  * The form is fixed at fm_create; the environment variable FM_HA=0 read there
  * disables form 2 and FM_HA_GROUPS=0 makes it compute every baseline separately. */
